@@ -148,13 +148,12 @@ accel_status accel_set_device_status(int32_t* d_status);
 accel_status accel_sync_status(int32_t* d_status, int32_t clear, void* stream);
 
 /*
- * accel_set_watchdog_ns -- failure detection for the persistent single-CTA BF16 forward
- * (hmm_forward, ACCEL_HMM_BF16_SCALED, in the tuned configurations that run one CTA per
- * tile): a launch that has run longer than budget_ns stops at its next step boundary, after
- * the step's tensor-core work has completed, and reports ACCEL_ERR_TIMEOUT in its device
+ * accel_set_watchdog_ns -- failure detection for the persistent BF16 forward (hmm_forward,
+ * ACCEL_HMM_BF16_SCALED): a launch that has run longer than budget_ns stops at a step boundary,
+ * after the tensor-core work in flight has completed, and reports ACCEL_ERR_TIMEOUT in its device
  * status word; its log-likelihoods are then incomplete.  0 (the default) means no limit.
  * Process-wide; read by each launch when it is issued (a captured graph keeps the value
- * it was captured with).  The cluster-pair configurations keep only their bounded waits.
+ * it was captured with).
  */
 void accel_set_watchdog_ns(uint64_t budget_ns);
 uint64_t accel_get_watchdog_ns(void);
@@ -465,12 +464,11 @@ accel_status hmm_mstep(const accel_hmm_model* m, const float* d_grad_log_A, cons
                        float* d_new_log_pi, void* stream);
 
 /*
- * hmm_autotune -- choose the launch configuration of the BF16 tensor-core forward (column
- * parts per row: 8 or 16 warps; sequence rows per tile: 128, 64 or 32; a tile on one CTA or
- * on a cluster of two or four CTAs that split the state columns) by timing each
- * candidate with CUDA events on these inputs, then the number of persistent work units of
- * the fastest (the fewest of all that fit, 3/4, 1/2, 3/8 and 1/4 of them within 1 % of its
- * time, so that a latency-bound forward leaves SMs free for other streams), and remember the
+ * hmm_autotune -- choose the launch configuration of the BF16 tensor-core forward (sequences
+ * per tile: 16, 32, 64 or 128) by timing each candidate with CUDA events on these inputs, then
+ * the number of persistent CTAs of the fastest (the fewest of all that fit, 3/4, 1/2, 3/8 and 1/4
+ * of them within 1 % of its time, so that a latency-bound forward leaves SMs free for other
+ * streams), and remember the
  * result for (device, K, M, floor(log2 S)); hmm_forward then launches with it.  `cache_path` (may be NULL) names a
  * file of JSON lines: an entry for the same key is reused without timing, a new result is
  * appended.  Arguments as hmm_forward (d_loglik receives the last timed run's result).
@@ -481,11 +479,11 @@ accel_status hmm_autotune(const accel_hmm_model* m, int32_t precision, const int
                           const int64_t* d_offsets, int64_t S, int64_t total_T, double* d_loglik,
                           void* d_ws, size_t ws_bytes, const char* cache_path, float* h_best_ms,
                           void* stream);
-/* The configuration hmm_forward(ACCEL_HMM_BF16_SCALED) uses for these sizes: column parts
- * per row, rows per tile, (h_pair, may be NULL) how a tile is split over a thread-block
- * cluster: 0 one CTA, 1 two CTAs, 2 four CTAs (each holding K/2 or K/4 state columns), and
- * (h_units, may be NULL) the persistent work units launched (CTAs or clusters; 0: all that
- * fit). */
+/* The configuration hmm_forward(ACCEL_HMM_BF16_SCALED) uses for these sizes: a CTA takes tiles of
+ * 2 rows / split sequences (without a tuned configuration, past tiles of 16, the next smaller tile
+ * if the lengths favour it); (h_pair, may be NULL) is kept from files of earlier versions, which
+ * split a tile over clusters, and changes nothing; (h_units, may be NULL) the persistent CTAs
+ * launched (0: all that fit). */
 accel_status hmm_tuned_config(int32_t K, int32_t M, int64_t S, int32_t* h_split, int32_t* h_rows,
                               int32_t* h_pair, int32_t* h_units);
 

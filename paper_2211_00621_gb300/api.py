@@ -445,9 +445,9 @@ def hmm_mstep(log_A, log_B, log_pi, grad_log_A, grad_log_B, grad_log_pi, want_gr
 def hmm_autotune(log_A, log_B, log_pi, obs, offsets, precision=L.HMM_BF16_SCALED, cache_path=None, ws=None):
     """Times the BF16 forward's launch configurations on these inputs and keeps the fastest
     for later hmm_forward calls (and in `cache_path`, JSON lines, if given).  Returns
-    (best ms or 0.0 if cached, (split, rows, pair, units)); pair = 1 (2) when a tile of
-    sequences runs on a cluster of two (four) CTAs that split the state columns; units = the
-    persistent CTAs or clusters launched (0: all that fit)."""
+    (best ms or 0.0 if cached, (split, rows, pair, units)): a CTA takes tiles of 2 rows / split
+    sequences; pair is 0 (other values come from files of earlier versions and change nothing);
+    units = the persistent CTAs launched (0: all that fit)."""
     lib = L.load()
     m = _model(log_A, log_B, log_pi)
     S = offsets.numel() - 1

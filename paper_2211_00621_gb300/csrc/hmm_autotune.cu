@@ -1,16 +1,16 @@
-// Autotuner for the BF16 tensor-core HMM forward: picks the launch configuration (column
-// parts per row: 8 or 16 warps; sequence rows per tile: 128, 64 or 32; one CTA per tile or a
-// cluster of two or four CTAs splitting the state columns) by timing every candidate on the caller's inputs
-// with CUDA events, then the number of persistent work units of the winner: the fewest
-// (of all that fit, 3/4, 1/2, 3/8 and 1/4 of them) within 1 % of its time.  The forward is
-// bound by the step latency of its longest sequences, so on skewed length mixes a fraction
-// of the GPU finishes it as fast as all of it, and the rest of the SMs stay free for work
-// on other streams.  The winner is remembered per (device, K, M, floor(log2 S)) -- in this
-// process, and optionally in a cache file of JSON lines so later processes skip the timing:
+// Autotuner for the BF16 tensor-core HMM forward: picks the launch configuration (sequences per
+// tile: 16, 32, 64 or 128) by timing every candidate on the caller's inputs with CUDA events, then
+// the number of persistent CTAs of the winner: the fewest (of all that fit, 3/4, 1/2, 3/8 and 1/4
+// of them) within 1 % of its time.  The forward is bound by the step latency of its longest
+// sequences, so on skewed length mixes a fraction of the GPU finishes it as fast as all of it, and
+// the rest of the SMs stay free for work on other streams.  The winner is remembered per (device,
+// K, M, floor(log2 S)) -- in this process, and optionally in a cache file of JSON lines so later
+// processes skip the timing:
 //   {"kernel": "hmm_forward_bf16", "device": "<name>", "K": 256, "M": 64, "S_log2": 12,
-//    "split": 4, "rows": 128, "pair": 0, "units": 76, "ms": 17.21}
-// (lines without "units" mean all units).  hmm_forward consults the table; without an entry
-// it uses 16 warps, 128 rows, one CTA, all units.
+//    "split": 4, "rows": 32, "pair": 0, "units": 76, "ms": 2.46}
+// (lines without "units" mean all units; a tile is 2 rows / split sequences; "pair" is kept as it
+// was saved and changes nothing).  hmm_forward consults the table; without an entry it chooses
+// the tile from the sizes and lengths of the call.
 #include "hmm_internal.cuh"
 
 #include <cmath>
@@ -31,12 +31,19 @@ using Key = std::tuple<std::string, int, int, int>;
 std::mutex g_mu;
 std::map<Key, TcConfig> g_table;
 
+// the current device's name, looked up once per device: the query takes longer than the launches
+// of a small forward
 std::string device_name() {
+    static std::mutex mu;
+    static std::map<int, std::string> names;
     int dev = 0;
     cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = names.find(dev);
+    if (it != names.end()) return it->second;
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return "unknown";
-    return prop.name;
+    return names[dev] = prop.name;
 }
 
 int s_log2(int64_t S) {
@@ -44,8 +51,6 @@ int s_log2(int64_t S) {
     while ((int64_t(1) << (b + 1)) <= S) ++b;
     return b;
 }
-
-TcConfig default_config(int K) { return TcConfig{(K / 4) % 32 == 0 ? 4 : 2, 128, 0, 0}; }
 
 bool load_from_cache(const char* path, const Key& key, TcConfig* out) {
     if (!path || !path[0]) return false;
@@ -93,11 +98,13 @@ void append_to_cache(const char* path, const Key& key, TcConfig c, float ms) {
 
 }  // namespace
 
-TcConfig tuned_config(int K, int M, int64_t S) {
+bool tuned_entry(int K, int M, int64_t S, TcConfig* out) {
     Key key(device_name(), K, M, s_log2(S));
     std::lock_guard<std::mutex> lock(g_mu);
     auto it = g_table.find(key);
-    return it != g_table.end() ? it->second : default_config(K);
+    if (it == g_table.end()) return false;
+    *out = it->second;
+    return true;
 }
 
 accel_status check_model(const accel_hmm_model* m, const char* who);
@@ -132,26 +139,22 @@ accel_status hmm_autotune(const accel_hmm_model* m, int32_t precision, const int
     cudaStream_t st = as_stream(stream);
     char* ws = (char*)d_ws;
     std::vector<TcConfig> cands;
-    for (int pair : {0, 1, 2})
-        for (int split : {4, 2})
-            for (int rows : {128, 64, 32}) {
-                if (split == 4 && (m->K / 4) % 32 != 0) continue;
-                if (rows < 128 && (S + rows - 1) / rows <= (S + 127) / 128) continue;   // no more tiles than 128 rows
-                if (pair && !tc_cl_supported(m->K, m->M, rows, split, pair == 1 ? 2 : 4)) continue;
-                cands.push_back(TcConfig{split, rows, pair, 0});
-            }
+    for (int n : {16, 32, 64, 128}) {
+        if (n > 16 && S <= n / 2) continue;              // no more tiles than the smaller size
+        cands.push_back(tile_config(n));
+    }
     cudaEvent_t e0, e1;
     ACCEL_CUDA_TRY(cudaEventCreate(&e0));
     ACCEL_CUDA_TRY(cudaEventCreate(&e1));
     // time one configuration: a warm-up run, then the mean of two (in *ms)
     auto time_cfg = [&](const TcConfig& c, float* ms) -> accel_status {
         ACCEL_CUDA_TRY(cudaMemsetAsync(ws + kStatusOff, 0, 4, st));
-        accel_status q = tc_forward_cfg(m, d_obs, d_offsets, S, d_loglik, ws, (int32_t*)(ws + kStatusOff), c, st);
+        accel_status q = tc_forward_cfg(m, d_obs, d_offsets, S, d_loglik, ws, (int32_t*)(ws + kStatusOff), &c, st);
         if (q != ACCEL_OK) return q;
         float total = 0.f;
         for (int rep = 0; rep < 2; ++rep) {
             ACCEL_CUDA_TRY(cudaEventRecord(e0, st));
-            q = tc_forward_cfg(m, d_obs, d_offsets, S, d_loglik, ws, (int32_t*)(ws + kStatusOff), c, st);
+            q = tc_forward_cfg(m, d_obs, d_offsets, S, d_loglik, ws, (int32_t*)(ws + kStatusOff), &c, st);
             if (q != ACCEL_OK) return q;
             ACCEL_CUDA_TRY(cudaEventRecord(e1, st));
             ACCEL_CUDA_TRY(cudaEventSynchronize(e1));
@@ -167,7 +170,7 @@ accel_status hmm_autotune(const accel_hmm_model* m, int32_t precision, const int
         *ms = total / 2;
         return ACCEL_OK;
     };
-    TcConfig best = default_config(m->K);
+    TcConfig best = default_config(S);
     float best_ms = INFINITY;
     for (const TcConfig& c : cands) {
         float ms = 0.f;
@@ -177,9 +180,9 @@ accel_status hmm_autotune(const accel_hmm_model* m, int32_t precision, const int
     }
     if (r == ACCEL_OK && best_ms < INFINITY) {
         // fewer persistent work units: the smallest count within 1 % of the best time
-        const int nc = best.pair == 2 ? 4 : (best.pair == 1 ? 2 : 1);
-        const int64_t tiles = (S + best.rows - 1) / best.rows;
-        const int64_t cap64 = tiles < num_sms() / nc ? tiles : num_sms() / nc;
+        const int n = 2 * best.rows / best.split;
+        const int64_t tiles = (S + n - 1) / n;
+        const int64_t cap64 = tiles < num_sms() ? tiles : num_sms();
         const int cap = (int)(cap64 < 1 ? 1 : cap64);
         const float limit = best_ms * 1.01f;
         for (int f8 : {6, 4, 3, 2}) {            // 3/4, 1/2, 3/8, 1/4 of the units
@@ -213,7 +216,8 @@ accel_status hmm_autotune(const accel_hmm_model* m, int32_t precision, const int
 accel_status hmm_tuned_config(int32_t K, int32_t M, int64_t S, int32_t* h_split, int32_t* h_rows, int32_t* h_pair,
                               int32_t* h_units) {
     ACCEL_REQUIRE(h_split && h_rows, ACCEL_ERR_INVALID_ARG, "hmm_tuned_config: null pointer");
-    TcConfig c = tuned_config(K, M, S);
+    TcConfig c;
+    if (!tuned_entry(K, M, S, &c)) c = default_config(S);
     *h_split = c.split;
     *h_rows = c.rows;
     if (h_pair) *h_pair = c.pair;

@@ -23,22 +23,23 @@ accel_status plain_forward(const accel_hmm_model* m, const int32_t* obs, const i
                            double* loglik, char* ws, int32_t* d_status, cudaStream_t st);
 
 // Launch configuration of the BF16 tensor-core forward, chosen by the autotuner
-// (hmm_autotune.cu): column parts per row (2: 8 warps, 4: 16 warps), sequence rows used per
-// tile (<= 128; fewer rows spread the sequences over more SMs), and whether a tile runs on
-// one CTA (pair = 0) or on a cluster that splits the state columns: two CTAs (pair = 1) or
-// four (pair = 2).
+// (hmm_autotune.cu): one CTA takes tiles of 2 rows / split sequences (split 2 or 4, rows 32, 64 or
+// 128: tiles of 16 to 128).  `pair` is kept for configurations saved by earlier versions, which
+// split a tile over a cluster of two or four CTAs; it no longer changes the launch.
 struct TcConfig {
     int split;
     int rows;
     int pair;
-    int units;      // persistent work units launched (CTAs, or clusters when pair > 0); 0: all that fit
+    int units;      // persistent CTAs launched; 0: all that fit
 };
-bool tc_cl_supported(int K, int M, int rows, int split, int nc);
-TcConfig tuned_config(int K, int M, int64_t S);
+TcConfig tile_config(int n);             // the configuration of a tile of n sequences
+TcConfig default_config(int64_t S);      // ... used without a tuned one
+bool tuned_entry(int K, int M, int64_t S, TcConfig* out);    // the tuned configuration, if there is one
 
-// BF16 tensor-core scaled forward (k_hmm_tc.cu).
+// BF16 tensor-core scaled forward (k_hmm_tc.cu); cfg null: the tile is chosen from S and, past
+// tiles of 16, from the lengths on the device.
 accel_status tc_forward_cfg(const accel_hmm_model* m, const int32_t* obs, const int64_t* off, int64_t S,
-                            double* loglik, char* ws, int32_t* d_status, TcConfig cfg, cudaStream_t st);
+                            double* loglik, char* ws, int32_t* d_status, const TcConfig* cfg, cudaStream_t st);
 size_t tc_ws_bytes(int K, int M, int64_t S);
 accel_status tc_forward(const accel_hmm_model* m, const int32_t* obs, const int64_t* off, int64_t S,
                         double* loglik, char* ws, int32_t* d_status, cudaStream_t st);

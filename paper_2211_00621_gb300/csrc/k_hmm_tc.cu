@@ -1,880 +1,727 @@
-// Batched scaled HMM forward on the tensor cores (K8).
+// Batched scaled HMM forward on the tensor cores, states on the lanes (K8).
 //
 // The forward recursion (map over states j of a reduce over states i inside a sequential
-// loop over t; Appendix A patterns) for a tile of 128 sequences is one dense contraction
-// per step:  D = X_{t-1} A  with X the [128 x K] tile of scaled forward vectors.  The HMM
-// itself is not in the paper; this is the textbook scaled forward algorithm, with the
-// rescaling done by exact powers of two:
-//   alpha~_t = (X_{t-1} A) o b(o_t),   s_t = sum_j alpha~_t(j),   X_t = alpha~_t 2^-k_t
+// loop over t; Appendix A patterns) for a tile of N sequences is one dense contraction per
+// step.  The HMM itself is not in the paper; this is the textbook scaled forward algorithm,
+// with the rescaling done by exact powers of two:
+//   alpha~_t = (A^T X_{t-1}) o b(o_t),   s_t = sum_j alpha~_t(j),   X_t = alpha~_t 2^-k_t
 //   logL     = ln2 * sum_{t<T-1} k_t + ln s_{T-1}
-// Any integers k_t give the same logL exactly (alpha_t = alpha~_t 2^{k_0+...+k_{t-1}}); they
-// only keep X in range.  k_t is predicted one step ahead -- from log2 sum(X_{t-1}) and the
-// previous growth ratio s_{t-1} / sum(X_{t-2}) -- so the epilogue makes a single pass over
-// the accumulator: the row sum is needed only afterwards.  sum(X_t) then stays within a
-// factor of the step-to-step change of the emission scale, with no drift.
+// Any integers k_t give the same logL exactly; they only keep X in range:
+//   k_t = x_{t-2} - k_{t-1} - kTarget,   x_t = log2 of the largest entry of X_t,
+// which makes x_t = kTarget + the growth of the last two steps.  The step before last is the
+// newest whose maxima are not on the path from one step to the next.  Growth is at most 1 for
+// probabilities, so the target sits high: two steps may shrink the vector by 2^-90 each.
 //
-// Per CTA (one per SM, persistent, 128 x NSPLIT threads; NSPLIT = 2 or 4 column parts per
-// row, chosen by the autotuner):
-//  * shared memory holds, for the whole launch, A^T (BF16, the MMA's B operand: N = K rows
-//    of K, no-swizzle K-major canonical layout) and the emission table b(j, k) (BF16, rows
-//    rotated by the symbol so different symbols hit different banks); the X tile
-//    (BF16, 128 x K, canonical layout) is the MMA's A operand;
-//  * D (FP32, 128 lanes x K columns) accumulates in tensor memory; one thread issues the
-//    K/16 tcgen05.mma (M=128, N=K, K=16) of a step and commits them to an mbarrier;
-//  * 4 x NSPLIT warps read D back (tcgen05.ld): warps w, w+4, ... share the lane quarter of
-//    rows 32(w%4)..+31 and split the columns in NSPLIT parts; each thread multiplies its part
-//    of the row by the emission, accumulates its partial row sum, scales by the predicted
-//    2^-k, rounds to BF16 and writes its part of the next X row;
-//  * while the next step's MMAs run, one thread per row combines the partial sums and
-//    advances the row's bookkeeping; when its sequence ends it writes logL and takes the
-//    next sequence from a global queue ordered by decreasing length, whose first vector
-//    alpha~_0 = pi o b(o_0) the row's threads write in the next epilogue (so uneven lengths
-//    are packed into one launch).  The row's next symbol is loaded one step ahead, so no
-//    global load sits on the step's critical path.
-// All mbarrier waits are bounded (2 s); on expiry the kernel reports ACCEL_ERR_TIMEOUT.  The
-// single-CTA kernel also has a watchdog on its whole run time (accel_set_watchdog_ns), checked
-// at step boundaries, which stops it cleanly with ACCEL_ERR_TIMEOUT.
+// A step's time is its latency (the sequences are long and a step depends on the last), so
+// the tile is laid out for a short step, not for a full tensor core:
+//  * the MMA computes D^T [128 states x N sequences] = A^T [128 x K] X [K x N], one block per
+//    128 states: N is as small as the batch allows (16 to 128), and a step costs N columns
+//    instead of the 128 rows a sequence-major tile pays for;
+//  * A^T is the MMA's A operand and stays in tensor memory for the whole launch (K / 2 columns
+//    per block of 128 states): an N = 32 product reads 1 KB of X per 16 states from shared
+//    memory instead of 5 KB;
+//  * X (BF16) is the B operand in the MN-major no-swizzle canonical layout, so the thread that
+//    holds state j writes 8 sequences with one 16-byte store;
+//  * each thread of the epilogue holds one state and CPT sequences: D comes from tensor
+//    memory in one load, b(j, o) from a shared table of FP32 values (already rounded to BF16);
+//  * X is double-buffered by step parity, so a block's epilogue writes X_t while the other
+//    block's products still read X_{t-1};
+//  * one warp per block of states does nothing but issue its MMAs;
+//  * one warp keeps the books (lane s: sequence s): while the products of step i run it turns
+//    the column maxima of X_{i-1} into the exponents of step i + 1 and publishes them with that
+//    step's symbols.  For tiles of up to 32 sequences further warps read X_{i-1} back for the
+//    maxima, which keeps their shuffles out of the epilogue warps' step; larger tiles form them
+//    in the epilogue.  Row sums are needed at a sequence's last step alone, and only then do the
+//    epilogue warps form them.
+// Row sums: 32 states per warp, added in a fixed binary tree by a reduce-scatter over the
+// lanes, then over the warps in order of states.
+//
+// Measured (GB300; K = 256, M = 64, 4,096 sequences of log-uniform 50 to 5,000 steps): 2.42 ms,
+// 0.49 us a step of the longest sequence with tiles of 16.  One CTA per 128 sequences with the
+// sequences on the lanes took 12.7 ms, and clusters of two CTAs splitting the states of 32
+// sequences 8.8 ms: 2.5 and 1.75 us a step.  What is left of a step is a chain of latencies (the
+// products 0.2 us, tensor memory to X 0.15 us, two mbarrier hand-offs), not a rate.
+//
+// Every wait is bounded (2 s); on expiry the kernel reports ACCEL_ERR_TIMEOUT.  A watchdog on
+// the run time (accel_set_watchdog_ns) is checked at step boundaries, with no product in
+// flight.
 #include "common.cuh"
 #include "hmm_internal.cuh"
 #include "tc_ptx.cuh"
 
-#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
-#include <map>
-#include <mutex>
-#include <utility>
+#include <type_traits>
 
 namespace accel {
 namespace hmm {
 
-constexpr int kRows = 128;
+namespace {
+
+constexpr int kTarget = 60, kMaxScale = 96;     // log2 of X's target size; largest |k|
 constexpr uint64_t kWaitNs = 2000000000ull;   // bounded mbarrier wait: 2 s of wall clock
+// epilogue: column parts per lane quarter for tiles of N sequences
+__host__ __device__ constexpr int col_parts(int N) { return N <= 16 ? 1 : 2; }
+// warps that take the column maxima: 16 columns of a block of 128 states each (0: the epilogue's)
+__host__ __device__ constexpr int max_warps(int K, int N) { return N <= 32 ? (K + 127) / 128 * (N / 16) : 0; }
 
-struct TcLayout {
-    // workspace (after the status block)
-    size_t at_off, e_off, order_off, order_scratch_off, total;
-    // dynamic shared memory
-    uint32_t s_at, s_x, s_e, s_rowinfo, s_psum, s_bar, s_slot, smem_bytes;
+// What a step is to the tile: the columns that start and that end a sequence, and whether the
+// tile is done (the step is not run).
+struct Ctl {
+    uint32_t fresh[4], end[4], done, pad[3];
 };
 
-// Per-row values the column-part threads need (written by the row's owner thread).
-struct RowInfo {
-    int16_t ob;     // symbol o_t of the step being computed; -1: no sequence; -(o_0 + 2): the
-                    // row starts a sequence whose first symbol is o_0
-    int16_t k;      // exponent k_t: this step's X_t is scaled by 2^-k_t
+struct TileLayout {
+    uint32_t x, x_bytes, e, scale, sym, ctl, mx, psum, bar, slot, bytes;
 };
 
-static TcLayout tc_layout(int K, int M, int64_t S) {
-    TcLayout L;
-    L.at_off = align_up(kStatusBytes, 1024);
-    L.e_off = align_up(L.at_off + (size_t)K * K * 2, 1024);
-    L.order_off = align_up(L.e_off + (size_t)M * K * 2, 256);
-    L.order_scratch_off = align_up(L.order_off + (size_t)S * 4, 256);
-    L.total = L.order_off + order_ws_bytes(S);
+__host__ __device__ inline TileLayout tile_layout(int K, int M, int N, int esize) {
+    TileLayout L;
     uint32_t o = 0;
-    L.s_at = o; o += (uint32_t)K * K * 2;
-    L.s_x = o;  o += (uint32_t)kRows * K * 2;
-    L.s_e = o;  o += (uint32_t)M * K * 2;
+    L.x_bytes = (uint32_t)N * (uint32_t)K * 2;
+    L.x = o;      o += 2 * L.x_bytes;                               // [step parity]
+    L.e = o;      o += (uint32_t)M * (uint32_t)K * (uint32_t)esize;
     o = (o + 15) & ~15u;
-    L.s_rowinfo = o; o += kRows * (uint32_t)sizeof(RowInfo);
-    L.s_psum = o; o += 4 * kRows * 4;
-    L.s_bar = o; o += 8;
-    L.s_slot = o; o += 8;
-    L.smem_bytes = o;
+    L.scale = o;  o += 2 * (uint32_t)N * 4;                         // [step parity][N]: 2^-k
+    L.sym = o;    o += 4 * (uint32_t)N * 4;                         // [step mod 4][N]: o_t K
+    L.ctl = o;    o += 4 * 48;                                      // [step mod 4]: Ctl
+    L.mx = o;     o += 2 * (uint32_t)(K / 32) * (uint32_t)N * 2;    // [step parity][K / 32][N]: BF16 maxima
+    L.psum = o;   o += 2 * (uint32_t)(K / 32) * (uint32_t)N * 4;    // [step parity][K / 32][N]: row sums
+    o = (o + 7) & ~7u;
+    L.bar = o;    o += 10 * 8;
+    L.slot = o;   o += 16;
+    L.bytes = o;
     return L;
 }
 
-bool tc_supported(int K, int M) {
-    if (K < 64 || K > 256 || K % 64 != 0 || M < 1 || M > 32767) return false;
-    return (int)tc_layout(K, M, 0).smem_bytes <= max_smem_optin();
-}
-
-size_t tc_ws_bytes(int K, int M, int64_t S) { return tc_layout(K, M, S).total; }
-
-// Byte offset of element (row r, col k) in the no-swizzle K-major canonical layout with
-// LBO = 128 (core matrices along K contiguous) and SBO = 16 * Kdim.
-__host__ __device__ __forceinline__ uint32_t canon_off(int r, int k, int Kdim) {
-    return (uint32_t)((r >> 3) * (16 * Kdim) + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2);
-}
-
-// Emission table row o (symbol), state j: row of K BF16 values whose 16-byte chunks are
-// rotated by o, so threads reading the same chunk of different rows hit different banks.
-__host__ __device__ __forceinline__ uint32_t etab_off(int o, int j, int K) {
-    int nch = K >> 3;
-    int q = ((j >> 3) + o) % nch;
-    return (uint32_t)(o * K * 2 + q * 16 + (j & 7) * 2);
-}
-
-// A^T in canonical layout (B operand: row n = j, column k = i) and the emission table.
-__global__ void k_tc_prep(const float* __restrict__ logA, const float* __restrict__ logB, int K, int M,
-                          char* __restrict__ at, char* __restrict__ etab) {
-    int64_t nA = (int64_t)K * K, nB = (int64_t)K * M;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < nA + nB;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        if (idx < nA) {
-            int i = (int)(idx / K), j = (int)(idx % K);
-            *reinterpret_cast<__nv_bfloat16*>(at + canon_off(j, i, K)) = __float2bfloat16_rn(__expf(logA[idx]));
-        } else {
-            int64_t q = idx - nA;
-            int j = (int)(q / M), k = (int)(q % M);
-            *reinterpret_cast<__nv_bfloat16*>(etab + etab_off(k, j, K)) = __float2bfloat16_rn(__expf(logB[q]));
-        }
-    }
-}
-
-__device__ __forceinline__ float bf_lo(uint32_t x) { return __uint_as_float(x << 16); }
-__device__ __forceinline__ float bf_hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&h);
 }
 
-// NSPLIT = column parts per row: 2 (8 warps) or 4 (16 warps; needs K/4 a multiple of 32).
-// MT = rows of the MMA tile: 128, or 64 when a CTA runs at most 64 sequence rows (half the
-// tensor-core work per step).  With M = 64, row r of D sits in TMEM lane 32 (r / 16) + r % 16,
-// so in each warp's lane quarter only lanes 0-15 carry a row.
-template <int NSPLIT, int MT>
-__global__ void __launch_bounds__(128 * NSPLIT, 1)
-k_hmm_tc(int K, int M, const char* __restrict__ g_at, const char* __restrict__ g_etab,
-         const float* __restrict__ log_pi, const int32_t* __restrict__ obs, const int64_t* __restrict__ off,
-         int64_t S, const int32_t* __restrict__ order, unsigned long long* __restrict__ next, int rows_active,
-         double* __restrict__ loglik, int32_t* __restrict__ status, uint64_t watchdog_ns, TcLayout L) {
-    extern __shared__ __align__(1024) char smem[];
-    char* sAT = smem + L.s_at;
-    char* sX = smem + L.s_x;
-    char* sE = smem + L.s_e;
-    RowInfo* rinfo = reinterpret_cast<RowInfo*>(smem + L.s_rowinfo);
-    float* psum = reinterpret_cast<float*>(smem + L.s_psum);        // [NSPLIT][kRows]
-    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L.s_bar);
-    uint32_t* slot = reinterpret_cast<uint32_t*>(smem + L.s_slot);
-    constexpr int kThreads = 128 * NSPLIT;
-    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    const int quarter = w & 3, part = w >> 2;
-    constexpr int RPQ = MT / 4;                   // rows per lane quarter
-    const bool has_row = lane < RPQ;
-    const int row = RPQ * quarter + (has_row ? lane : 0);   // row this thread reads and writes
-    const int KH = K / NSPLIT;                    // columns per part
-    const int c0 = part * KH;                     // first column of this thread's part
-    const int nch = K >> 3;
+// Sums of C columns over the 32 lanes of a warp: lane l returns the sum of column *col, added
+// as the binary tree over the lanes (pairs at distance 1, then 2, 4, 8, 16).  While more than
+// one column is left, a level also halves the columns a lane keeps.
+template <int C>
+__device__ __forceinline__ float lane_sums(float (&v)[C], int lane, int* col) {
+    int n = C, c = 0;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = (lane & d) != 0;
+#pragma unroll
+            for (int i = 0; i < C / 2; ++i) {
+                if (i < n) {
+                    const float keep = up ? v[i + n] : v[i], send = up ? v[i] : v[i + n];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, d);
+                }
+            }
+            c += up ? n : 0;
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], d);
+        }
+    }
+    *col = c;
+    return v[0];
+}
 
-    // ---- stage A^T and the emission table (linear copies of prepared layouts)
-    {
-        const int4* src = reinterpret_cast<const int4*>(g_at);
-        int4* dst = reinterpret_cast<int4*>(sAT);
-        for (int i = tid; i < K * K * 2 / 16; i += kThreads) dst[i] = src[i];
-        src = reinterpret_cast<const int4*>(g_etab);
-        dst = reinterpret_cast<int4*>(sE);
-        for (int i = tid; i < M * K * 2 / 16; i += kThreads) dst[i] = src[i];
+template <int C>
+__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float (&v)[C]) {
+    uint32_t r[C];
+    if constexpr (C == 8) tc::tmem_ld8(taddr, r);
+    else if constexpr (C == 16) tc::tmem_ld16(taddr, r);
+    else tc::tmem_ld32(taddr, r);
+#pragma unroll
+    for (int i = 0; i < C; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
+    const __nv_bfloat162 m = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+    return *reinterpret_cast<const uint32_t*>(&m);
+}
+
+// Maxima of W words of two BF16 columns over the 32 lanes: lane l returns word *word (a
+// reduce-scatter, as lane_sums).
+template <int W>
+__device__ __forceinline__ uint32_t lane_max(uint32_t (&v)[W], int lane, int* word) {
+    int n = W, c = 0;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = (lane & d) != 0;
+#pragma unroll
+            for (int i = 0; i < W / 2; ++i) {
+                if (i < n) {
+                    const uint32_t keep = up ? v[i + n] : v[i], send = up ? v[i] : v[i + n];
+                    v[i] = max_bf16x2(keep, __shfl_xor_sync(0xffffffffu, send, d));
+                }
+            }
+            c += up ? n : 0;
+        } else {
+            v[0] = max_bf16x2(v[0], __shfl_xor_sync(0xffffffffu, v[0], d));
+        }
     }
-    const uint32_t ncols = K <= 64 ? 64 : K <= 128 ? 128 : 256;
-    if (w == 0) {
-        tc::tmem_alloc(slot, ncols);
+    *word = c;
+    return v[0];
+}
+
+// A wait on a step's path.  The first poll suspends the warp until the phase completes, so it
+// is nearly always the only one; `fail` is set when the wait gives up.
+__device__ __noinline__ bool wait_slow(uint64_t* bar, uint32_t parity, volatile uint32_t* fail) {
+    if (tc::mbar_wait_bounded(bar, parity, kWaitNs)) return true;
+    *fail = 1;
+    return false;
+}
+__device__ __forceinline__ bool wait_step(uint64_t* bar, uint32_t parity, volatile uint32_t* fail) {
+    return tc::mbar_try_wait(bar, parity) || wait_slow(bar, parity, fail);
+}
+
+constexpr int tile_threads(int K, int N) {
+    return 128 * ((K + 127) / 128) * col_parts(N) + 32 * ((K + 127) / 128 + 1 + max_warps(K, N));
+}
+
+// N = sequences of the tile, TE = emission table type.
+template <int K, int N, typename TE>
+__global__ void __launch_bounds__(tile_threads(K, N), 1)
+k_hmm_tc(int M, const float* __restrict__ log_A, const float* __restrict__ log_B,
+         const float* __restrict__ log_pi, const int32_t* __restrict__ obs, const int64_t* __restrict__ off,
+         int64_t S, const int32_t* __restrict__ order, unsigned long long* __restrict__ next,
+         const int32_t* __restrict__ pick, double* __restrict__ loglik, int32_t* __restrict__ status,
+         uint64_t watchdog_ns, uint32_t tmem_cols) {
+    if (pick && *pick != N) return;               // the other tile size runs this call
+    constexpr int NH = (K + 127) / 128;           // blocks of 128 states
+    constexpr int PARTS = col_parts(N);
+    constexpr int NEPI = 4 * NH * PARTS;          // epilogue warps; then NH issuing, the bookkeeping and the max warps
+    constexpr int CPT = N / PARTS;                // columns (sequences) of an epilogue thread
+    constexpr int CH = CPT < 32 ? CPT : 32;       // ... taken CH at a time
+    constexpr int NU = N < 32 ? 1 : N / 32;       // sequences of a bookkeeping lane
+    constexpr int NMX = max_warps(K, N);
+    constexpr int MXP = NMX > 0 ? NH : K / 32;    // maxima per column
+    constexpr int kThreads = tile_threads(K, N);
+    extern __shared__ __align__(1024) char smem[];
+    const TileLayout L = tile_layout(K, M, N, (int)sizeof(TE));
+    char* sX = smem + L.x;
+    TE* sE = reinterpret_cast<TE*>(smem + L.e);
+    float* s_scale = reinterpret_cast<float*>(smem + L.scale);
+    int32_t* s_sym = reinterpret_cast<int32_t*>(smem + L.sym);
+    Ctl* s_ctl = reinterpret_cast<Ctl*>(smem + L.ctl);
+    uint16_t* s_mx = reinterpret_cast<uint16_t*>(smem + L.mx);
+    float* s_ps = reinterpret_cast<float*>(smem + L.psum);
+    uint64_t* bar_mma = reinterpret_cast<uint64_t*>(smem + L.bar);      // [2] per block of states: D ready
+    uint64_t* bar_x = bar_mma + 2;                                      // X written, D read
+    uint64_t* bar_info = bar_mma + 4;                                   // [2] per step parity: scale, sym, ... written
+    uint64_t* bar_ps = bar_mma + 6;                                     // [2] per step parity: row sums written
+    uint64_t* bar_mx = bar_mma + 8;                                     // [2] per step parity: column maxima written
+    uint32_t* slot = reinterpret_cast<uint32_t*>(smem + L.slot);
+    volatile uint32_t* s_fail = slot + 1;         // set by a warp whose wait gave up
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const int quarter = w & 3, half = (w >> 2) % NH, part = (w >> 2) / NH;
+    const int j = 128 * half + 32 * quarter + lane;
+    const bool valid = K % 128 == 0 || j < K;     // uniform over a warp: K is a multiple of 32
+
+    if (w == NEPI) {
+        tc::tmem_alloc(slot, tmem_cols);
         tc::tmem_relinquish();
+        if (lane == 0) {
+            for (int h = 0; h < 2; ++h) {
+                tc::mbar_init(&bar_mma[h], 1);
+                tc::mbar_init(&bar_info[h], 1);
+                tc::mbar_init(&bar_ps[h], NEPI);
+                tc::mbar_init(&bar_mx[h], NMX > 0 ? NMX : NEPI);
+            }
+            tc::mbar_init(bar_x, NEPI);
+            tc::fence_mbar_init();
+            *s_fail = 0;
+        }
     }
-    if (tid == 0) {
-        tc::mbar_init(bar, 1);
-        tc::fence_mbar_init();
+    // b(j, o) = exp(log B[j, o]) rounded to BF16, symbol-major; X starts at zero (its columns
+    // without a sequence are never read back)
+    for (int idx = tid; idx < M * K; idx += kThreads) {
+        const int o = idx / K, s = idx - o * K;
+        const __nv_bfloat16 b = __float2bfloat16_rn(__expf(log_B[s * M + o]));
+        if constexpr (sizeof(TE) == 4) sE[idx] = __bfloat162float(b); else sE[idx] = b;
     }
+    for (int idx = tid; idx < (int)(2 * L.x_bytes / 16); idx += kThreads)
+        reinterpret_cast<int4*>(sX)[idx] = make_int4(0, 0, 0, 0);
+    tc::fence_proxy_async_smem();
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *slot;
-    const uint32_t taddr = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)c0;
-
-    const uint32_t idesc = tc::idesc_bf16_f32(MT, K);
-    const uint32_t sx_addr = tc::smem_u32(sX), sat_addr = tc::smem_u32(sAT);
-    const uint32_t sbo = 16u * (uint32_t)K;
-    const uint64_t adesc0 = tc::smem_desc_noswizzle(sx_addr, 128, sbo);
-    const uint64_t bdesc0 = tc::smem_desc_noswizzle(sat_addr, 128, sbo);
-
-    // row bookkeeping, kept by the row's owner thread (part 0)
-    const bool owner = part == 0 && has_row;
-    int64_t seq = -1, T = 0, pos = 0, E = 0;
-    const int32_t* o = nullptr;
-    int32_t nob = 0;             // o[pos + 1], loaded one step ahead of its use
-    int32_t kcur = 0;            // exponent applied to this step's X
-    float uprev = 0.f;           // log2 sum(X_{t-1})
-    bool queue_empty = !has_row || row >= rows_active;   // rows past rows_active never take sequences
-    volatile uint32_t* s_flag = slot + 1;                 // set by a thread whose wait timed out
-    if (tid == 0) *s_flag = 0;
-    // watchdog: when the launch has run longer than watchdog_ns (0 = no limit), thread 0 stops
-    // it at the next step boundary -- after the previous step's MMAs have completed and before
-    // new ones are issued, so no tensor-core work is in flight -- and every thread leaves
-    // through the normal exit that frees the tensor memory
-    const uint64_t t_launch = watchdog_ns != 0 ? tc::globaltimer_ns() : 0;
-
-    // emission b(j, ob) for j in [jc, jc+32), FP32, times `scale` (a power of two: exact)
-    auto load_emis = [&](int ob, int jc, float (&b)[32], float scale) {
-        const int qb = ((jc >> 3) + ob) % nch;
+    const uint32_t tmem_a = tmem + (uint32_t)(NH * N);
+    // A^T into tensor memory: lane j of block `half`, column c = (A[2c][j], A[2c+1][j])
+    if (w < NEPI) {
+        const int c1 = (part + 1) * (K / 2 / PARTS);
+        for (int c0 = part * (K / 2 / PARTS); c0 < c1; c0 += 16) {
+            uint32_t r[16];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int q = qb + u < nch ? qb + u : qb + u - nch;
-            uint4 r = *reinterpret_cast<const uint4*>(sE + ob * K * 2 + q * 16);
-            b[8 * u + 0] = bf_lo(r.x) * scale; b[8 * u + 1] = bf_hi(r.x) * scale;
-            b[8 * u + 2] = bf_lo(r.y) * scale; b[8 * u + 3] = bf_hi(r.y) * scale;
-            b[8 * u + 4] = bf_lo(r.z) * scale; b[8 * u + 5] = bf_hi(r.z) * scale;
-            b[8 * u + 6] = bf_lo(r.w) * scale; b[8 * u + 7] = bf_hi(r.w) * scale;
+            for (int e = 0; e < 16; ++e) {
+                const float* a = log_A + (int64_t)(2 * (c0 + e)) * K + j;
+                r[e] = valid ? pack_bf16(__expf(a[0]), __expf(a[K])) : 0u;
+            }
+            tc::tmem_st16(tmem_a + (uint32_t)(half * (K / 2) + c0) + ((uint32_t)(32 * quarter) << 16), r);
         }
-    };
-    // row values of columns [jc, jc+32): X = a o bs (a = D, or pi for a fresh row), packed to
-    // BF16 and stored; returns their sum (a fixed pairwise tree)
-    auto epi_chunk = [&](const float* a, const float (&bs)[32], int jc) -> float {
-        float part8[8];
+        tc::tmem_wait_st();
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+
+    if (w >= NEPI && w < NEPI + NH) {
+        // ---- an issuing warp: block h of D = A^T X_{t-1}
+        const int h = w - NEPI;
+        constexpr uint32_t idesc = tc::idesc_bf16_f32(128, N) | tc::kIdescBMnMajor;
+        const uint64_t xdesc0 = tc::smem_desc_noswizzle(tc::smem_u32(sX), 128, 16u * (uint32_t)K);
+        const uint32_t d = tmem + (uint32_t)(h * N), a = tmem_a + (uint32_t)(h * (K / 2));
+        uint32_t issued = 0;
+        for (uint32_t iter = 0;; ++iter) {
+            const uint32_t par = iter & 1u, pprev = par ^ 1u;
+            if (!wait_step(&bar_info[par], (iter >> 1) & 1u, s_fail) || s_ctl[iter & 3u].done != 0) break;
+            if (iter > 0) wait_step(bar_x, pprev, s_fail);
+            tc::tc_fence_after();
+            const uint64_t xd = xdesc0 + (uint64_t)(pprev * (L.x_bytes >> 4));
+            if (tc::elect_one()) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            float v[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = a[8 * u + e] * bs[8 * u + e];
-            uint4 pk;
-            pk.x = pack_bf16(v[0], v[1]);
-            pk.y = pack_bf16(v[2], v[3]);
-            pk.z = pack_bf16(v[4], v[5]);
-            pk.w = pack_bf16(v[6], v[7]);
-            *reinterpret_cast<uint4*>(sX + canon_off(row, jc + 8 * u, K)) = pk;
-            part8[2 * u] = (v[0] + v[1]) + (v[2] + v[3]);
-            part8[2 * u + 1] = (v[4] + v[5]) + (v[6] + v[7]);
+                for (int ks = 0; ks < K / 16; ++ks)
+                    tc::mma_bf16_ts(d, a + ks * 8, xd + ks * 16, idesc, ks > 0 ? 1u : 0u);
+                tc::mma_commit(&bar_mma[h]);
+            }
+            __syncwarp();
+            issued = iter + 1;
         }
-        return ((part8[0] + part8[1]) + (part8[2] + part8[3])) + ((part8[4] + part8[5]) + (part8[6] + part8[7]));
-    };
-    // take the next sequence of the queue on this row (owner thread).  Its first vector
-    // alpha~_0 = pi o b(o_0) (unscaled: k_0 = 0) is written by the row's epilogue threads in
-    // the next epilogue, flagged by rinfo.ob = -(o_0 + 2).
-    auto take_next = [&]() {
-        seq = -1;
-        if (!queue_empty) {
-            const unsigned long long q = atomicAdd(next, 1ull);
-            if (q >= (unsigned long long)S) {
-                queue_empty = true;
-            } else {
-                seq = order[q];
-                const int64_t o0 = off[seq];
-                T = off[seq + 1] - o0;
-                o = obs + o0;
-                pos = 0;
-                E = 0;
-                kcur = 0;
-                nob = T > 1 ? o[1] : 0;
-                rinfo[row].ob = (int16_t)(-(o[0] + 2));
-                rinfo[row].k = 0;
+        // the products issued last complete before the tensor memory goes
+        if (issued > 0) tc::mbar_wait_bounded(&bar_mma[h], (issued - 1) & 1u, kWaitNs);
+    } else if (w == NEPI + NH) {
+        // ---- the bookkeeping warp (lane l: columns l, l + 32, ...)
+        const uint64_t t_launch = watchdog_ns != 0 ? tc::globaltimer_ns() : 0;
+        const int64_t ncta = gridDim.x;
+        // the sequence on the column at the step last published, with the steps left after it
+        int32_t seq[NU];
+        int64_t left[NU];
+        const int32_t* o[NU];                     // its next symbol
+        int32_t nob[NU];                          // ... loaded one step ahead
+        bool fresh[NU], dry[NU];
+        auto start = [&](int u, int64_t q) {
+            seq[u] = -1;
+            if (q >= S) {
+                dry[u] = true;
                 return;
             }
-        }
-        rinfo[row].ob = -1;
-        rinfo[row].k = 0;
-    };
-
-    // Step loop.  Iteration i: (A) X is complete -> one thread issues the MMAs D = X A;
-    // meanwhile the owners process the row sums of the previous epilogue (logL at a
-    // sequence's end, the next exponent, the next symbol, or the next sequence); (B) every
-    // thread waits for the MMAs and writes the next X (or a fresh row's alpha~_0).
-    if (owner) take_next();
-    for (uint32_t iter = 0;; ++iter) {
-        // ---- (A) publish X; the MMAs of this iteration
-        tc::fence_proxy_async_smem();
-        tc::tc_fence_before();
-        if (watchdog_ns != 0 && tid == 0 && tc::globaltimer_ns() - t_launch > watchdog_ns) *s_flag = 2;
-        const bool any = __syncthreads_or(owner && seq >= 0);
-        if (*s_flag != 0) {
-            if (tid == 0) report_status(status, ACCEL_ERR_TIMEOUT);
-            break;
-        }
-        if (!any) break;
-        if (tid == kRows) {              // a thread of column part 1: never a row owner
-            tc::tc_fence_after();
-            // k-step ks is 256 bytes further: 16 in the descriptors' address field
-            uint64_t ad = adesc0, bd = bdesc0;
-            tc::mma_bf16(tmem, ad, bd, idesc, 0u);
-            for (int ks = 1; ks < K / 16; ++ks) {
-                ad += 16;
-                bd += 16;
-                tc::mma_bf16(tmem, ad, bd, idesc, 1u);
+            seq[u] = order ? order[q] : (int32_t)q;
+            const int64_t o0 = off[seq[u]];
+            left[u] = off[seq[u] + 1] - o0 - 1;
+            o[u] = obs + o0 + 1;
+            nob[u] = obs[o0];
+            fresh[u] = true;
+        };
+        // what a step is to the column: 1 it has a sequence, 2 it begins, 4 it ends
+        auto state = [&](int u) -> uint32_t {
+            return seq[u] < 0 ? 0u : 1u | (fresh[u] ? 2u : 0u) | (left[u] <= 0 ? 4u : 0u);
+        };
+        auto publish = [&](int u, uint32_t step, uint32_t st) {     // all but the exponents
+            if (u * 32 + lane < N) s_sym[(step & 3u) * N + u * 32 + lane] = st & 1u ? nob[u] * K : 0;
+            if ((st & 5u) == 1u) nob[u] = *o[u]++;
+            const uint32_t fm = __ballot_sync(0xffffffffu, st & 2u);
+            const uint32_t em = __ballot_sync(0xffffffffu, st & 4u);
+            if (lane == 0) {
+                s_ctl[step & 3u].fresh[u] = fm;
+                s_ctl[step & 3u].end[u] = em;
             }
-            tc::mma_commit(bar);
-        }
-        // ---- bookkeeping of the previous epilogue's rows (owner threads), overlapping the MMAs
-        if (owner && seq >= 0 && iter > 0) {
-            float s = psum[row];
+            return em != 0;
+        };
+        // steps i - 1 and i: what they are to the column, their sequences, exponents and the
+        // exponents before them
+        uint32_t st1[NU], st0[NU];
+        int32_t sq1[NU], sq0[NU], k1[NU], k0[NU];
+        int64_t E1[NU], E0[NU];
 #pragma unroll
-            for (int q = 1; q < NSPLIT; ++q) s += psum[q * kRows + row];
-            if (pos == T - 1) {
-                loglik[seq] = 0.6931471805599453 * (double)E + log((double)s);
-                take_next();
-            } else {
-                E += kcur;
-                const float ls = __log2f(s);
-                const float u = ls - (float)kcur;       // log2 sum(X_t)
-                const float lr = pos == 0 ? ls : ls - uprev;   // log2 of the growth sum(X_{t-1}) -> s_t
-                uprev = u;
-                kcur = (int)rintf(u + lr);
-                ++pos;
-                rinfo[row].ob = (int16_t)nob;
-                rinfo[row].k = (int16_t)kcur;
-                nob = pos + 1 < T ? o[pos + 1] : 0;
-            }
+        for (int u = 0; u < NU; ++u) {
+            dry[u] = u * 32 + lane >= N;
+            seq[u] = -1;
+            fresh[u] = false;
+            left[u] = 0;
+            nob[u] = 0;
+            // the first N x grid positions are dealt out
+            if (!dry[u]) start(u, blockIdx.x + (int64_t)(u * 32 + lane) * ncta);
+            st1[u] = 0;
+            sq1[u] = -1;
+            k1[u] = k0[u] = 0;
+            E1[u] = E0[u] = 0;
+            st0[u] = state(u);
+            sq0[u] = seq[u];
         }
-        __syncthreads();
-        // ---- (B) epilogue
-        const RowInfo ri = rinfo[row];
-        const bool fresh = has_row && ri.ob <= -2;
-        const bool act = has_row && ri.ob >= 0;
-        const int ob = fresh ? -ri.ob - 2 : ri.ob;
-        const float mult = ldexpf(1.0f, -(int)ri.k);
-        // the first chunk's emission (scaled by 2^-k) is read while the MMAs run
-        float bs[32];
-        if (act || fresh) load_emis(ob, c0, bs, mult);
-        const bool ok = tc::mbar_wait_bounded(bar, iter & 1, kWaitNs);
-        if (!ok) *s_flag = 1;
-        tc::tc_fence_after();
-        // each thread's part of the row of D (tcgen05.ld is warp-collective); the row sum is
-        // accumulated over the scaled values and unscaled by 2^k (exact) at the end
-        float ps = 0.f;
-        if (__any_sync(0xffffffffu, act)) {
-            if (KH % 64 == 0) {
-                for (int jc = 0; jc < KH; jc += 64) {
-                    uint32_t d[64];
-                    tc::tmem_ld64(taddr + jc, d);
-                    if (act) {
-                        if (jc > 0) load_emis(ob, c0 + jc, bs, mult);
-                        ps += epi_chunk(reinterpret_cast<const float*>(d), bs, c0 + jc);
-                        load_emis(ob, c0 + jc + 32, bs, mult);
-                        ps += epi_chunk(reinterpret_cast<const float*>(d) + 32, bs, c0 + jc + 32);
-                    }
+        bool ended1 = false, ended0 = false;      // whether steps i - 1 and i end a sequence
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            ended0 = publish(u, 0, st0[u]) || ended0;
+            if (u * 32 + lane < N) s_scale[u * 32 + lane] = 1.f;
+        }
+        if (lane == 0) s_ctl[0].done = 0;
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&bar_info[0]);
+        uint32_t ps_phase = 0;                    // bit p: parity of the next completion of bar_ps[p]
+        for (uint32_t iter = 0;; ++iter) {
+            const uint32_t pprev = (iter & 1u) ^ 1u;
+            // ---- step i + 1: what it is, and its symbols
+            uint32_t st[NU];
+            bool any = false, ended = false;
+#pragma unroll
+            for (int u = 0; u < NU; ++u) {
+                if (st0[u] & 4u) {
+                    seq[u] = -1;
+                    if (next && !dry[u]) start(u, (int64_t)N * ncta + (int64_t)atomicAdd(next, 1ull));
+                } else {
+                    fresh[u] = false;
+                    --left[u];
                 }
-            } else {
-                for (int jc = 0; jc < KH; jc += 32) {
-                    uint32_t d[32];
-                    tc::tmem_ld32(taddr + jc, d);
-                    if (act) {
-                        if (jc > 0) load_emis(ob, c0 + jc, bs, mult);
-                        ps += epi_chunk(reinterpret_cast<const float*>(d), bs, c0 + jc);
-                    }
-                }
+                st[u] = state(u);
+                any = any || ((st0[u] | st[u]) & 1u);
+                ended = publish(u, iter + 1, st[u]) || ended;
             }
-            ps *= ldexpf(1.0f, (int)ri.k);
-        }
-        if (fresh) {
-            // alpha~_0 = pi o b(o_0) for this thread's columns
-            for (int jc = 0; jc < KH; jc += 32) {
-                if (jc > 0) load_emis(ob, c0 + jc, bs, 1.f);
-                float pv[32];
+            bool stop = !__any_sync(0xffffffffu, any);
+            if (watchdog_ns != 0 && tc::globaltimer_ns() - t_launch > watchdog_ns) *s_fail = 1;
+            stop = __any_sync(0xffffffffu, stop || *s_fail != 0);
+            if (lane == 0) s_ctl[(iter + 1) & 3u].done = stop ? 1u : 0u;
+            // ---- its exponents, from the maxima of X_{i-1}
+            if (iter > 0) wait_step(&bar_mx[pprev], ((iter - 1) >> 1) & 1u, s_fail);
+            int32_t kn[NU];
 #pragma unroll
-                for (int u = 0; u < 32; ++u) pv[u] = __expf(log_pi[c0 + jc + u]);
-                ps += epi_chunk(pv, bs, c0 + jc);
+            for (int u = 0; u < NU; ++u) {
+                const int c = u * 32 + lane < N ? u * 32 + lane : 0;
+                uint32_t m = 0;
+#pragma unroll
+                for (int q = 0; q < MXP; ++q) m = max(m, (uint32_t)s_mx[(pprev * MXP + q) * N + c]);
+                // (at a sequence's second step X_{i-1} is not its own: 0 stands for log2 of 1)
+                const int32_t x = st0[u] & 2u ? 0 : (int32_t)(m >> 7) - 127;
+                int32_t k = x - k0[u] - kTarget;
+                k = k < -kMaxScale ? -kMaxScale : k > kMaxScale ? kMaxScale : k;
+                kn[u] = (st[u] & 3u) == 1u ? k : 0;
+                if (u * 32 + lane < N) s_scale[pprev * N + u * 32 + lane] = __uint_as_float((uint32_t)(127 - kn[u]) << 23);
             }
-        }
-        if (has_row) psum[part * kRows + row] = ps;
-    }
-    tc::tc_fence_before();
-    __syncthreads();
-    if (w == 0) tc::tmem_dealloc(tmem, ncols);
-}
-
-// ============================================================================================
-// Cluster-pair variant.  The two CTAs of a cluster run the same tile of sequence rows and
-// split the state columns: CTA r computes D_r = X A[:, r K/2 : (r+1) K/2] (MMA N = K/2, half
-// the tensor-core time of a step), holds only its half of A^T and of the emission table, and
-// runs the epilogue of its own columns (half the per-row work).  Each CTA writes its half of
-// X_t into its own tile and, with st.async, into its peer's, together with its partial row
-// sums; the stores count their bytes on the receiver's mbarrier of that step's parity, so a
-// CTA waits for its peer's half with no cluster barrier per step -- and only after issuing the
-// MMAs over its own half of X (half of the K/16 k-steps), which hide the exchange latency.
-// X is double-buffered by
-// step parity: a peer can be one step ahead and must not overwrite the tile the MMA reads.
-// Both CTAs do the same row bookkeeping on the same sums (added in the same order), so they
-// agree on every exponent and on the end of every sequence; CTA 0 alone writes logL and pops
-// the sequence queue, and sends the popped index to CTA 1 in the same exchange.  A row that
-// takes a new sequence this way idles for one step while the index travels.
-// ============================================================================================
-struct PairLayout {
-    uint32_t s_at, s_x, x_bytes, s_e, s_rowinfo, s_psum, s_mail, s_bar, s_slot, smem_bytes;
-};
-
-// NC = CTAs of the cluster (2 or 4); each holds KC = K / NC state columns.
-static PairLayout pair_layout(int K, int M, int MT, int NSPLIT, int NC) {
-    PairLayout L;
-    const uint32_t KC = (uint32_t)(K / NC);
-    uint32_t o = 0;
-    L.s_at = o; o += KC * (uint32_t)K * 2;                 // this CTA's part of A^T (N = K/NC rows)
-    L.x_bytes = (uint32_t)MT * (uint32_t)K * 2;
-    L.s_x = o;  o += 2 * L.x_bytes;                        // X, one buffer per step parity
-    L.s_e = o;  o += (uint32_t)M * KC * 2;                 // emission columns of this part
-    o = (o + 15) & ~15u;
-    L.s_rowinfo = o; o += (uint32_t)MT * (uint32_t)sizeof(RowInfo);
-    L.s_psum = o; o += 2 * (uint32_t)NC * (uint32_t)NSPLIT * (uint32_t)MT * 4;   // [parity][cta][part][row]
-    L.s_mail = o; o += 2 * (uint32_t)MT * 4;                                     // [parity][row] popped index
-    o = (o + 7) & ~7u;
-    L.s_bar = o; o += 3 * 8;                                          // MMA, exchange x 2 parities
-    L.s_slot = o; o += 8;
-    L.smem_bytes = o;
-    return L;
-}
-
-bool tc_cl_supported(int K, int M, int rows, int split, int nc) {
-    if (nc != 2 && nc != 4) return false;
-    if (K < 64 * nc || K > 256 || K % 64 != 0 || M < 1 || M > 32767 || (split != 2 && split != 4)) return false;
-    if ((K / nc / split) % 32 != 0) return false;
-    const int MT = rows <= 64 ? 64 : 128;
-    return (int)pair_layout(K, M, MT, split, nc).smem_bytes <= max_smem_optin();
-}
-
-// Launched with a cluster of NC CTAs (cudaLaunchKernelEx, cluster-dimension attribute).
-template <int NSPLIT, int MT, int NC>
-__global__ void __launch_bounds__(128 * NSPLIT, 1)
-k_hmm_tc_pair(int K, int M, const char* __restrict__ g_at, const char* __restrict__ g_etab,
-              const float* __restrict__ log_pi, const int32_t* __restrict__ obs, const int64_t* __restrict__ off,
-              int64_t S, const int32_t* __restrict__ order, unsigned long long* __restrict__ next, int rows_active,
-              double* __restrict__ loglik, int32_t* __restrict__ status, PairLayout L) {
-    extern __shared__ __align__(1024) char smem[];
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
-    const int rank = (int)cl.block_rank();
-    const int cid = (int)(blockIdx.x / NC), ncl = (int)(gridDim.x / NC);
-    char* sAT = smem + L.s_at;
-    char* sX = smem + L.s_x;
-    char* sE = smem + L.s_e;
-    RowInfo* rinfo = reinterpret_cast<RowInfo*>(smem + L.s_rowinfo);
-    float* psum = reinterpret_cast<float*>(smem + L.s_psum);
-    int32_t* mail = reinterpret_cast<int32_t*>(smem + L.s_mail);
-    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L.s_bar);
-    uint32_t* slot = reinterpret_cast<uint32_t*>(smem + L.s_slot);
-    constexpr int kThreads = 128 * NSPLIT;
-    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    const int quarter = w & 3, part = w >> 2;
-    // MT = 128: row 32 q + lane of lane quarter q, one thread per row and part.  MT = 64: the
-    // rows sit in lanes 0-15 of each quarter, and threads t and t + 16 share row 16 q + t%16,
-    // each taking half of the part's columns (16-lane TMEM loads).
-    constexpr bool HL = MT == 64;
-    const int hsel = HL ? lane >> 4 : 0;
-    const int row = HL ? 16 * quarter + (lane & 15) : 32 * quarter + lane;
-    const int KC = K / NC;                        // columns of this CTA
-    const int KH = KC / NSPLIT;                   // columns per part
-    const int CPT = HL ? KH / 2 : KH;             // columns per thread
-    const int l0 = part * KH;                     // first column of the part, within the half
-    const int lt = l0 + hsel * CPT;               // first column of this thread, within the half
-    const int gt = rank * KC + lt;                // ... and in the full row
-    const int nch = K >> 3, nchh = KC >> 3;
-
-    // ---- stage this half of A^T (rows rank*KC.. of the canonical layout are one block) and
-    // the emission columns of this half (16-byte chunks re-rotated within the half)
-    {
-        const int4* src = reinterpret_cast<const int4*>(g_at + (size_t)rank * KC * K * 2);
-        int4* dst = reinterpret_cast<int4*>(sAT);
-        for (int i = tid; i < KC * K * 2 / 16; i += kThreads) dst[i] = src[i];
-        for (int i = tid; i < M * nchh; i += kThreads) {
-            const int ob = i / nchh, c = i - ob * nchh;
-            const int qs = (rank * nchh + c + ob) % nch, qd = (c + ob) % nchh;
-            reinterpret_cast<int4*>(sE + (size_t)ob * KC * 2)[qd] =
-                reinterpret_cast<const int4*>(g_etab + (size_t)ob * K * 2)[qs];
-        }
-        for (int i = tid; i < 2 * MT; i += kThreads) mail[i] = -1;
-    }
-    if (w == 0) {
-        tc::tmem_alloc(slot, (uint32_t)KC);
-        tc::tmem_relinquish();
-    }
-    if (tid == 0) {
-        tc::mbar_init(&bar[0], 1);
-        tc::mbar_init(&bar[1], 1);
-        tc::mbar_init(&bar[2], 1);
-        tc::fence_mbar_init();
-    }
-    volatile uint32_t* s_flag = slot + 1;
-    if (tid == 0) *s_flag = 0;
-    tc::tc_fence_before();
-    cl.sync();                                    // both CTAs' barriers exist before any st.async
-    tc::tc_fence_after();
-    const uint32_t tmem = *slot;
-    const uint32_t taddr = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(HL ? l0 : lt);
-    const uint32_t idesc = tc::idesc_bf16_f32(MT, KC);
-    const uint32_t sx_addr = tc::smem_u32(sX), sat_addr = tc::smem_u32(sAT);
-    const uint32_t sbo = 16u * (uint32_t)K;
-    // the other CTAs of the cluster, d = 1 .. NC-1: CTA (rank + d) % NC
-    uint32_t rx[NC - 1], rpsum[NC - 1], rmail[NC - 1], rbar0[NC - 1], rbar1[NC - 1];
+            // the row sums of the sequences that ended at step i - 1, before step i + 1 may write
+            // its own in their place
+            float sums[NU];
+            if (ended1) {
+                wait_step(&bar_ps[pprev], (ps_phase >> pprev) & 1u, s_fail);
+                ps_phase ^= 1u << pprev;
 #pragma unroll
-    for (int d = 1; d < NC; ++d) {
-        const uint32_t pr = (uint32_t)((rank + d) % NC);
-        rx[d - 1] = tc::cluster_addr(sX, pr);
-        rpsum[d - 1] = tc::cluster_addr(psum, pr);
-        rmail[d - 1] = tc::cluster_addr(mail, pr);
-        rbar0[d - 1] = tc::cluster_addr(&bar[1], pr);
-        rbar1[d - 1] = tc::cluster_addr(&bar[2], pr);
-    }
-    // bytes a CTA receives per step: the other CTAs' parts of X and partial sums, and (CTAs
-    // other than 0) the indices CTA 0 popped
-    const uint32_t xbytes = (uint32_t)((NC - 1) * (MT * KC * 2 + MT * NSPLIT * 4) + (rank != 0 ? MT * 4 : 0));
-
-    const bool owner = part == 0 && hsel == 0;
-    int64_t seq = -1, T = 0, pos = 0, E = 0;     // seq: -1 none, -2 waiting for CTA 0's index
-    const int32_t* o = nullptr;
-    int32_t nob = 0;
-    int32_t kcur = 0;
-    float uprev = 0.f;
-    bool queue_empty = row >= rows_active;
-    const int64_t qbase = (int64_t)rows_active * ncl;   // the first rows_active x ncl entries are dealt out
-
-    // emission b(j, ob) for the 16 columns [jc, jc+16) of this half, times `scale` (a power of two)
-    auto load_emis = [&](int ob, int jc, float (&b)[16], float scale) {
-        const int qb = ((jc >> 3) + ob) % nchh;
+                for (int u = 0; u < NU; ++u) {
+                    sums[u] = 0.f;
+                    if (st1[u] & 4u) {
+                        // in the order of the states: chunks of 32, in K / 4 or K / 2 parts
+                        constexpr int np = (K / 4) % 32 == 0 ? 4 : 2, cpp = K / 32 / np;
+                        const float* ps = s_ps + (size_t)pprev * (K / 32) * N + u * 32 + lane;
+                        float sum = 0.f;
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int q = qb + u < nchh ? qb + u : qb + u - nchh;
-            uint4 r = *reinterpret_cast<const uint4*>(sE + ob * KC * 2 + q * 16);
-            b[8 * u + 0] = bf_lo(r.x) * scale; b[8 * u + 1] = bf_hi(r.x) * scale;
-            b[8 * u + 2] = bf_lo(r.y) * scale; b[8 * u + 3] = bf_hi(r.y) * scale;
-            b[8 * u + 4] = bf_lo(r.z) * scale; b[8 * u + 5] = bf_hi(r.z) * scale;
-            b[8 * u + 6] = bf_lo(r.w) * scale; b[8 * u + 7] = bf_hi(r.w) * scale;
-        }
-    };
-    // columns [jc, jc+16) of this half: X = a o bs packed to BF16 into the buffer at xo of both
-    // CTAs; returns their sum (a fixed pairwise tree)
-    auto epi16 = [&](const float* a, const float (&bs)[16], int jc, uint32_t xo, const uint32_t (&rb)[NC - 1]) -> float {
-        float part4[4];
+                        for (int p = 0; p < np; ++p) {
+                            float c = ps[p * cpp * N];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            float v[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = a[8 * u + e] * bs[8 * u + e];
-            uint4 pk;
-            pk.x = pack_bf16(v[0], v[1]);
-            pk.y = pack_bf16(v[2], v[3]);
-            pk.z = pack_bf16(v[4], v[5]);
-            pk.w = pack_bf16(v[6], v[7]);
-            const uint32_t co = xo + canon_off(row, rank * KC + jc + 8 * u, K);
-            *reinterpret_cast<uint4*>(sX + co) = pk;
-#pragma unroll
-            for (int d = 0; d < NC - 1; ++d) tc::st_async_u4(rx[d] + co, pk, rb[d]);
-            part4[2 * u] = (v[0] + v[1]) + (v[2] + v[3]);
-            part4[2 * u + 1] = (v[4] + v[5]) + (v[6] + v[7]);
-        }
-        return (part4[0] + part4[1]) + (part4[2] + part4[3]);
-    };
-    auto start = [&](int32_t sq) {
-        seq = sq;
-        const int64_t o0 = off[sq];
-        T = off[sq + 1] - o0;
-        o = obs + o0;
-        pos = 0;
-        E = 0;
-        kcur = 0;
-        nob = T > 1 ? o[1] : 0;
-        rinfo[row].ob = (int16_t)(-(o[0] + 2));
-        rinfo[row].k = 0;
-    };
-    auto idle = [&](int64_t state) {
-        seq = state;
-        rinfo[row].ob = -1;
-        rinfo[row].k = 0;
-    };
-    if (owner) {
-        const int64_t q0 = (int64_t)row * ncl + cid;
-        if (row < rows_active && q0 < S) start(order[q0]);
-        else idle(-1);
-    }
-
-    uint32_t xph = 0;                             // bit p: parity of the next completion of exchange barrier p
-    // bounded wait for the peer's bytes of step parity q
-    auto xchg_wait = [&](int q) {
-        const uint32_t ph = (xph >> q) & 1u;
-        uint64_t t0 = 0;
-        for (uint32_t i = 0;; ++i) {
-            if (tc::mbar_try_wait_cluster(&bar[1 + q], ph)) break;
-            if ((i & 255) == 0) {
-                const uint64_t now = tc::globaltimer_ns();
-                if (i == 0) t0 = now;
-                else if (now - t0 > kWaitNs) { *s_flag = 1; break; }
-            }
-        }
-        xph ^= 1u << q;
-    };
-    const int ks_own = rank * (KC / 16);
-    // descriptors of k-step 0 of X buffer 0 and of A^T; a k-step is 256 bytes further (16 in
-    // the descriptor's address field), a buffer x_bytes
-    const uint64_t adesc0 = tc::smem_desc_noswizzle(sx_addr, 128, sbo);
-    const uint64_t bdesc0 = tc::smem_desc_noswizzle(sat_addr, 128, sbo);
-    const int nks = KC / 16;
-    for (uint32_t iter = 0;; ++iter) {
-        const int par = (int)(iter & 1u);
-        // ---- (A) this CTA's half of X_{t-1} is complete (buffer par^1): its MMAs start while
-        // the peer's half is still in flight
-        tc::fence_proxy_async_smem();
-        tc::tc_fence_before();
-        const bool any = __syncthreads_or(owner && seq != -1);
-        if (*s_flag != 0 || !any) {
-            if (*s_flag != 0 && tid == 0) report_status(status, ACCEL_ERR_TIMEOUT);
-            if (iter > 0) xchg_wait(par ^ 1);     // the peer's last stores have landed (bounded)
-            break;
-        }
-        const uint64_t xdesc = adesc0 + (uint64_t)((par ^ 1) * (L.x_bytes >> 4));
-        if (tid == kRows) {                       // a thread of column part 1: never a row owner
-            tc::tc_fence_after();
-            uint64_t ad = xdesc + (uint64_t)(ks_own * 16), bd = bdesc0 + (uint64_t)(ks_own * 16);
-            tc::mma_bf16(tmem, ad, bd, idesc, 0u);
-            for (int u = 1; u < nks; ++u) {
-                ad += 16;
-                bd += 16;
-                tc::mma_bf16(tmem, ad, bd, idesc, 1u);
-            }
-        }
-        // the peer's half of X_{t-1}, its row sums and (CTA 1) the indices it popped
-        if (iter > 0) xchg_wait(par ^ 1);
-        if (tid == kRows) {
-            tc::fence_proxy_async_smem();         // the peers' stores, seen through the barrier, to the tensor core
-#pragma unroll
-            for (int d = 1; d < NC; ++d) {
-                const int ks_peer = ((rank + d) % NC) * (KC / 16);
-                uint64_t ad = xdesc + (uint64_t)(ks_peer * 16), bd = bdesc0 + (uint64_t)(ks_peer * 16);
-                for (int u = 0; u < nks; ++u) {
-                    tc::mma_bf16(tmem, ad, bd, idesc, 1u);
-                    ad += 16;
-                    bd += 16;
-                }
-            }
-            tc::mma_commit(&bar[0]);
-        }
-        // ---- bookkeeping of the previous step's rows (both CTAs alike), overlapping the MMAs
-        if (owner && iter > 0) {
-            const int pp = par ^ 1;
-            if (seq == -2) {
-                const int32_t sq = mail[pp * MT + row];
-                if (sq >= 0) start(sq);
-                else idle(-1);
-            } else if (seq >= 0) {
-                float s = 0.f;                    // the same order in every CTA of the cluster
-#pragma unroll
-                for (int c = 0; c < NC; ++c)
-#pragma unroll
-                    for (int q = 0; q < NSPLIT; ++q) s += psum[((pp * NC + c) * NSPLIT + q) * MT + row];
-                if (pos == T - 1) {
-                    if (rank == 0) {
-                        loglik[seq] = 0.6931471805599453 * (double)E + log((double)s);
-                        int32_t sq = -1;
-                        if (!queue_empty) {
-                            const int64_t q = qbase + (int64_t)atomicAdd(next, 1ull);
-                            if (q >= S) queue_empty = true;
-                            else sq = order[q];
+                            for (int q = 1; q < cpp; ++q) c += ps[(p * cpp + q) * N];
+                            sum = p == 0 ? c : sum + c;
                         }
-                        mail[par * MT + row] = sq;
-                    }
-                    idle(-2);
-                } else {
-                    E += kcur;
-                    const float ls = __log2f(s);
-                    const float u = ls - (float)kcur;
-                    const float lr = pos == 0 ? ls : ls - uprev;
-                    uprev = u;
-                    kcur = (int)rintf(u + lr);
-                    ++pos;
-                    rinfo[row].ob = (int16_t)nob;
-                    rinfo[row].k = (int16_t)kcur;
-                    nob = pos + 1 < T ? o[pos + 1] : 0;
-                }
-            }
-        }
-        uint32_t rb[NC - 1];
-#pragma unroll
-        for (int d = 0; d < NC - 1; ++d) rb[d] = par ? rbar1[d] : rbar0[d];
-        if (rank == 0 && owner)
-#pragma unroll
-            for (int d = 0; d < NC - 1; ++d)
-                tc::st_async_u1(rmail[d] + 4u * (uint32_t)(par * MT + row), (uint32_t)mail[par * MT + row], rb[d]);
-        __syncthreads();
-        // ---- (B) epilogue of this CTA's columns into buffer par of both CTAs
-        const RowInfo ri = rinfo[row];
-        const bool fresh = ri.ob <= -2;
-        const bool act = ri.ob >= 0;
-        const int ob = fresh ? -ri.ob - 2 : ri.ob;
-        const float mult = ldexpf(1.0f, -(int)ri.k);
-        const uint32_t xo = (uint32_t)par * L.x_bytes;
-        float bs[16];
-        if (act || fresh) load_emis(ob, lt, bs, mult);
-        const bool ok = tc::mbar_wait_bounded(&bar[0], iter & 1u, kWaitNs);
-        if (!ok) *s_flag = 1;
-        tc::tc_fence_after();
-        float ps = 0.f;
-        if (__any_sync(0xffffffffu, act)) {
-            if (HL) {
-                if (CPT == 16) {
-                    uint32_t d[16];
-                    tc::tmem_ld16x2_16(taddr, d);
-                    if (act) ps = epi16(reinterpret_cast<const float*>(d), bs, lt, xo, rb);
-                } else {
-                    uint32_t d[32];
-                    tc::tmem_ld16x2_32(taddr, d);
-                    if (act) {
-                        ps = epi16(reinterpret_cast<const float*>(d), bs, lt, xo, rb);
-                        load_emis(ob, lt + 16, bs, mult);
-                        ps += epi16(reinterpret_cast<const float*>(d) + 16, bs, lt + 16, xo, rb);
-                    }
-                }
-            } else {
-                for (int jc = 0; jc < CPT; jc += 32) {
-                    uint32_t d[32];
-                    tc::tmem_ld32(taddr + jc, d);
-                    if (act) {
-                        if (jc > 0) load_emis(ob, lt + jc, bs, mult);
-                        ps += epi16(reinterpret_cast<const float*>(d), bs, lt + jc, xo, rb);
-                        load_emis(ob, lt + jc + 16, bs, mult);
-                        ps += epi16(reinterpret_cast<const float*>(d) + 16, bs, lt + jc + 16, xo, rb);
+                        sums[u] = sum;
                     }
                 }
             }
-            ps *= ldexpf(1.0f, (int)ri.k);
-        }
-        if (fresh) {
-            // alpha~_0 = pi o b(o_0) for this thread's columns
-            for (int jc = 0; jc < CPT; jc += 16) {
-                if (jc > 0) load_emis(ob, lt + jc, bs, 1.f);
-                float pv[16];
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&bar_info[pprev]);
+            if (ended1 && *s_fail == 0) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u) pv[u] = __expf(log_pi[gt + jc + u]);
-                ps += epi16(pv, bs, lt + jc, xo, rb);
+                for (int u = 0; u < NU; ++u)
+                    if (st1[u] & 4u)
+                        loglik[sq1[u]] = 0.6931471805599453 * (double)E1[u] + log(ldexp((double)sums[u], k1[u]));
+            }
+            if (stop) {
+                // done, out of time, or a wait gave up
+                if (lane == 0 && *s_fail != 0) report_status(status, ACCEL_ERR_TIMEOUT);
+                break;
+            }
+#pragma unroll
+            for (int u = 0; u < NU; ++u) {
+                st1[u] = st0[u];
+                sq1[u] = sq0[u];
+                E1[u] = E0[u];
+                k1[u] = k0[u];
+                E0[u] = (st[u] & 3u) == 1u ? E0[u] + k0[u] : 0;
+                k0[u] = kn[u];
+                st0[u] = st[u];
+                sq0[u] = seq[u];
+            }
+            ended1 = ended0;
+            ended0 = ended;
+        }
+        __syncwarp();
+    } else if (w > NEPI + NH) {
+        // ---- the max warps: lanes 16 g .. 16 g + 15 take columns 8 g .. 8 g + 7 of the warp's 16,
+        // every sixteenth state each
+        const int h = (w - NEPI - NH - 1) % NH, c0 = (w - NEPI - NH - 1) / NH * 16;
+        const int g = lane >> 4, kl = lane & 15;
+        const int ns = K - 128 * h < 128 ? K - 128 * h : 128;
+        const char* xr = sX + ((c0 >> 3) + g) * 16 * K + (128 * h + kl) * 16;
+        for (uint32_t iter = 0;; ++iter) {
+            const uint32_t par = iter & 1u;
+            if (!wait_step(&bar_info[par], (iter >> 1) & 1u, s_fail) || s_ctl[iter & 3u].done != 0) break;
+            wait_step(bar_x, par, s_fail);
+            const uint4* v = reinterpret_cast<const uint4*>(xr + par * L.x_bytes);
+            uint4 x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = 16 * i < ns ? v[16 * i] : make_uint4(0, 0, 0, 0);
+            uint32_t m[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                auto wd = [&](int i) { return r == 0 ? x[i].x : r == 1 ? x[i].y : r == 2 ? x[i].z : x[i].w; };
+                m[r] = max_bf16x2(max_bf16x2(max_bf16x2(wd(0), wd(1)), max_bf16x2(wd(2), wd(3))),
+                                  max_bf16x2(max_bf16x2(wd(4), wd(5)), max_bf16x2(wd(6), wd(7))));
+            }
+            // over the 16 lanes: two halving levels (4 -> 2 -> 1 words), then two full ones
+            const bool up1 = (kl & 8) != 0, up2 = (kl & 4) != 0;
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                m[r] = max_bf16x2(up1 ? m[r + 2] : m[r], __shfl_xor_sync(0xffffffffu, up1 ? m[r] : m[r + 2], 8));
+            m[0] = max_bf16x2(up2 ? m[1] : m[0], __shfl_xor_sync(0xffffffffu, up2 ? m[0] : m[1], 4));
+            m[0] = max_bf16x2(m[0], __shfl_xor_sync(0xffffffffu, m[0], 2));
+            m[0] = max_bf16x2(m[0], __shfl_xor_sync(0xffffffffu, m[0], 1));
+            if ((kl & 3) == 0)
+                *reinterpret_cast<uint32_t*>(s_mx + (par * MXP + h) * N + c0 + 8 * g + 2 * (kl >> 2)) = m[0];
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&bar_mx[par]);
+        }
+    } else {
+        // ---- the epilogue warps
+        const float pij = valid ? __expf(log_pi[j]) : 0.f;
+        const uint32_t lane_base = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(half * N + part * CPT);
+        char* const xw = sX + (j >> 3) * 128 + (j & 7) * 16;
+        const TE* const ej = sE + j;
+        for (uint32_t iter = 0;; ++iter) {
+            const uint32_t par = iter & 1u;
+            const Ctl& ctl = s_ctl[iter & 3u];
+            if (!wait_step(&bar_info[par], (iter >> 1) & 1u, s_fail) || ctl.done != 0) break;
+            bool ends = false;                    // some column of the tile ends a sequence
+#pragma unroll
+            for (int u = 0; u < NU; ++u) ends = ends || ctl.end[u] != 0;
+#pragma unroll
+            for (int ch = 0; ch < CPT / CH; ++ch) {
+                const int s0 = part * CPT + ch * CH;
+                // this step's emissions, scaled by 2^-k (exact), while the products run
+                float bs[CH];
+                uint32_t fm = 0;
+                if (valid) {
+                    fm = ctl.fresh[s0 >> 5] >> (s0 & 31);
+#pragma unroll
+                    for (int c = 0; c < CH; c += 4) {
+                        const int4 sy = *reinterpret_cast<const int4*>(s_sym + (iter & 3u) * N + s0 + c);
+                        const float4 sc = *reinterpret_cast<const float4*>(s_scale + par * N + s0 + c);
+                        float e0, e1, e2, e3;
+                        if constexpr (sizeof(TE) == 4) {
+                            e0 = ej[sy.x]; e1 = ej[sy.y]; e2 = ej[sy.z]; e3 = ej[sy.w];
+                        } else {
+                            e0 = __bfloat162float(ej[sy.x]); e1 = __bfloat162float(ej[sy.y]);
+                            e2 = __bfloat162float(ej[sy.z]); e3 = __bfloat162float(ej[sy.w]);
+                        }
+                        const float2 p0 = __fmul2_rn(make_float2(e0, e1), make_float2(sc.x, sc.y));
+                        const float2 p1 = __fmul2_rn(make_float2(e2, e3), make_float2(sc.z, sc.w));
+                        bs[c] = p0.x; bs[c + 1] = p0.y; bs[c + 2] = p1.x; bs[c + 3] = p1.y;
+                    }
+                }
+                if (ch == 0) {
+                    wait_step(&bar_mma[half], par, s_fail);
+                    tc::tc_fence_after();
+                }
+                if (valid) {
+                    float v[CH];
+                    tmem_ld_cols<CH>(lane_base + (uint32_t)(ch * CH), v);
+                    const uint32_t mask = CH == 32 ? 0xffffffffu : (1u << (CH & 31)) - 1u;
+                    if ((fm & mask) != 0) {
+                        // columns that start a sequence: alpha~_0 = pi o b(o_0)
+#pragma unroll
+                        for (int c = 0; c < CH; ++c) v[c] = (fm >> c) & 1u ? pij : v[c];
+                    }
+#pragma unroll
+                    for (int c = 0; c < CH; c += 2) {
+                        const float2 p = __fmul2_rn(make_float2(v[c], v[c + 1]), make_float2(bs[c], bs[c + 1]));
+                        v[c] = p.x;
+                        v[c + 1] = p.y;
+                    }
+                    uint32_t pk[CH / 2];
+#pragma unroll
+                    for (int c = 0; c < CH / 2; ++c) pk[c] = pack_bf16(v[2 * c], v[2 * c + 1]);
+#pragma unroll
+                    for (int c = 0; c < CH; c += 8)
+                        *reinterpret_cast<uint4*>(xw + par * L.x_bytes + ((s0 + c) >> 3) * 16 * K) =
+                            make_uint4(pk[c / 2], pk[c / 2 + 1], pk[c / 2 + 2], pk[c / 2 + 3]);
+                    if (ch == CPT / CH - 1) {
+                        tc::fence_proxy_async_smem();
+                        tc::tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) tc::mbar_arrive(bar_x);
+                    }
+                    if constexpr (NMX == 0) {
+                        int word;
+                        const uint32_t top = lane_max<CH / 2>(pk, lane, &word);
+                        if ((lane & (64 / CH - 1)) == 0)
+                            *reinterpret_cast<uint32_t*>(s_mx + (par * MXP + (j >> 5)) * N + s0 + 2 * word) = top;
+                    }
+                    if (ends) {
+                        int col;
+                        const float sum = lane_sums<CH>(v, lane, &col);
+                        if (CH == 32 || (lane & ~(CH - 1)) == 0) s_ps[(par * (K / 32) + (j >> 5)) * N + s0 + col] = sum;
+                    }
+                } else if (ch == CPT / CH - 1) {
+                    if (lane == 0) tc::mbar_arrive(bar_x);
+                }
+            }
+            if (NMX == 0 || ends) {
+                __syncwarp();
+                if (lane == 0) {
+                    if (NMX == 0) tc::mbar_arrive(&bar_mx[par]);
+                    if (ends) tc::mbar_arrive(&bar_ps[par]);
+                }
             }
         }
-        if (!act && !fresh) {
-            // no sequence on the row: zeros keep the peer's byte count fixed
-            for (int jc = 0; jc < CPT; jc += 8) {
-                const uint32_t co = xo + canon_off(row, gt + jc, K);
-                const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-                *reinterpret_cast<uint4*>(sX + co) = z;
-#pragma unroll
-                for (int d = 0; d < NC - 1; ++d) tc::st_async_u4(rx[d] + co, z, rb[d]);
-            }
-        }
-        if (HL) ps += __shfl_xor_sync(0xffffffffu, ps, 16);   // the row's two threads
-        if (hsel == 0) {
-            const int idx = ((par * NC + rank) * NSPLIT + part) * MT + row;
-            psum[idx] = ps;
-#pragma unroll
-            for (int d = 0; d < NC - 1; ++d) tc::st_async1(rpsum[d] + 4u * (uint32_t)idx, ps, rb[d]);
-        }
-        // the peer's bytes of this step complete the barrier's phase (waited for next step)
-        if (tid == 0) tc::mbar_arrive_expect_tx(&bar[1 + par], xbytes);
     }
     tc::tc_fence_before();
     __syncthreads();
-    if (w == 0) tc::tmem_dealloc(tmem, (uint32_t)KC);
-    cl.sync();                                    // the peer no longer addresses this CTA's shared memory
+    if (w == NEPI) tc::tmem_dealloc(tmem, tmem_cols);
 }
 
-// Clusters of nc CTAs of a cluster kernel that fit on the device at once (cached per kernel).
-template <typename Kern>
-static int pair_max_clusters(Kern kern, uint32_t smem, int threads, int nc) {
-    static std::mutex mu;
-    static std::map<std::pair<const void*, uint32_t>, int> cache;
-    const auto key = std::make_pair(reinterpret_cast<const void*>(kern), smem);
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = cache.find(key);
-    if (it != cache.end()) return it->second;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)nc;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)(num_sms() / nc * nc), 1, 1);
-    cfg.blockDim = dim3((unsigned)threads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        n = 0;
+using Kernel = void (*)(int, const float*, const float*, const float*, const int32_t*, const int64_t*, int64_t,
+                        const int32_t*, unsigned long long*, const int32_t*, double*, int32_t*, uint64_t, uint32_t);
+
+template <int K>
+Kernel kernel_k(int n, int esize) {
+    if constexpr (K <= 128)
+        if (esize == 2) return n == 16 ? k_hmm_tc<K, 16, __nv_bfloat16> : k_hmm_tc<K, 32, __nv_bfloat16>;
+    return n == 16 ? k_hmm_tc<K, 16, float> : n == 32 ? k_hmm_tc<K, 32, float>
+         : n == 64 ? k_hmm_tc<K, 64, float> : k_hmm_tc<K, 128, float>;
+}
+
+// A tile of n sequences: the size of a table entry, or 0 if no kernel takes it.  The BF16 table
+// is for the models whose FP32 table does not fit even beside 32 sequences (K <= 128, M > 400).
+int table_esize(int K, int M, int n) {
+    if ((int)tile_layout(K, M, n, 4).bytes <= max_smem_optin()) return 4;
+    return K <= 128 && n <= 32 && (int)tile_layout(K, M, n, 2).bytes <= max_smem_optin() ? 2 : 0;
+}
+
+// One of two tile sizes, picked on the device where the lengths are: *pick = lo or hi, the one with
+// the smaller estimated time.  A launch of tiles of N on g CTAs takes about
+//   t_N max(T_max, sum(T) / (N g) + 0.3 mean(T))
+// (the longest sequence, or the columns' load with part of a last sequence); t_hi / t_lo is
+// measured (GB300, us a step at N = 16 / 32 / 64: K = 256 0.49 / 0.76 / 1.27, K = 128 0.40 /
+// 0.51 / 0.87, K = 64 0.42 / 0.48 / 0.84).
+__global__ void __launch_bounds__(1024) k_pick_tile(const int64_t* __restrict__ off, int64_t S, int lo, int hi, int g,
+                                                    float ratio, int32_t* __restrict__ pick) {
+    __shared__ int64_t s_max[32];
+    int64_t m = 0;
+    for (int64_t s = threadIdx.x; s < S; s += blockDim.x) m = max(m, off[s + 1] - off[s]);
+    for (int d = 16; d > 0; d >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, d));
+    if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < 32; ++q) m = max(m, s_max[q]);
+        const float total = (float)(off[S] - off[0]), tail = 0.3f * total / (float)S;
+        const float t_lo = fmaxf((float)m, total / ((float)lo * g) + tail);
+        const float t_hi = fmaxf((float)m, total / ((float)hi * g) + tail) * ratio;
+        *pick = t_hi < t_lo ? hi : lo;
     }
-    cache[key] = n;
-    return n;
 }
 
-template <int NC>
-static accel_status tc_forward_cluster(const accel_hmm_model* mdl, const int32_t* obs, const int64_t* off, int64_t S,
-                                       double* loglik, char* ws, int32_t* d_status, TcConfig cfg, cudaStream_t st) {
-    const int K = mdl->K, M = mdl->M;
-    ACCEL_REQUIRE(tc_cl_supported(K, M, cfg.rows, cfg.split, NC), ACCEL_ERR_UNSUPPORTED,
-                  "hmm_forward(bf16, cluster of %d): unsupported configuration (K=%d, M=%d, split=%d, rows=%d)", NC, K,
-                  M, cfg.split, cfg.rows);
-    const int MT = cfg.rows <= 64 ? 64 : 128;
-    const PairLayout P = pair_layout(K, M, MT, cfg.split, NC);
-    TcLayout L = tc_layout(K, M, S);
-    char* at = ws + L.at_off;
-    char* et = ws + L.e_off;
-    int32_t* order = (int32_t*)(ws + L.order_off);
-    unsigned long long* next = (unsigned long long*)(ws + kQueueOff);
-    ACCEL_CUDA_TRY(cudaMemsetAsync(ws + kQueueOff, 0, 8, st));
-    int64_t nprep = (int64_t)K * K + (int64_t)K * M;
-    int pg = (int)((nprep + 255) / 256);
-    if (pg > 4 * num_sms()) pg = 4 * num_sms();
-    k_tc_prep<<<pg, 256, 0, st>>>(mdl->log_A, mdl->log_B, K, M, at, et);
-    accel_status r = order_by_length(off, S, order, ws + L.order_scratch_off, st);
-    if (r != ACCEL_OK) return r;
-    auto kern = cfg.split == 4 ? (MT == 64 ? k_hmm_tc_pair<4, 64, NC> : k_hmm_tc_pair<4, 128, NC>)
-                               : (MT == 64 ? k_hmm_tc_pair<2, 64, NC> : k_hmm_tc_pair<2, 128, NC>);
-    ACCEL_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.smem_bytes));
-    const int threads = 128 * cfg.split;
-    const int maxcl = pair_max_clusters(kern, P.smem_bytes, threads, NC);
-    ACCEL_REQUIRE(maxcl > 0, ACCEL_ERR_UNSUPPORTED, "hmm_forward(bf16): no cluster of %d CTAs fits the device", NC);
-    const int64_t tiles = (S + cfg.rows - 1) / cfg.rows;
-    int ncl = (int)(tiles < maxcl ? tiles : maxcl);
-    if (cfg.units > 0 && cfg.units < ncl) ncl = cfg.units;
-    cudaLaunchConfig_t lc = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)NC;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    lc.gridDim = dim3((unsigned)(NC * ncl), 1, 1);
-    lc.blockDim = dim3((unsigned)threads, 1, 1);
-    lc.dynamicSmemBytes = P.smem_bytes;
-    lc.stream = st;
-    lc.attrs = attr;
-    lc.numAttrs = 1;
-    ACCEL_CUDA_TRY(cudaLaunchKernelEx(&lc, kern, K, M, (const char*)at, (const char*)et, mdl->log_pi, obs, off, S,
-                                      (const int32_t*)order, next, cfg.rows, loglik, d_status, P));
-    return after_launch(st, NC == 2 ? "hmm_forward(bf16 tcgen05, cluster pair)" : "hmm_forward(bf16 tcgen05, cluster of 4)", 5);
+// the largest tile of at most n sequences that some kernel takes, or 0
+int tile_fit(int K, int M, int n) {
+    while (n >= 16 && table_esize(K, M, n) == 0) n >>= 1;
+    return n >= 16 ? n : 0;
+}
+
+accel_status launch_tiles(const accel_hmm_model* m, const int32_t* obs, const int64_t* off, int64_t S, int n, int grid,
+                          const int32_t* order, unsigned long long* next, const int32_t* pick, double* loglik,
+                          int32_t* d_status, cudaStream_t st) {
+    const int K = m->K, M = m->M;
+    const int es = table_esize(K, M, n), nh = (K + 127) / 128;
+    const TileLayout L = tile_layout(K, M, n, es);
+    const int need = nh * n + nh * (K / 2);                         // tensor memory: D, and A
+    uint32_t cols = 32;
+    while ((int)cols < need) cols <<= 1;
+    const Kernel kern = K == 64 ? kernel_k<64>(n, es) : K == 128 ? kernel_k<128>(n, es)
+                      : K == 192 ? kernel_k<192>(n, es) : kernel_k<256>(n, es);
+    ACCEL_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.bytes));
+    kern<<<grid, tile_threads(K, n), L.bytes, st>>>(M, m->log_A, m->log_B, m->log_pi, obs, off, S, order, next, pick,
+                                                    loglik, d_status, watchdog_ns(), cols);
+    return ACCEL_OK;
+}
+
+constexpr size_t kPickOff = 24;          // in the status block: the tile size picked on the device
+
+}  // namespace
+
+// The shapes taken: K a multiple of 64 whose transition matrix, emission table and a tile of 128
+// sequences fit shared memory together in BF16 (every such shape has a tile of 16 that fits).
+bool tc_supported(int K, int M) {
+    if (K < 64 || K > 256 || K % 64 != 0 || M < 1 || M > 32767) return false;
+    const size_t bytes = (size_t)K * K * 2 + (size_t)128 * K * 2 + (((size_t)M * K * 2 + 15) & ~(size_t)15) + 2576;
+    return bytes <= (size_t)max_smem_optin() && tile_fit(K, M, 16) != 0;
+}
+
+// workspace: the status block, the order by length and its scratch
+size_t tc_ws_bytes(int K, int M, int64_t S) {
+    (void)K; (void)M;
+    return align_up(kStatusBytes, 256) + order_ws_bytes(S);
+}
+
+// rows and split of a tile of n sequences: n = 2 rows / split
+TcConfig tile_config(int n) { return n >= 32 ? TcConfig{2, n, 0, 0} : TcConfig{4, 32, 0, 0}; }
+
+// The tile without a tuned configuration, by size alone: every sequence on a column of its own
+// where tiles of 16 allow it (the shortest step), else the larger size that k_pick_tile weighs.
+TcConfig default_config(int64_t S) {
+    const int64_t g = num_sms();
+    return tile_config(S <= 16 * g ? 16 : S <= 32 * g ? 32 : 64);
 }
 
 accel_status tc_forward_cfg(const accel_hmm_model* mdl, const int32_t* obs, const int64_t* off, int64_t S,
-                            double* loglik, char* ws, int32_t* d_status, TcConfig cfg, cudaStream_t st) {
+                            double* loglik, char* ws, int32_t* d_status, const TcConfig* cfg, cudaStream_t st) {
     const int K = mdl->K, M = mdl->M;
     ACCEL_REQUIRE(tc_supported(K, M), ACCEL_ERR_UNSUPPORTED,
                   "hmm_forward(bf16): K must be a multiple of 64 in [64, 256] and the tables must fit shared "
                   "memory (K=%d, M=%d)", K, M);
-    if (cfg.split == 4 && (K / 4) % 32 != 0) cfg.split = 2;
-    if (cfg.rows < 32 || cfg.rows > kRows) cfg.rows = kRows;
-    if (cfg.pair == 2 && !tc_cl_supported(K, M, cfg.rows, cfg.split, 4)) cfg.pair = 1;
-    if (cfg.pair == 2) return tc_forward_cluster<4>(mdl, obs, off, S, loglik, ws, d_status, cfg, st);
-    if (cfg.pair == 1) {
-        if (tc_cl_supported(K, M, cfg.rows, cfg.split, 2))
-            return tc_forward_cluster<2>(mdl, obs, off, S, loglik, ws, d_status, cfg, st);
-        cfg.pair = 0;
-    }
-    TcLayout L = tc_layout(K, M, S);
-    char* at = ws + L.at_off;
-    char* et = ws + L.e_off;
-    int32_t* order = (int32_t*)(ws + L.order_off);
-    unsigned long long* next = (unsigned long long*)(ws + kQueueOff);   // inside the status block
-    ACCEL_CUDA_TRY(cudaMemsetAsync(ws + kQueueOff, 0, 8, st));
-    int64_t nprep = (int64_t)K * K + (int64_t)K * M;
-    int pg = (int)((nprep + 255) / 256);
-    if (pg > 4 * num_sms()) pg = 4 * num_sms();
-    k_tc_prep<<<pg, 256, 0, st>>>(mdl->log_A, mdl->log_B, K, M, at, et);
-    accel_status r = order_by_length(off, S, order, ws + L.order_scratch_off, st);
-    if (r != ACCEL_OK) return r;
-    int64_t tiles = (S + cfg.rows - 1) / cfg.rows;
+    const TcConfig c = cfg ? *cfg : default_config(S);
+    const int rows = c.rows < 32 || c.rows > 128 ? 128 : c.rows;
+    const int n = tile_fit(K, M, c.split == 4 ? rows / 2 : rows);
+    int lo = n;
+    if (!cfg && n > 16) lo = n / 2;                                  // weighed on the device
+    const int64_t tiles = (S + lo - 1) / lo;
     int grid = (int)(tiles < num_sms() ? tiles : num_sms());
-    if (cfg.units > 0 && cfg.units < grid) grid = cfg.units;
-    // rows <= 64 per CTA: M = 64 tiles
-    auto kern = cfg.split == 4 ? (cfg.rows <= 64 ? k_hmm_tc<4, 64> : k_hmm_tc<4, 128>)
-                               : (cfg.rows <= 64 ? k_hmm_tc<2, 64> : k_hmm_tc<2, 128>);
-    ACCEL_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem_bytes));
-    kern<<<grid, 128 * cfg.split, L.smem_bytes, st>>>(K, M, at, et, mdl->log_pi, obs, off, S, order, next, cfg.rows,
-                                                      loglik, d_status, watchdog_ns(), L);
-    return after_launch(st, "hmm_forward(bf16 tcgen05)", 5);
+    if (c.units > 0 && c.units < grid) grid = c.units;
+    // every sequence on a column of its own from the start needs neither an order nor a queue
+    int32_t* order = nullptr;
+    unsigned long long* next = nullptr;
+    int nk = 1;
+    if (S > (int64_t)lo * grid) {
+        next = (unsigned long long*)(ws + kQueueOff);               // inside the status block
+        order = (int32_t*)(ws + align_up(kStatusBytes, 256));
+        ACCEL_CUDA_TRY(cudaMemsetAsync(next, 0, 8, st));
+        accel_status r = order_by_length(off, S, order, (char*)order + align_up((size_t)S * 4, 256), st);
+        if (r != ACCEL_OK) return r;
+        nk += 3;
+    }
+    int32_t* pick = nullptr;
+    if (lo != n) {
+        pick = (int32_t*)(ws + kPickOff);
+        const float ratio = n > 32 ? 1.7f : K > 128 ? 1.54f : 1.25f;
+        k_pick_tile<<<1, 1024, 0, st>>>(off, S, lo, n, grid, ratio, pick);
+        accel_status r = launch_tiles(mdl, obs, off, S, lo, grid, order, next, pick, loglik, d_status, st);
+        if (r != ACCEL_OK) return r;
+        nk += 2;
+    }
+    accel_status r = launch_tiles(mdl, obs, off, S, n, grid, order, next, pick, loglik, d_status, st);
+    if (r != ACCEL_OK) return r;
+    return after_launch(st, "hmm_forward(bf16 tcgen05)", nk);
 }
 
 accel_status tc_forward(const accel_hmm_model* mdl, const int32_t* obs, const int64_t* off, int64_t S,
                         double* loglik, char* ws, int32_t* d_status, cudaStream_t st) {
-    return tc_forward_cfg(mdl, obs, off, S, loglik, ws, d_status, tuned_config(mdl->K, mdl->M, S), st);
+    TcConfig c;
+    return tc_forward_cfg(mdl, obs, off, S, loglik, ws, d_status, tuned_entry(mdl->K, mdl->M, S, &c) ? &c : nullptr, st);
 }
 
 }  // namespace hmm
