@@ -160,11 +160,11 @@ uint64_t accel_get_watchdog_ns(void);
 
 /*
  * accel_set_sm_budget -- the most SMs the forward recursion of hmm_adjoint /
- * hmm_adjoint_forward may occupy (its persistent CTA-pair launch, K in {64, 128, 256} with
- * planned groups), so that it can run beside another stream's persistent kernel instead of
- * waiting for the whole GPU: the launch takes min(n, #SMs) / 2 pairs, but at least enough to
- * hold every sequence in two groups of 16.  0 (the default) means every SM.  The backward
- * rounds always use every SM.  Results do not depend on it (each sequence's forward
+ * hmm_adjoint_forward may occupy (its persistent launch), so that it can run beside another
+ * stream's persistent kernel instead of waiting for the whole GPU: the launch takes the share
+ * of its CTAs that n SMs hold, but at least one (in the checkpointed form, enough pairs to hold
+ * every sequence in two groups of 16).  0 (the default) means every SM.  The backward pass always
+ * uses every SM.  Results do not depend on it (each sequence's forward
  * arithmetic is the same in any group).  Per host thread; read when a call is issued.
  */
 void accel_set_sm_budget(int32_t n_sms);
@@ -371,9 +371,12 @@ accel_status hmm_forward(const accel_hmm_model* m, int32_t precision, const int3
  *   d_grad_log_A[i*K+j]  = sum_s w_s sum_{t<T_s} P(z_t=i, z_{t+1}=j | o^s)  (expected transitions)
  *   d_grad_log_B[j*M+k]  = sum_s w_s sum_t P(z_t=j | o^s) [o^s_t = k]      (expected emissions)
  *   d_grad_log_pi[j]     = sum_s w_s P(z_1=j | o^s)
- * computed by a hand-written adjoint of the scaled forward recursion: a forward pass that
- * keeps alpha only every ceil(sqrt(T_s)) steps, then, segment by segment in reverse, a
- * recomputation of alpha from its checkpoint and the backward (beta) recursion.
+ * computed by a hand-written adjoint of the scaled forward recursion.  With a workspace of
+ * hmm_adjoint_workspace_size bytes every alpha is kept (three float32 rows of the padded state
+ * count per time step, up to 32 GiB in all) and the backward pass recomputes nothing.  With less,
+ * down to hmm_adjoint_min_workspace_size bytes, or for more rows than that, the forward keeps
+ * alpha only every ceil(sqrt(T_s)) steps, and the backward recomputes it segment by segment in
+ * reverse.  Both forms give the same results up to FP32 rounding.
  *  d_weights  device float64 [S] or NULL (all ones).
  *  d_loglik   device float64 [S] or NULL: the forward's logL_s.
  *  max_T      the largest sequence length (sizes the checkpoint storage; hmm_max_length
@@ -382,13 +385,14 @@ accel_status hmm_forward(const accel_hmm_model* m, int32_t precision, const int3
  *             else recorded in the device status word (accel_set_device_status).
  *  Outputs are overwritten (not accumulated); d_grad_log_pi may be NULL.
  *  Streams: the work is ordered after what `stream` already holds, and what `stream` enqueues
- *  next runs after it.  On K = 64, 128 or 256 the backward part runs on three streams the
- *  library creates once per host thread and device (the backward and recomputation passes at
- *  the highest stream priority, the count kernels at the lowest).  It forks from `stream`
+ *  next runs after it.  The checkpointed form on K = 64, 128 or 256 runs its backward part on three
+ *  streams the library creates once per host thread and device (the backward and recomputation
+ *  passes at the highest stream priority, the count kernels at the lowest).  It forks from `stream`
  *  and joins it again through events, so a capture of `stream` into a CUDA graph takes the
  *  whole call.  Two host threads calling at once each use their own streams.
  */
 size_t hmm_adjoint_workspace_size(const accel_hmm_model* m, int64_t S, int64_t total_T, int64_t max_T);
+size_t hmm_adjoint_min_workspace_size(const accel_hmm_model* m, int64_t S, int64_t total_T, int64_t max_T);
 accel_status hmm_adjoint(const accel_hmm_model* m, const int32_t* d_obs, const int64_t* d_offsets,
                          int64_t S, int64_t total_T, int64_t max_T, const double* d_weights,
                          double* d_loglik, float* d_grad_log_A, float* d_grad_log_B,
@@ -397,8 +401,8 @@ accel_status hmm_adjoint(const accel_hmm_model* m, const int32_t* d_obs, const i
 /*
  * hmm_adjoint_forward / hmm_adjoint_backward -- hmm_adjoint in two calls, for a forward pass
  * whose gradient is taken later (e.g. an autograd function): the forward writes logL_s
- * (d_loglik, may be NULL) and leaves its saved state -- the ceil(sqrt(T_s)) checkpoints of
- * alpha, their exponents, the sequence order and grouping -- in d_ws; the backward then runs
+ * (d_loglik, may be NULL) and leaves its saved state -- every alpha, or the ceil(sqrt(T_s))
+ * checkpoints of it, the exponents, the sequence order and grouping -- in d_ws; the backward then runs
  * the recomputation and the backward recursion from that state and writes the gradients as
  * hmm_adjoint does.  Both calls take the same model, observations, offsets, sizes and
  * workspace (hmm_adjoint_workspace_size bytes), and the model's log parameters must not change

@@ -323,6 +323,15 @@ def hmm_forward(log_A, log_B, log_pi, obs, offsets, precision=L.HMM_FP32_LOG, to
     return out
 
 
+def _adjoint_ws(lib, m, S, total_T, max_T, device):
+    """The adjoint's workspace: with every alpha kept, or the smaller one of the checkpointed form
+    where that much memory is not to be had."""
+    try:
+        return _ws(lib.hmm_adjoint_workspace_size(C.byref(m), S, total_T, max_T), device)
+    except torch.OutOfMemoryError:
+        return _ws(lib.hmm_adjoint_min_workspace_size(C.byref(m), S, total_T, max_T), device)
+
+
 def hmm_adjoint(log_A, log_B, log_pi, obs, offsets, weights=None, max_T: int | None = None, want_loglik=True,
                 ws=None):
     """Gradients of sum_s w_s logL_s w.r.t. (log_A, log_B, log_pi) (float32) and logL
@@ -338,9 +347,8 @@ def hmm_adjoint(log_A, log_B, log_pi, obs, offsets, weights=None, max_T: int | N
     gB = torch.empty(K, M, dtype=torch.float32, device=obs.device)
     gpi = torch.empty(K, dtype=torch.float32, device=obs.device)
     ll = torch.empty(S, dtype=torch.float64, device=obs.device) if want_loglik else None
-    need = lib.hmm_adjoint_workspace_size(C.byref(m), S, obs.numel(), max_T)
-    if ws is None or ws.numel() < need:
-        ws = _ws(need, obs.device)
+    if ws is None or ws.numel() < lib.hmm_adjoint_min_workspace_size(C.byref(m), S, obs.numel(), max_T):
+        ws = _adjoint_ws(lib, m, S, obs.numel(), max_T, obs.device)
     if weights is not None and weights.dtype != torch.float64:
         weights = weights.to(torch.float64)
     L.check("hmm_adjoint", lib.hmm_adjoint(C.byref(m), _ptr(obs), _ptr(offsets), S, obs.numel(), max_T,
@@ -351,7 +359,7 @@ def hmm_adjoint(log_A, log_B, log_pi, obs, offsets, weights=None, max_T: int | N
 
 class AdjointSaved:
     """The state hmm_adjoint_forward leaves for hmm_adjoint_backward: the workspace (with the
-    checkpoints of alpha) and the sizes it was made for."""
+    alphas or their checkpoints) and the sizes it was made for."""
 
     def __init__(self, ws, S, total_T, max_T):
         self.ws, self.S, self.total_T, self.max_T = ws, S, total_T, max_T
@@ -367,7 +375,7 @@ def hmm_adjoint_forward(log_A, log_B, log_pi, obs, offsets, max_T: int | None = 
     if max_T is None:
         max_T = int(hmm_max_length(offsets).item()) if S else 0
     ll = torch.empty(S, dtype=torch.float64, device=obs.device) if out is None else out
-    ws = _ws(lib.hmm_adjoint_workspace_size(C.byref(m), S, obs.numel(), max_T), obs.device)
+    ws = _adjoint_ws(lib, m, S, obs.numel(), max_T, obs.device)
     L.check("hmm_adjoint_forward", lib.hmm_adjoint_forward(C.byref(m), _ptr(obs), _ptr(offsets), S, obs.numel(), max_T,
                                                            _ptr(ll), _ptr(ws), ws.numel(), _stream()))
     return ll, AdjointSaved(ws, S, obs.numel(), max_T)

@@ -1,5 +1,5 @@
-// Hand-written adjoint of the scaled HMM forward recursion (K9), with sqrt(T)
-// checkpointing.
+// Hand-written adjoint of the scaled HMM forward recursion (K9): the entry points, and the form with
+// sqrt(T) checkpointing (hmm_adj_rows.cu keeps every alpha instead, where memory allows it).
 //
 // Gradients of L = sum_s w_s logL_s with respect to log A, log B, log pi taken as free
 // parameters are the (weighted) forward-backward expected counts.  The HMM is not in the
@@ -31,6 +31,7 @@
 // path the backward of round r, the recomputation of round r + 1 and the counts of earlier
 // rounds run at the same time on three streams, each round's rows in buffers of its own.
 // Every accumulation has a fixed order, so results are deterministic.
+#include "hmm_adj_rows.cuh"
 #include "hmm_internal.cuh"
 #include "simt_stream.cuh"
 
@@ -1873,9 +1874,15 @@ accel_status check_model(const accel_hmm_model* m, const char* who);
 extern "C" {
 
 size_t hmm_adjoint_workspace_size(const accel_hmm_model* m, int64_t S, int64_t total_T, int64_t max_T) {
-    (void)total_T;
     if (!m || S < 0) return 0;
-    return adj::layout(m->K, m->M, S, max_T).total;
+    const size_t rows = rows::rows_ws_bytes(m->K, m->M, S, total_T);
+    return rows > 0 ? rows : adj::layout(m->K, m->M, S, max_T).total;
+}
+
+size_t hmm_adjoint_min_workspace_size(const accel_hmm_model* m, int64_t S, int64_t total_T, int64_t max_T) {
+    if (!m || S < 0) return 0;
+    const size_t rows = rows::rows_ws_bytes(m->K, m->M, S, total_T), cp = adj::layout(m->K, m->M, S, max_T).total;
+    return rows > 0 && rows < cp ? rows : cp;
 }
 
 }  // extern "C"
@@ -1891,6 +1898,8 @@ struct Plan {
     int K, M, nb, nsU, nsC;
     size_t sm_b, sm_c;
     bool use_cluster, xi_tc, counts_tc, planned;
+    bool use_rows;              // every alpha kept (hmm_adj_rows.cu), with these arguments
+    rows::RowsArgs ra;
     float* cntp;
     float* Upart;
     char* ws;
@@ -1908,7 +1917,12 @@ static accel_status setup(const char* who, const accel_hmm_model* m, const int32
     P.M = M;
     P.L = layout(K, M, S, max_T);
     const Layout& L = P.L;
-    ACCEL_REQUIRE(ws_bytes >= L.total, ACCEL_ERR_WORKSPACE, "%s: workspace %zu < %zu bytes", who, ws_bytes, L.total);
+    // every alpha is kept where the sizes allow it and the workspace holds them; a workspace of
+    // hmm_adjoint_min_workspace_size bytes takes the checkpoints instead
+    const size_t rows_bytes = rows::rows_ws_bytes(K, M, S, total_T);
+    P.use_rows = rows_bytes > 0 && ws_bytes >= rows_bytes;
+    ACCEL_REQUIRE(P.use_rows || ws_bytes >= L.total, ACCEL_ERR_WORKSPACE, "%s: workspace %zu < %zu bytes", who, ws_bytes,
+                  L.total);
     ACCEL_REQUIRE(S * (int64_t)L.Cmax <= (int64_t)INT32_MAX, ACCEL_ERR_UNSUPPORTED,
                   "%s: S x ceil(sqrt(max_T)) = %lld rows exceeds 2^31-1", who, (long long)(S * (int64_t)L.Cmax));
     P.sm_b = smem_bwd(K, M, L.Cmax);
@@ -1951,6 +1965,8 @@ static accel_status setup(const char* who, const accel_hmm_model* m, const int32
     // the streaming kernels hold the whole emission table in shared memory
     ACCEL_REQUIRE(P.use_cluster || S == 0 || P.sm_b <= (size_t)max_smem_optin(), ACCEL_ERR_UNSUPPORTED,
                   "%s: emission table too large for shared memory (K=%d, M=%d)", who, K, M);
+    P.ra = rows::RowsArgs{m, d_obs, d_offsets, S, total_T, L.Cmax, d_ws, p.status};
+    if (P.use_rows) return ACCEL_OK;
     P.xi_tc = P.use_cluster && xi_tc_supported(K);
     P.counts_tc = P.xi_tc && xi_tc_counts_supported(K, M);
     P.nsU = P.xi_tc ? xi_tc_partials(K, M, P.counts_tc) : kSplit;
@@ -1986,6 +2002,7 @@ static accel_status setup(const char* who, const accel_hmm_model* m, const int32
 // Phase 1: parameters prepared, sequences ordered and (cluster path) grouped, the forward pass
 // with its checkpoints and logL.  Everything phase 2 reads stays in the workspace.
 static accel_status run_forward(Plan& P, const accel_hmm_model* m, double* d_loglik, cudaStream_t st, int& nlaunch) {
+    if (P.use_rows) return rows::rows_forward(P.ra, d_loglik, st, nlaunch);
     Prm& p = P.p;
     const Layout& L = P.L;
     const int K = P.K, M = P.M;
@@ -2068,6 +2085,7 @@ struct EventSet {
 // the gradients.  Reads phase 1's checkpoints, order and plan; clears its own accumulators.
 static accel_status run_backward(Plan& P, const double* d_weights, float* d_grad_log_A, float* d_grad_log_B,
                                  float* d_grad_log_pi, cudaStream_t st, int& nlaunch) {
+    if (P.use_rows) return rows::rows_backward(P.ra, d_weights, d_grad_log_A, d_grad_log_B, d_grad_log_pi, st, nlaunch);
     Prm& p = P.p;
     const Layout& L = P.L;
     const int K = P.K, M = P.M;
