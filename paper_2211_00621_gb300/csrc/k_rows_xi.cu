@@ -10,12 +10,16 @@
 // are added, rounded to nearest, to sums in registers: 8 truncations, about 3e-7.
 //
 // Pipeline: 512 splitter threads, one piece of a 16-row chunk each (eight rows of one column, loaded
-// one chunk ahead straight from global memory), write the three parts into a stage (no-swizzle
+// two chunks ahead straight from global memory), write the three parts into a stage (no-swizzle
 // K-major canonical layout, 16-byte stores); the stage's mbarrier counts them; one warp issues the
 // chunk's six MMAs under elect.sync (in a divergent branch each costs about 100 cycles) and commits
 // them to the stage's second mbarrier, which the splitters wait on before they refill it.  The
 // accumulators are double-buffered in tensor memory (all 512 columns), so the splitters take a
 // block's sums while the next block's products run.  Every wait is bounded.
+//
+// What bounds it: the splitters' instructions (about 650 issue slots a chunk and scheduler); DRAM and
+// the tensor cores are at a third.  1.13M rows at K = 256: 1.13 ms (2.3 GB of operands, 0.34 ms at the
+// copy rate).  One chunk in flight and an arrival per thread and stage: 1.50 ms.
 #include "hmm_adj_rows.cuh"
 #include "tc_ptx.cuh"
 
@@ -33,7 +37,7 @@ constexpr int kKC = 16;                         // rows per chunk (one MMA's red
 constexpr int kBlock = 128;                     // rows between flushes
 constexpr int kChunks = kBlock / kKC;
 constexpr int kStages = 4;
-constexpr int kPrefetch = 8;                    // chunks brought into L2 ahead
+constexpr int kPrefetch = 12;                   // chunks brought into L2 ahead
 constexpr uint64_t kWait = 2000000000ull;
 
 // Canonical K-major offset of the 16 bytes (n, k = 8 kq .. + 7) of a [rows][kKC] BF16 block: core
@@ -66,6 +70,9 @@ constexpr uint32_t part_bytes(int K) { return 2u * tile(K) * kKC * 2; }       //
 constexpr uint32_t stage_bytes(int K) { return 3 * part_bytes(K); }
 constexpr uint32_t smem_bytes(int K) { return kStages * stage_bytes(K); }
 
+// (with the bounded loop out of line behind a first poll: 1.23 ms, 1.13 so)
+__device__ __forceinline__ bool wait(uint64_t* bar, uint32_t parity) { return tc::mbar_wait_bounded(bar, parity, kWait); }
+
 template <int K>
 __global__ void __launch_bounds__(kThreads, 1) k_rows_xi(const float* __restrict__ X, const float* __restrict__ Q,
                                                          const int32_t* __restrict__ d_rows, int nsplit,
@@ -87,10 +94,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_rows_xi(const float* __restrict
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             tc::mbar_init(&s_bar[s], 1);
-            tc::mbar_init(&s_full[s], kSplitThreads);
+            tc::mbar_init(&s_full[s], kSplitThreads / 32);
         }
-        tc::mbar_init(&s_read[0], kSplitThreads);
-        tc::mbar_init(&s_read[1], kSplitThreads);
+        tc::mbar_init(&s_read[0], kSplitThreads / 32);
+        tc::mbar_init(&s_read[1], kSplitThreads / 32);
         tc::fence_mbar_init();
         s_fail = 0;
     }
@@ -102,26 +109,29 @@ __global__ void __launch_bounds__(kThreads, 1) k_rows_xi(const float* __restrict
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = s_tmem;
-    const int64_t nchunks = r1 > r0 ? (r1 - r0 + kKC - 1) / kKC : 0;
+    const int nchunks = r1 > r0 ? (int)((r1 - r0 + kKC - 1) / kKC) : 0;
+    // chunk c's products have completed (its stage is c mod kStages)
+    auto done = [&](int c) {
+        return wait(&s_bar[c % kStages], (uint32_t)(c / kStages) & 1u);
+    };
     if (warp == kSplitThreads / 32) {
         // ---- the issuing warp
         constexpr uint32_t id = tc::idesc_bf16_f32(TN, TN);
-        int64_t issued = 0;
-        for (int64_t q = 0; q < nchunks; ++q) {
-            const int s = (int)(q % kStages);
-            const int64_t blk = q / kChunks;
+        constexpr uint64_t P = part_bytes(K) >> 4;
+        const uint64_t desc0 = tc::smem_desc_noswizzle(tc::smem_u32(smem), 128, 256);
+        int issued = 0;
+        for (int q = 0; q < nchunks; ++q) {
+            const int s = q % kStages, blk = q / kChunks;
             const bool first = q % kChunks == 0;
-            bool ok = tc::mbar_wait_bounded(&s_full[s], (uint32_t)((q / kStages) & 1), kWait);
+            bool ok = wait(&s_full[s], (uint32_t)(q / kStages) & 1u);
             // the pair's last block has been taken
-            if (first && blk >= 2) ok = tc::mbar_wait_bounded(&s_read[blk & 1], (uint32_t)((blk / 2 - 1) & 1), kWait) && ok;
-            if (!__all_sync(0xffffffffu, ok) || s_fail != 0) {
+            if (first && blk >= 2) ok = wait(&s_read[blk & 1], (uint32_t)(blk / 2 - 1) & 1u) && ok;
+            if (!ok || s_fail != 0) {
                 s_fail = 1;
                 break;
             }
             tc::tc_fence_after();
-            const uint64_t a = tc::smem_desc_noswizzle(tc::smem_u32(smem) + (uint32_t)s * stage_bytes(K), 128, 256);
-            const uint64_t b = a + (kQOff >> 4);
-            constexpr uint64_t P = part_bytes(K) >> 4;
+            const uint64_t a = desc0 + (uint64_t)(s * (stage_bytes(K) >> 4)), b = a + (kQOff >> 4);
             const uint32_t d = tmem + (uint32_t)(blk & 1) * kBuf, acc = first ? 0u : 1u;
             if (tc::elect_one()) {
                 tc::mma_bf16(d, a, b, id, acc);                          // hi hi
@@ -136,7 +146,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rows_xi(const float* __restrict
             issued = q + 1;
         }
         // the MMAs issued last complete before the tensor memory goes
-        if (issued > 0) tc::mbar_wait_bounded(&s_bar[(issued - 1) % kStages], (uint32_t)(((issued - 1) / kStages) & 1), kWait);
+        if (issued > 0) done(issued - 1);
     } else {
         // ---- the splitters: columns 0 .. TN - 1 are X's, TN .. 2 TN - 1 Q's, two row octets each
         const int col = tid % (2 * TN), kq = tid / (2 * TN);
@@ -146,14 +156,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_rows_xi(const float* __restrict
         const int qd = warp & 3, part = warp >> 2;                        // the thread's part of D
         const bool sums = 32 * part < TN;
         const uint32_t at = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(32 * part);
-        auto load = [&](float (&v)[8], int64_t q) {
-            const int64_t left = r1 - r0 - q * kKC - 8 * kq;              // rows from the piece's first
-            const float* p = src + q * kKC * K;
+        auto load = [&](float (&v)[8], int q) {
+            if (q >= nchunks || !mine) return;
+            const float* p = src + (int64_t)q * (kKC * K);
+            if (q + 1 < nchunks) {                                        // a whole chunk
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = mine && i < left ? __ldcg(p + i * K) : 0.f;
+                for (int i = 0; i < 8; ++i) v[i] = __ldcg(p + i * K);
+            } else {
+                const int left = (int)(r1 - r0) - q * kKC - 8 * kq;       // rows from the piece's first
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = i < left ? __ldcg(p + i * K) : 0.f;
+            }
         };
-        auto prefetch = [&](int64_t q) {
-            const int64_t row0 = r0 + q * kKC;
+        auto prefetch = [&](int q) {
+            if (q >= nchunks) return;
+            const int64_t row0 = r0 + (int64_t)q * kKC;
             const uint32_t bytes = (uint32_t)(r1 - row0 < kKC ? r1 - row0 : kKC) * K * 4;
             tc::bulk_prefetch_l2(Q + row0 * K, bytes);
             tc::bulk_prefetch_l2(X + row0 * K, bytes);
@@ -162,7 +179,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rows_xi(const float* __restrict
 #pragma unroll
         for (int e = 0; e < 32; ++e) acc[e] = 0.f;
         // take the sums of block blk, whose products have completed
-        auto flush = [&](int64_t blk) {
+        auto flush = [&](int blk) {
             tc::tc_fence_after();
             if (sums) {
                 uint32_t v[32];
@@ -174,40 +191,43 @@ __global__ void __launch_bounds__(kThreads, 1) k_rows_xi(const float* __restrict
                 for (int e = 0; e < 32; ++e) acc[e] += __uint_as_float(v[e]);
             }
             tc::tc_fence_before();
-            tc::mbar_arrive(&s_read[blk & 1]);
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&s_read[blk & 1]);
         };
-        auto done = [&](int64_t c) {                                      // chunk c's products have completed
-            return tc::mbar_wait_bounded(&s_bar[c % kStages], (uint32_t)((c / kStages) & 1), kWait);
-        };
-        if (tid == 0)
-            for (int64_t q = 0; q < kPrefetch && q < nchunks; ++q) prefetch(q);
-        float cur[8], nxt[8];
-        if (nchunks > 0) load(cur, 0);
-        bool ok = true;
-        for (int64_t c = 0; c < nchunks; ++c) {
-            const int s = (int)(c % kStages);
-            char* st = smem + (size_t)s * stage_bytes(K) + dst;
-            if (tid == 0 && c + kPrefetch < nchunks) prefetch(c + kPrefetch);
-            if (c + 1 < nchunks) load(nxt, c + 1);
+        // write chunk c from v and load chunk c + 2 into it; false: a wait gave up
+        auto step = [&](float (&v)[8], int c) -> bool {
+            const int s = c % kStages;
+            char* st = smem + s * stage_bytes(K) + dst;
+            if (tid == 0) prefetch(c + kPrefetch);
             // the stage's previous MMAs (chunk c - kStages) have completed
-            if (c >= kStages) ok = done(c - kStages);
-            if (!ok || s_fail != 0) break;
+            if (c >= kStages && !done(c - kStages)) return false;
             if (mine) {
-                *reinterpret_cast<uint4*>(st) = take_part(cur);
-                *reinterpret_cast<uint4*>(st + part_bytes(K)) = take_part(cur);
-                *reinterpret_cast<uint4*>(st + 2 * part_bytes(K)) = take_part(cur);
+                *reinterpret_cast<uint4*>(st) = take_part(v);
+                *reinterpret_cast<uint4*>(st + part_bytes(K)) = take_part(v);
+                *reinterpret_cast<uint4*>(st + 2 * part_bytes(K)) = take_part(v);
             }
+            load(v, c + 2);
             tc::fence_proxy_async_smem();
-            tc::mbar_arrive(&s_full[s]);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) cur[i] = nxt[i];
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&s_full[s]);
             // a block's sums, when the wait above was for its last chunk
             if (c >= kChunks && c % kChunks == kStages - 1) flush(c / kChunks - 1);
+            return s_fail == 0;
+        };
+        if (tid == 0)
+            for (int q = 0; q < kPrefetch; ++q) prefetch(q);
+        float v0[8], v1[8];
+        load(v0, 0);
+        load(v1, 1);
+        bool ok = true;
+        for (int c = 0; c < nchunks && ok; c += 2) {
+            ok = step(v0, c);
+            if (ok && c + 1 < nchunks) ok = step(v1, c + 1);
         }
-        if (ok && s_fail == 0) {
+        if (ok) {
             // the blocks not taken yet: the last one, and the one before it if it ended less than a
             // stage's depth before the end
-            const int64_t lastb = nchunks > 0 ? (nchunks - 1) / kChunks : 0;
+            const int lastb = nchunks > 0 ? (nchunks - 1) / kChunks : 0;
             if (lastb >= 1 && (nchunks - 1) % kChunks < kStages - 1 && (ok = done(lastb * kChunks - 1))) flush(lastb - 1);
             if (nchunks > 0 && ok && (ok = done(nchunks - 1))) flush(lastb);
             // row r of the tile: lane r (TN = 128) or lane 32 (r / 16) + r % 16 (TN = 64)
