@@ -15,8 +15,6 @@
 #include "hmm_rows.cuh"
 
 #include <algorithm>
-#include <map>
-#include <mutex>
 
 namespace accel {
 namespace hmm {
@@ -92,6 +90,7 @@ __device__ __forceinline__ void fwd_epilogue(const RowsPrm& p, int rank, int cid
                                              Waits& wt) {
     using C = Cfg<KP>;
     Epilogue<KP> ep(sm, rank);
+    const int u = ep.u;
     const int64_t n = (int64_t)p.ncl * kG;
     const int Cmax = p.Cmax;
     const int32_t* obs = p.obs + p.off[0];       // rows and symbols count from the first sequence
@@ -104,94 +103,87 @@ __device__ __forceinline__ void fwd_epilogue(const RowsPrm& p, int rank, int cid
     };
     Vec<C::EC> pi;
     pi.load(p.pi + c);
-    // the warp's two slots: the sequence, the step to compute (row, steps left after it), its symbol and
+    // the warp's slot: the sequence, the step to compute (row, steps left after it), its symbol and
     // the one after
-    Slot s[2];
-    int32_t row[2], left[2], sym[2], nsym[2];
-    bool fresh[2];
+    Slot s;
+    int32_t row, left, sym, nsym;
+    bool fresh;
     // the step computed last: whether there was one, whether it ended its sequence, the CTA's sum of it
-    int32_t pseq[2];
-    bool pon[2], plast[2];
-    float psum[2];
-    int64_t E[2];
-    auto begin = [&](int u) {
-        next_seq(s[u], p.S, n, p.order, p.off, fits);
-        fresh[u] = true;
-        if (s[u].seq < 0) return;
-        row[u] = s[u].o0;
-        left[u] = s[u].T - 1;
-        sym[u] = obs[row[u]];
-        nsym[u] = left[u] > 0 ? obs[row[u] + 1] : 0;
+    int32_t pseq;
+    bool pon, plast;
+    float psum;
+    int64_t E;
+    auto begin = [&]() {
+        next_seq(s, p.S, n, p.order, p.off, fits);
+        fresh = true;
+        if (s.seq < 0) return;
+        row = (int32_t)s.o0;
+        left = (int32_t)s.T - 1;
+        sym = obs[row];
+        nsym = left > 0 ? obs[row + 1] : 0;
     };
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        s[u].k = -1;
-        s[u].sl = cid + p.ncl * (ep.e + 4 * u);
-        row[u] = left[u] = sym[u] = nsym[u] = 0;
-        pon[u] = plast[u] = false;
-        pseq[u] = -1;
-        psum[u] = 0.f;
-        E[u] = 0;
-        begin(u);
-    }
-    const int32_t iters = half[0] > half[1] ? half[0] : half[1];
-    for (int32_t it = 0; it <= iters; ++it) {
-        const int b = it & 1, pb = b ^ 1;
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            if (it > half[u]) continue;          // the half has finished
-            const bool on = s[u].seq >= 0;
-            Vec<C::EC> em, o;
-            if (on) em.load(p.BT + (size_t)sym[u] * KP + c);
-            float sum = psum[u];
-            if (it > 0) {
-                if (C::NC == 2) {                // the peer's sum: in the order of the columns
-                    wt.cluster(&sm.x_peer[u][pb], step_phase(it - 1));
-                    const float q = sm.peer[pb][ep.e + 4 * u];
-                    sum = rank == 0 ? sum + q : q + sum;
-                }
-                if (it < half[u]) {
-                    wt.local(&sm.out_full[u], (uint32_t)(it - 1) & 1u);
-                    o.load(&sm.out[u][ep.e][ep.col]);
-                }
+    s.k = -1;
+    s.sl = cid + p.ncl * ep.g;
+    row = left = sym = nsym = 0;
+    pon = plast = false;
+    pseq = -1;
+    psum = 0.f;
+    E = 0;
+    begin();
+    const int32_t steps = half[u];
+    for (int32_t it = 0; it <= steps; ++it) {
+        const int b = (int)(it & 1), pb = b ^ 1;
+        const bool on = s.seq >= 0;
+        Vec<C::EC> em, o;
+        if (on) em.load(p.BT + (size_t)sym * KP + c);
+        float sum = psum;
+        if (it > 0) {
+            if (C::NC == 2) {                // the peer's sum: in the order of the columns
+                wt.cluster(&sm.x_peer[u][pb], step_phase(it - 1));
+                const float q = sm.peer[pb][ep.g];
+                sum = rank == 0 ? sum + q : q + sum;
             }
-            const int ex = scale_exp(sum);
-            if (it < half[u]) {
-                const float sc = pow2_scale(ex);
-                Vec<C::EC> x;
+            if (it < steps) {
+                wt.local(&sm.out_full[u], (uint32_t)(it - 1) & 1u);
+                o.load(&sm.out[u][ep.g & 3][ep.col]);
+            }
+        }
+        const int ex = scale_exp(sum);
+        if (it < steps) {
+            const float sc = pow2_scale(ex);
+            Vec<C::EC> x;
 #pragma unroll
-                for (int h = 0; h < C::EC; ++h) x.v[h] = on ? (fresh[u] ? pi.v[h] : o.v[h] * sc) * em.v[h] : 0.f;
-                psum[u] = ep.warp_sum(x);
-                ep.put(u, b, x, true, psum[u]);
-                if (on) x.store(p.X + (size_t)row[u] * KP + c);
-            }
-            // the books of the step before
-            if (pon[u]) {
-                if (plast[u]) {
-                    if (lead) {
-                        p.clast[pseq[u]] = sum;
-                        if (p.loglik) p.loglik[pseq[u]] = 0.6931471805599453 * (double)E[u] + log((double)sum);
-                    }
-                    E[u] = 0;
-                } else {
-                    if (lead) p.e[row[u] - 1] = ex;      // the sequence goes on: the row before this one
-                    E[u] += ex;
+            for (int h = 0; h < C::EC; ++h) x.v[h] = on ? (fresh ? pi.v[h] : o.v[h] * sc) * em.v[h] : 0.f;
+            psum = ep.warp_sum(x);
+            ep.put(b, x, true, psum);
+            if (on) x.store(p.X + (size_t)row * KP + c);
+        }
+        // the books of the step before
+        if (pon) {
+            if (plast) {
+                if (lead) {
+                    p.clast[pseq] = sum;
+                    if (p.loglik) p.loglik[pseq] = 0.6931471805599453 * (double)E + log((double)sum);
                 }
+                E = 0;
+            } else {
+                if (lead) p.e[row - 1] = ex;      // the sequence goes on: the row before this one
+                E += ex;
             }
-            // on to the next step
-            pon[u] = on;
-            plast[u] = left[u] == 0;
-            pseq[u] = s[u].seq;
-            if (on) {
-                if (left[u] == 0) {
-                    begin(u);
-                } else {
-                    fresh[u] = false;
-                    ++row[u];
-                    --left[u];
-                    sym[u] = nsym[u];
-                    nsym[u] = left[u] > 0 ? obs[row[u] + 1] : 0;
-                }
+        }
+        // on to the next step
+        pon = on;
+        plast = left == 0;
+        pseq = s.seq;
+        if (on) {
+            if (left == 0) {
+                begin();
+            } else {
+                fresh = false;
+                ++row;
+                --left;
+                sym = nsym;
+                nsym = left > 0 ? obs[row + 1] : 0;
             }
         }
     }
@@ -203,100 +195,93 @@ __device__ __forceinline__ void bwd_epilogue(const RowsPrm& p, int rank, int cid
                                              Waits& wt) {
     using C = Cfg<KP>;
     Epilogue<KP> ep(sm, rank);
+    const int u = ep.u;
     const int64_t n = (int64_t)p.ncl * kG;
     const int Cmax = p.Cmax;
     const int32_t* obs = p.obs + p.off[0];
     const int c = rank * C::Kh + ep.col;
     auto fits = [&](int64_t T) { return seg_len(T) <= Cmax; };
-    // the warp's two slots: the step to compute (row, steps left below it), its symbol and the one
+    // the warp's slot: the step to compute (row, steps left below it), its symbol and the one
     // below, the exponents of the two steps below, the sequence's weight and 1 / c_{T-1}
-    Slot s[2];
-    int32_t row[2], left[2], sym[2], nsym[2], eb[2], neb[2];
-    float wgt[2], cinv[2];
-    bool fresh[2];
-    auto begin = [&](int u) {
-        next_seq(s[u], p.S, n, p.order, p.off, fits);
-        fresh[u] = true;
-        if (s[u].seq < 0) return;
-        left[u] = s[u].T - 1;
-        row[u] = s[u].o0 + left[u];
-        sym[u] = obs[row[u]];
-        eb[u] = left[u] > 0 ? p.e[row[u] - 1] : 0;
-        nsym[u] = left[u] > 0 ? obs[row[u] - 1] : 0;
-        neb[u] = left[u] > 1 ? p.e[row[u] - 2] : 0;
-        wgt[u] = p.w ? (float)p.w[s[u].seq] : 1.f;
-        cinv[u] = 1.f / p.clast[s[u].seq];
+    Slot s;
+    int32_t row, left, sym, nsym, eb, neb;
+    float wgt, cinv;
+    bool fresh;
+    auto begin = [&]() {
+        next_seq(s, p.S, n, p.order, p.off, fits);
+        fresh = true;
+        if (s.seq < 0) return;
+        left = (int32_t)s.T - 1;
+        row = (int32_t)s.o0 + left;
+        sym = obs[row];
+        eb = left > 0 ? p.e[row - 1] : 0;
+        nsym = left > 0 ? obs[row - 1] : 0;
+        neb = left > 1 ? p.e[row - 2] : 0;
+        wgt = p.w ? (float)p.w[s.seq] : 1.f;
+        cinv = 1.f / p.clast[s.seq];
     };
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        s[u].k = -1;
-        s[u].sl = cid + p.ncl * (ep.e + 4 * u);
-        row[u] = left[u] = sym[u] = nsym[u] = eb[u] = neb[u] = 0;
-        wgt[u] = cinv[u] = 0.f;
-        begin(u);
+    {
+        s.k = -1;
+        s.sl = cid + p.ncl * ep.g;
+        row = left = sym = nsym = eb = neb = 0;
+        wgt = cinv = 0.f;
+        begin();
     }
-    const int32_t iters = half[0] > half[1] ? half[0] : half[1];
-    for (int32_t it = 0; it < iters; ++it) {
-        const int b = it & 1;
+    const int32_t steps = half[u];
+    for (int32_t it = 0; it < steps; ++it) {
+        const int b = (int)(it & 1);
+        const bool on = s.seq >= 0, more = on && left > 0;
+        Vec<C::EC> em, xr, o;
+        if (on) {
+            em.load(p.BT + (size_t)sym * KP + c);
+            xr.load(p.X + (size_t)row * KP + c);
+            // the rows of the coming steps on their way into L2
+            if ((ep.lane & 7) == 0 && left >= 4)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(p.X + (size_t)(row - 4) * KP + c));
+        }
+        if (it > 0) {
+            wt.local(&sm.out_full[u], (uint32_t)(it - 1) & 1u);
+            o.load(&sm.out[u][ep.g & 3][ep.col]);
+        }
+        const float sc = pow2_scale(eb);
+        Vec<C::EC> R, v;
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            if (it >= half[u]) continue;         // the half has finished
-            const bool on = s[u].seq >= 0, more = on && left[u] > 0;
-            Vec<C::EC> em, xr, o;
-            if (on) {
-                em.load(p.BT + (size_t)sym[u] * KP + c);
-                xr.load(p.X + (size_t)row[u] * KP + c);
-                // the rows of the coming steps on their way into L2
-                if ((ep.lane & 7) == 0 && left[u] >= 4)
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(p.X + (size_t)(row[u] - 4) * KP + c));
-            }
-            if (it > 0) {
-                wt.local(&sm.out_full[u], (uint32_t)(it - 1) & 1u);
-                o.load(&sm.out[u][ep.e][ep.col]);
-            }
-            const float sc = pow2_scale(eb[u]);
-            Vec<C::EC> R, v;
+        for (int h = 0; h < C::EC; ++h) {
+            R.v[h] = fresh ? cinv : o.v[h];
+            v.v[h] = more ? em.v[h] * R.v[h] * sc : 0.f;
+        }
+        ep.put(b, v, false, 0.f);
+        if (on) {
+            Vec<C::EC> g, q;
 #pragma unroll
             for (int h = 0; h < C::EC; ++h) {
-                R.v[h] = fresh[u] ? cinv[u] : o.v[h];
-                v.v[h] = more ? em.v[h] * R.v[h] * sc : 0.f;
+                g.v[h] = wgt * xr.v[h] * R.v[h];
+                q.v[h] = wgt * v.v[h];
             }
-            ep.put(u, b, v, false, 0.f);
-            if (on) {
-                Vec<C::EC> g, q;
+            const size_t at = (size_t)row * KP + c;
+            g.store(p.Gm + at);
+            if (more) q.store(p.Q + at - KP);
+            if (fresh) {
+                Vec<C::EC> z;
 #pragma unroll
-                for (int h = 0; h < C::EC; ++h) {
-                    g.v[h] = wgt[u] * xr.v[h] * R.v[h];
-                    q.v[h] = wgt[u] * v.v[h];
-                }
-                const size_t at = (size_t)row[u] * KP + c;
-                g.store(p.Gm + at);
-                if (more) q.store(p.Q + at - KP);
-                if (fresh[u]) {
-                    Vec<C::EC> z;
-#pragma unroll
-                    for (int h = 0; h < C::EC; ++h) z.v[h] = 0.f;
-                    z.store(p.Q + at);           // no transition leaves the last step
-                }
-                if (!more) {
-                    begin(u);
-                } else {
-                    fresh[u] = false;
-                    --row[u];
-                    --left[u];
-                    sym[u] = nsym[u];
-                    eb[u] = neb[u];
-                    nsym[u] = left[u] > 0 ? obs[row[u] - 1] : 0;
-                    neb[u] = left[u] > 1 ? p.e[row[u] - 2] : 0;
-                }
+                for (int h = 0; h < C::EC; ++h) z.v[h] = 0.f;
+                z.store(p.Q + at);           // no transition leaves the last step
+            }
+            if (!more) {
+                begin();
+            } else {
+                fresh = false;
+                --row;
+                --left;
+                sym = nsym;
+                eb = neb;
+                nsym = left > 0 ? obs[row - 1] : 0;
+                neb = left > 1 ? p.e[row - 2] : 0;
             }
         }
     }
     // the last steps' parts have landed before this CTA's shared memory goes
-    if (C::NC == 2)
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-            if (half[u] > 0) wt.cluster(&sm.x_peer[u][(half[u] - 1) & 1], step_phase(half[u] - 1));
+    if (C::NC == 2 && steps > 0) wt.cluster(&sm.x_peer[u][(steps - 1) & 1], step_phase(steps - 1));
 }
 
 template <int KP, bool BWD>
@@ -460,51 +445,9 @@ Layout layout(int K, int M, int64_t S, int64_t total_T) {
     return L;
 }
 
-// Clusters of the recurrences resident at once on the device (cached per device and kernel).
-template <typename Kern>
-int max_clusters(Kern kern, int nc) {
-    static std::mutex mu;
-    static std::map<std::pair<int, const void*>, int> cache;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const auto key = std::make_pair(dev, reinterpret_cast<const void*>(kern));
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = cache.find(key);
-    if (it != cache.end()) return it->second;
-    int n = 0;
-    if (nc == 2) {
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3((unsigned)(num_sms() / 2 * 2), 1, 1);
-        cfg.blockDim = dim3(kT, 1, 1);
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) n = 0;
-    } else if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kT, 0) == cudaSuccess) {
-        n *= num_sms();
-    }
-    cudaGetLastError();
-    if (n < 1) n = num_sms() / nc;
-    cache[key] = n;
-    return n;
-}
-
 using Kern = void (*)(RowsPrm);
 Kern fwd_kernel(int KP) { return KP == 64 ? k_rows<64, false> : KP == 128 ? k_rows<128, false> : k_rows_pair<false>; }
 Kern bwd_kernel(int KP) { return KP == 64 ? k_rows<64, true> : KP == 128 ? k_rows<128, true> : k_rows_pair<true>; }
-
-// Clusters of a launch: all that are resident, but no more than there are sequences; with a budget
-// of SMs, those that fit it.
-int clusters_for(Kern kern, int KP, int64_t S, int budget) {
-    const int nc = KP == 256 ? 2 : 1;
-    int64_t n = max_clusters(kern, nc);
-    if (budget > 0) n = std::min<int64_t>(n, std::max<int64_t>(1, n * budget / num_sms()));
-    return (int)std::max<int64_t>(1, std::min(n, S));
-}
 
 void fill(RowsPrm& p, const Layout& L, const RowsArgs& a) {
     char* ws = (char*)a.ws;

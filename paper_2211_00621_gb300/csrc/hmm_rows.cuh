@@ -2,13 +2,15 @@
 // step matrix in registers: one step of up to 8 sequences is out[g][j] = sum_i x[g][i] Mx[i][j].
 //
 // States are padded to KP = 64, 128 or 256 (zero probabilities add exact zeros); a CTA owns Kh = KP /
-// NC of them.  It has 8 contraction warps and 4 epilogue warps.
+// NC of them.  It has 8 contraction warps and 8 epilogue warps.
 //  * Contraction warp w takes WC = Kh / 8 columns, lane 4 ip + cg the rows 32 q + 4 ip .. + 3
 //    (q < KP / 32) and CW = WC / 4 columns: the thread's KP / 8 x CW block of Mx is loaded once per
 //    kernel.  The vectors come from shared memory (8 x 16 consecutive bytes a load); the rows' partial
 //    sums meet by a reduce-scatter over the 8 row lanes, not through shared memory.
-//  * Epilogue warp e owns sequence slots e and e + 4: all of a slot's bookkeeping is uniform over a
-//    warp, a row of the CTA's columns is one vector access, and its sum one warp reduction.
+//  * Epilogue warp g owns sequence slot g: all of a slot's bookkeeping is uniform over a warp, a row of
+//    the CTA's columns is one vector access, and its sum one warp reduction.  (4 warps of two slots
+//    each: a warp that waits for one half is late for the other; 4.8 ms where the log-space forward
+//    takes 3.9.)
 //
 // The 8 slots are two halves of 4 that run as two interleaved recurrences: a phase is one step of one
 // half, and the halves take turns, so that the epilogue, the hand-overs between the warps and the
@@ -16,6 +18,7 @@
 // hide behind the other half's products.  A half whose slots have all finished is left out.  In one
 // group of warps that did both (and a CTA barrier per step) a step took 5,300 cycles at K = 256, of
 // which the FMA pipe was busy 2,350: two warps per scheduler cannot cover the epilogue's latencies.
+// Now a step of both halves takes about 3,600 cycles, of which the FMA pipe needs 2,048.
 //
 // Slots and sequences: slot sl = cluster + clusters * g of n = 8 * clusters runs the sequences
 // k n + sl (k even) and k n + n - 1 - sl (k odd) of the order (by decreasing length), one after the
@@ -27,12 +30,17 @@
 
 #include <cooperative_groups.h>
 
+#include <algorithm>
+#include <map>
+#include <mutex>
+#include <utility>
+
 namespace accel {
 namespace hmm {
 namespace rows {
 
 constexpr int kCon = 256;       // contraction threads
-constexpr int kEpi = 128;       // epilogue threads
+constexpr int kEpi = 256;       // epilogue threads
 constexpr int kT = kCon + kEpi;
 constexpr int kG = 8;           // slots per cluster
 constexpr uint64_t kWaitNs = 2000000000ull;
@@ -82,12 +90,12 @@ struct Vec {
     }
 };
 
-// Registers of the two kinds of warps (K = 256: the launch gives 168 each).
+// Registers of the two kinds of warps (K = 256: the launch gives 128 each).
 template <int KP> __device__ __forceinline__ void regs_contraction() {
-    if constexpr (KP == 256) asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
+    if constexpr (KP == 256) asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
 }
 template <int KP> __device__ __forceinline__ void regs_epilogue() {
-    if constexpr (KP == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+    if constexpr (KP == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
 }
 
 // Bounded waits.  One that gives up reports and is not repeated: the kernel then finishes with
@@ -115,13 +123,13 @@ struct Waits {
     }
 };
 // the parity of the phase of step i's barrier of parity i & 1
-__device__ __forceinline__ uint32_t step_phase(int32_t i) { return (uint32_t)(i >> 1) & 1u; }
+__device__ __forceinline__ uint32_t step_phase(uint32_t i) { return (i >> 1) & 1u; }
 
 template <int KP>
 __device__ __forceinline__ void init_bars(Smem<KP>& sm) {
     if (threadIdx.x == 0) {
         for (int q = 0; q < 4; ++q) {
-            tc::mbar_init(&sm.x_own[q >> 1][q & 1], kEpi / 32);
+            tc::mbar_init(&sm.x_own[q >> 1][q & 1], 4);
             tc::mbar_init(&sm.x_peer[q >> 1][q & 1], 1);
         }
         tc::mbar_init(&sm.out_full[0], kCon / 32);
@@ -133,11 +141,11 @@ __device__ __forceinline__ void init_bars(Smem<KP>& sm) {
 // ---------------------------------------------------------------- slots
 __device__ __forceinline__ int64_t slot_at(int64_t n, int32_t sl, int64_t k) { return k * n + ((k & 1) ? n - 1 - sl : sl); }
 
-// The sequences of one slot, one after the other (rows and sequences fit 31 bits here).
+// The sequences of one slot, one after the other.
 struct Slot {
     int32_t k, sl;
     int32_t seq;           // -1: none left
-    int32_t o0, T;         // its first row (from the first sequence's offset), its length
+    int64_t o0, T;         // its first row (from the first sequence's offset), its length
 };
 
 // Advance the slot to its next sequence that is neither empty nor refused by `ok`.
@@ -153,16 +161,16 @@ __device__ __forceinline__ void next_seq(Slot& s, int64_t S, int64_t n, const in
         if (q >= S) continue;
         s.seq = order ? order[q] : (int32_t)q;
         const int64_t o0 = off[s.seq];
-        s.o0 = (int32_t)(o0 - off[0]);
-        s.T = (int32_t)(off[s.seq + 1] - o0);
+        s.o0 = o0 - off[0];
+        s.T = off[s.seq + 1] - o0;
         if (s.T > 0 && ok(s.T)) return;
     }
 }
 
 // The steps of the slots: half[h] = the largest of half h's (the first 8 warps count a slot each).
-template <typename Ok>
+template <typename Ok, typename I>
 __device__ __forceinline__ void slot_totals(int64_t* tot, int64_t S, int64_t n, int32_t cid, int32_t ncl,
-                                            const int32_t* order, const int64_t* off, Ok&& ok, int32_t (&half)[2]) {
+                                            const int32_t* order, const int64_t* off, Ok&& ok, I (&half)[2]) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (w < kG) {
         int64_t sum = 0;
@@ -180,7 +188,7 @@ __device__ __forceinline__ void slot_totals(int64_t* tot, int64_t S, int64_t n, 
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         half[h] = 0;
-        for (int g = 0; g < 4; ++g) half[h] = (int32_t)tot[4 * h + g] > half[h] ? (int32_t)tot[4 * h + g] : half[h];
+        for (int g = 0; g < 4; ++g) half[h] = (I)tot[4 * h + g] > half[h] ? (I)tot[4 * h + g] : half[h];
     }
 }
 
@@ -191,11 +199,6 @@ struct Contraction {
     int rank, w, lane, ip, cg;
     float2 a[2 * C::NQ][C::CW];                    // (rows 2k, 2k + 1) of the lane's 4 per q
 
-    // the row block of step q: the CTA's own half first
-    __device__ __forceinline__ int row0(int q) const {
-        if (C::NC == 1) return 32 * q;
-        return (q < C::NQ / 2 ? rank : rank ^ 1) * C::Kh + 32 * (q % (C::NQ / 2));
-    }
     __device__ __forceinline__ void load(const float* __restrict__ Mx, int r) {
         rank = r;
         w = threadIdx.x >> 5;
@@ -206,17 +209,16 @@ struct Contraction {
         for (int q = 0; q < C::NQ; ++q)
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-                const float* p = Mx + (size_t)(row0(q) + 4 * ip + 2 * k) * KP + rank * C::Kh + w * C::WC + cg * C::CW;
+                const float* p = Mx + (size_t)(32 * q + 4 * ip + 2 * k) * KP + rank * C::Kh + w * C::WC + cg * C::CW;
 #pragma unroll
                 for (int h = 0; h < C::CW; ++h) a[2 * q + k][h] = make_float2(p[h], p[KP + h]);
             }
     }
-    // rows [q0, q1) of the four vectors at x, added to acc
-    template <int Q0, int Q1>
+    // the products of the four vectors at x, added to acc
     __device__ __forceinline__ void add(const float* x, float2 (&acc)[4][C::CW]) const {
 #pragma unroll
-        for (int q = Q0; q < Q1; ++q) {
-            const float* xq = x + row0(q) + 4 * ip;
+        for (int q = 0; q < C::NQ; ++q) {
+            const float* xq = x + 32 * q + 4 * ip;
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
                 const float4 v = *reinterpret_cast<const float4*>(xq + g * C::ST);
@@ -262,12 +264,12 @@ struct Contraction {
 };
 
 // The contraction warps' part of a kernel: steps 1 .. half[u] - 1 of both halves.
-template <int KP>
-__device__ __forceinline__ void contraction_loop(const Contraction<KP>& m, Smem<KP>& sm, const int32_t (&half)[2], Waits& wt) {
+template <int KP, typename I>
+__device__ __forceinline__ void contraction_loop(const Contraction<KP>& m, Smem<KP>& sm, const I (&half)[2], Waits& wt) {
     using C = Cfg<KP>;
-    const int32_t iters = half[0] > half[1] ? half[0] : half[1];
-    for (int32_t it = 1; it < iters; ++it) {
-        const int pb = (it & 1) ^ 1;
+    const I iters = half[0] > half[1] ? half[0] : half[1];
+    for (I it = 1; it < iters; ++it) {
+        const int pb = (int)(it & 1) ^ 1;
         const uint32_t ph = step_phase(it - 1);
 #pragma unroll 1
         for (int u = 0; u < 2; ++u) {
@@ -279,13 +281,9 @@ __device__ __forceinline__ void contraction_loop(const Contraction<KP>& m, Smem<
                 for (int h = 0; h < C::CW; ++h) acc[g][h] = make_float2(0.f, 0.f);
             const float* x = &sm.x[pb][4 * u][0];
             wt.local(&sm.x_own[u][pb], ph);
-            if constexpr (C::NC == 2) {
-                m.template add<0, C::NQ / 2>(x, acc);
-                wt.cluster(&sm.x_peer[u][pb], ph);
-                m.template add<C::NQ / 2, C::NQ>(x, acc);
-            } else {
-                m.template add<0, C::NQ>(x, acc);
-            }
+            // (products of the own columns before this wait: a second bubble a phase, 3% slower)
+            if constexpr (C::NC == 2) wt.cluster(&sm.x_peer[u][pb], ph);
+            m.add(x, acc);
             m.reduce(acc, &sm.out[u][0][0]);
             __syncwarp();
             if (m.lane == 0) tc::mbar_arrive(&sm.out_full[u]);
@@ -298,11 +296,12 @@ template <int KP>
 struct Epilogue {
     using C = Cfg<KP>;
     Smem<KP>& sm;
-    int rank, e, lane;
+    int rank, g, u, lane;                          // the warp's slot and its half
     int col;                                       // the lane's first column within the CTA's
     uint32_t peer_x, peer_s, peer_bar;             // the peer's buffers (shared::cluster addresses)
     __device__ __forceinline__ Epilogue(Smem<KP>& s, int r) : sm(s), rank(r) {
-        e = (threadIdx.x - kCon) >> 5;
+        g = (threadIdx.x - kCon) >> 5;
+        u = g >> 2;
         lane = threadIdx.x & 31;
         col = C::EC * lane;
         if constexpr (C::NC == 2) {
@@ -315,8 +314,8 @@ struct Epilogue {
         }
     }
     // The slot's new vector (and a scalar of it) into parity b of both CTAs, and the end of the phase.
-    __device__ __forceinline__ void put(int u, int b, const Vec<C::EC>& v, bool scalar, float s) {
-        const int g = e + 4 * u, c = rank * C::Kh + col;
+    __device__ __forceinline__ void put(int b, const Vec<C::EC>& v, bool scalar, float s) {
+        const int c = rank * C::Kh + col;
         v.store(&sm.x[b][g][c]);
         if constexpr (C::NC == 2) {
             const uint32_t bar = peer_bar + 8u * (uint32_t)(2 * u + b);
@@ -326,7 +325,7 @@ struct Epilogue {
         __syncwarp();
         if (lane == 0) {
             tc::mbar_arrive(&sm.x_own[u][b]);
-            if (C::NC == 2 && e == 0)              // the peer's bytes of this step
+            if (C::NC == 2 && (g & 3) == 0)              // the peer's bytes of this step
                 tc::mbar_arrive_expect_tx(&sm.x_peer[u][b], (uint32_t)(4 * C::Kh * 4 + (scalar ? 4 * 4 : 0)));
         }
     }
@@ -339,6 +338,50 @@ struct Epilogue {
         return s;
     }
 };
+
+// ---------------------------------------------------------------- launches
+// Clusters of the recurrences resident at once on the device (cached per device and kernel).
+template <typename Kern>
+int max_clusters(Kern kern, int nc) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, int> cache;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const auto key = std::make_pair(dev, reinterpret_cast<const void*>(kern));
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = cache.find(key);
+    if (it != cache.end()) return it->second;
+    int n = 0;
+    if (nc == 2) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)(num_sms() / 2 * 2), 1, 1);
+        cfg.blockDim = dim3(kT, 1, 1);
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) n = 0;
+    } else if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kT, 0) == cudaSuccess) {
+        n *= num_sms();
+    }
+    cudaGetLastError();
+    if (n < 1) n = num_sms() / nc;
+    cache[key] = n;
+    return n;
+}
+
+// Clusters of a launch: all that are resident, but no more than there are sequences; with a budget
+// of SMs, those that fit it.
+template <typename Kern>
+int clusters_for(Kern kern, int KP, int64_t S, int budget) {
+    const int nc = KP == 256 ? 2 : 1;
+    int64_t n = max_clusters(kern, nc);
+    if (budget > 0) n = std::min<int64_t>(n, std::max<int64_t>(1, n * budget / num_sms()));
+    return (int)std::max<int64_t>(1, std::min(n, S));
+}
 
 }  // namespace rows
 }  // namespace hmm

@@ -10,19 +10,20 @@
 // Each sequence keeps la = c + r with r in FP32 and the running offset c (the sum of the
 // per-step maxima, a sum of log scale factors) in FP64.
 //
-// Two kernels:
-//  * k_plain_warp<J> (K <= 32 J, J <= 2): one warp per sequence, lane l owns states
-//    l and l + 32; the two columns of A it needs live in registers (K floats each), the
-//    emission table log B^T in shared memory; no block-wide synchronisation.
-//  * k_plain_cta (K <= 256): one CTA per group of G sequences (ordered by length so a
-//    group's lengths are alike); thread j owns state j of all G sequences and streams A's
-//    column j from L2, reusing each element G times.
+// k_plain_warp<J> (K <= 32 J, J <= 2): one warp per sequence, lane l owns states l and l + 32; the two
+// columns of A it needs live in registers (K floats each), the emission table log B^T in shared
+// memory; no block-wide synchronisation.  More states: k_hmm_rows_log.cu.
 #include "common.cuh"
 #include "hmm_internal.cuh"
-#include "simt_stream.cuh"
 
 namespace accel {
 namespace hmm {
+
+namespace rows {
+size_t log_ws_bytes(int K, int M, int64_t S);
+accel_status log_forward(const accel_hmm_model* m, const int32_t* obs, const int64_t* off, int64_t S, double* loglik,
+                         char* ws, int32_t* d_status, cudaStream_t st);
+}
 
 // ---------------------------------------------------------------- warp per sequence
 template <int J>
@@ -113,143 +114,7 @@ k_plain_warp(const float* __restrict__ logA, const float* __restrict__ logB, con
     if (lane == 0) loglik[s] = c + (double)m + log((double)e);
 }
 
-// ---------------------------------------------------------------- CTA per G sequences
-constexpr int kCtaThreads = 256;
-constexpr int kG = 8;
-
-// exp(log A) with row stride Kp (padding zero)
-__global__ void k_exp_f32(const float* __restrict__ in, float* __restrict__ out, int K, int Kp) {
-    int64_t n = (int64_t)K * Kp;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int r = (int)(i / Kp), c = (int)(i % Kp);
-        out[i] = c < K ? __expf(in[(int64_t)r * K + c]) : 0.f;
-    }
-}
-
-__host__ __device__ inline size_t cta_off_b(int Kp) { return align_up(simt::stream_smem_bytes(Kp), 16); }
-
-__global__ void __launch_bounds__(kCtaThreads)
-k_plain_cta(const float* __restrict__ Aexp, const float* __restrict__ logB, const float* __restrict__ logpi,
-            int K, int M, const int32_t* __restrict__ obs, const int64_t* __restrict__ off, int64_t S,
-            const int32_t* __restrict__ order, double* __restrict__ loglik, int32_t* __restrict__ status) {
-    extern __shared__ __align__(16) float smem_f[];
-    char* smem = reinterpret_cast<char*>(smem_f);
-    const int Kp = (K + 3) & ~3;                // padded row stride (16-byte rows)
-    simt::AStream as;
-    simt::as_init(as, smem, K, Kp);
-    float* sB = reinterpret_cast<float*>(smem + cta_off_b(Kp));                        // [M][K]
-    float* sP = sB + (((size_t)M * K + 3) & ~(size_t)3);                               // [kG][Kp]
-    __shared__ float s_red[kG][kCtaThreads / 32];
-    __shared__ int64_t s_T[kG], s_o0[kG];
-    const int j = threadIdx.x, lane = j & 31, w = j >> 5;
-    for (int idx = threadIdx.x; idx < M * K; idx += blockDim.x) {
-        int jj = idx / M, k = idx - jj * M;
-        sB[k * K + jj] = logB[idx];
-    }
-    int64_t seq[kG];
-#pragma unroll
-    for (int g = 0; g < kG; ++g) {
-        int64_t q = blockIdx.x * (int64_t)kG + g;
-        seq[g] = q < S ? order[q] : -1;
-    }
-    if (j < kG) {
-        int64_t sq = seq[j];
-        s_o0[j] = sq >= 0 ? off[sq] : 0;
-        s_T[j] = sq >= 0 ? off[sq + 1] - off[sq] : 0;
-    }
-    __syncthreads();
-    int64_t T[kG], o0[kG], Tmax = 0;
-#pragma unroll
-    for (int g = 0; g < kG; ++g) { T[g] = s_T[g]; o0[g] = s_o0[g]; Tmax = T[g] > Tmax ? T[g] : Tmax; }
-    const bool jv = j < K;
-    float r[kG];
-    double c[kG];
-#pragma unroll
-    for (int g = 0; g < kG; ++g) {
-        c[g] = 0.0;
-        r[g] = (jv && T[g] > 0) ? logpi[j] + sB[obs[o0[g]] * K + j] : -INFINITY;
-    }
-    simt::as_begin(as, Aexp);
-    for (int64_t t = 1; t < Tmax; ++t) {
-        // per-sequence maxima over states
-        float m[kG];
-        bool act[kG];
-#pragma unroll
-        for (int g = 0; g < kG; ++g) {
-            act[g] = t < T[g];
-            float v = r[g];
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, d));
-            if (lane == 0) s_red[g][w] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int g = 0; g < kG; ++g) {
-            float v = s_red[g][0];
-            for (int q = 1; q < kCtaThreads / 32; ++q) v = fmaxf(v, s_red[g][q]);
-            m[g] = v;
-            if (jv) sP[g * Kp + j] = act[g] ? __expf(r[g] - v) : 0.f;
-        }
-        __syncthreads();
-        float acc[kG];
-        if (!simt::as_matvec<kG>(as, sP, Kp, act, acc)) {
-            if (threadIdx.x == 0) report_status(status, ACCEL_ERR_TIMEOUT);
-            simt::as_drain(as);
-            return;
-        }
-#pragma unroll
-        for (int g = 0; g < kG; ++g) {
-            if (act[g]) {
-                int32_t ob = obs[o0[g] + t];
-                r[g] = jv ? __logf(acc[g]) + sB[ob * K + j] : -INFINITY;
-                c[g] += (double)m[g];
-            }
-        }
-        __syncthreads();   // sP and s_red reuse
-    }
-    if (!simt::as_end(as)) {
-        if (threadIdx.x == 0) report_status(status, ACCEL_ERR_TIMEOUT);
-        simt::as_drain(as);
-        return;
-    }
-    // logL = c + LSE_j r
-#pragma unroll
-    for (int g = 0; g < kG; ++g) {
-        float v = r[g];
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, d));
-        if (lane == 0) s_red[g][w] = v;
-    }
-    __syncthreads();
-    float m[kG];
-#pragma unroll
-    for (int g = 0; g < kG; ++g) {
-        float v = s_red[g][0];
-        for (int q = 1; q < kCtaThreads / 32; ++q) v = fmaxf(v, s_red[g][q]);
-        m[g] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int g = 0; g < kG; ++g) {
-        float e = jv ? __expf(r[g] - m[g]) : 0.f;
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) e += __shfl_xor_sync(0xffffffffu, e, d);
-        if (lane == 0) s_red[g][w] = e;
-    }
-    __syncthreads();
-    if (j < kG) {
-        int g = j;
-        float e = 0.f;
-        for (int q = 0; q < kCtaThreads / 32; ++q) e += s_red[g][q];
-        if (seq[g] >= 0) loglik[seq[g]] = c[g] + (double)m[g] + log((double)e);
-    }
-}
-
-size_t plain_ws_bytes(int K, int M, int64_t S) {
-    (void)M;
-    if (K <= 64) return 0;
-    return align_up((size_t)K * ((K + 3) & ~3) * 4, 256) + order_ws_bytes(S);
-}
+size_t plain_ws_bytes(int K, int M, int64_t S) { return K <= 64 ? 0 : rows::log_ws_bytes(K, M, S); }
 
 accel_status plain_forward(const accel_hmm_model* m, const int32_t* obs, const int64_t* off, int64_t S,
                            double* loglik, char* ws, int32_t* d_status, cudaStream_t st) {
@@ -267,19 +132,11 @@ accel_status plain_forward(const accel_hmm_model* m, const int32_t* obs, const i
         }
         return after_launch(st, "hmm_forward(fp32 warp)", 1);
     }
-    const int Kp = (K + 3) & ~3;
-    size_t smem = cta_off_b(Kp) + ((((size_t)M * K + 3) & ~(size_t)3) + (size_t)kG * Kp) * sizeof(float);
-    ACCEL_REQUIRE(smem <= (size_t)max_smem_optin(), ACCEL_ERR_UNSUPPORTED, "hmm_forward: M*K too large for the FP32 kernel");
-    float* Aexp = (float*)ws;
-    int32_t* order = (int32_t*)(ws + align_up((size_t)K * Kp * 4, 256));
-    char* order_scratch = (char*)order + align_up((size_t)S * 4, 256);
-    k_exp_f32<<<num_sms() * 2, 256, 0, st>>>(m->log_A, Aexp, K, Kp);
-    accel_status r = order_by_length(off, S, order, order_scratch, st);
-    if (r != ACCEL_OK) return r;
-    ACCEL_CUDA_TRY(cudaFuncSetAttribute(k_plain_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    unsigned grid = (unsigned)((S + kG - 1) / kG);
-    k_plain_cta<<<grid, kCtaThreads, smem, st>>>(Aexp, m->log_B, m->log_pi, K, M, obs, off, S, order, loglik, d_status);
-    return after_launch(st, "hmm_forward(fp32 cta)", 5);
+    // the models taken: a K x K stream ring, the emission table and eight vectors within shared memory
+    const size_t Kp = (size_t)((K + 3) & ~3);
+    const size_t bytes = align_up(3 * 32 * Kp * 4 + 24, 16) + ((((size_t)M * K + 3) & ~(size_t)3) + 8 * Kp) * sizeof(float);
+    ACCEL_REQUIRE(bytes <= (size_t)max_smem_optin(), ACCEL_ERR_UNSUPPORTED, "hmm_forward: M*K too large for the FP32 kernel");
+    return rows::log_forward(m, obs, off, S, loglik, ws, d_status, st);
 }
 
 }  // namespace hmm
