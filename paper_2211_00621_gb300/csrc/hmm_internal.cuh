@@ -17,7 +17,14 @@ constexpr size_t kQueueOff = 16;         // uint64 sequence-queue counter
 size_t order_ws_bytes(int64_t S);
 accel_status order_by_length(const int64_t* d_off, int64_t S, int32_t* d_order, char* scratch, cudaStream_t st);
 
-// FP32 log-space forward (k_hmm_plain.cu).
+// The largest of the warp's values (one instruction; NaNs are left out, as by fmaxf).
+__device__ __forceinline__ float warp_max_f32(float v) {
+    float m;
+    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+    return m;
+}
+
+// FP32 log-space forward (k_hmm_plain.cu, k_hmm_rows_log.cu).
 size_t plain_ws_bytes(int K, int M, int64_t S);
 accel_status plain_forward(const accel_hmm_model* m, const int32_t* obs, const int64_t* off, int64_t S,
                            double* loglik, char* ws, int32_t* d_status, cudaStream_t st);

@@ -64,9 +64,7 @@ __device__ __forceinline__ float warp_max(const Vec<N>& v) {
     float m = v.v[0];
 #pragma unroll
     for (int h = 1; h < N; ++h) m = fmaxf(m, v.v[h]);
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
-    return m;
+    return warp_max_f32(m);
 }
 
 // Shared memory beside the engine's: the maxima of the peer's columns.

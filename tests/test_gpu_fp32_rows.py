@@ -1,4 +1,4 @@
-"""The FP32 forward of more than 64 states: padded state counts, uneven slots, impossible states and
+"""The FP32 forward: padded state counts, uneven slots, impossible states and
 halves, the shortest sequences, offsets that start inside the observations."""
 import numpy as np
 import pytest
@@ -41,9 +41,20 @@ def test_matches_the_oracle(K, M, S, lo, hi):
     assert np.array_equal(got, _run(logs, p))
 
 
+# A warp per sequence: K around the lanes' columns, lengths around the chunks of 32 symbols, warps without
+# a sequence
+@pytest.mark.parametrize("K", [1, 2, 5, 31, 32, 33, 63, 64])
+@pytest.mark.parametrize("M,S,lo,hi", [(3, 70, 1, 70), (130, 9, 28, 36), (7, 1, 97, 97)])
+def test_up_to_64_states(K, M, S, lo, hi):
+    p, logs = _inputs(K, M, S, lo, hi, K + 3 * S)
+    got = _run(logs, p)
+    ref = ohmm.loglik_batch(p, params=ohmm.params_from_f32_logs(logs))
+    assert np.all(np.abs(got - ref) <= _bound(K, p["lengths"]))
+
+
 # One half of the states (and so one CTA of a pair) impossible at every step, at every other step, or
 # improbable beyond the range of FP32
-@pytest.mark.parametrize("K", [80, 256])
+@pytest.mark.parametrize("K", [40, 80, 256])
 @pytest.mark.parametrize("low", [-np.inf, -300.0])
 @pytest.mark.parametrize("side", [0, 1])
 def test_impossible_and_improbable_halves(K, low, side):
