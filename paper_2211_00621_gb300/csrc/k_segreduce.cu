@@ -18,6 +18,7 @@
 //    fixup kernel that folds the preceding tiles' carry-outs in tile order.
 #include "common.cuh"
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <type_traits>
@@ -416,6 +417,210 @@ k_segsum(const Tin* __restrict__ data, int64_t N, const int64_t* __restrict__ of
     }
 }
 
+// Integer sums as a stream: resident CTAs, each over a contiguous range of whole tiles, so that the
+// next tile's vectors (and its segments' offsets) are on their way while a tile is summed.
+//  * A warp takes an eighth of the tile: coalesced 16-byte loads into registers, through its own part of
+//    the staging buffer (swizzled) to IT contiguous elements a lane, one warp scan of the lanes' sums.  A
+//    position's prefix is the sums of the warps and lanes before it plus at most IT elements, read back
+//    from the buffer.
+//  * A segment ends in the first tile that reaches its last element, and its sum is the difference of
+//    the prefixes at its ends, which count from the CTA's first element on: a segment open at the end of a
+//    tile only leaves the prefix of its start behind.  Wrapping 64-bit addition forms a group, so
+//    differences are exact.  A lane looks up one boundary, a warp 32 (and so 31 segments); warps without
+//    any go on to the next tile.  Ranges meet by the fix-up kernel, as tiles do.
+//  * One barrier a tile (buffers alternate): it counts the segments that end in the tile.
+// The CTA finds its first segment by a 32-way search of the offsets while its first tile is under way;
+// no partition pass over the offsets.
+//
+// What bounds it: the tiles' latencies (half the issue slots are used, 70% of the copy rate).  2^20
+// segments of 0 to 256 32-bit elements: 111 us (537 MB; a plain read of them takes 97); the partition, a
+// CTA per tile (k_segsum) and the fix-up: 154 us.  Tried: cp.async into a third buffer instead of
+// registers (132 us), a prefix per vector (132: the shared memory it takes is L1 that the loads and the
+// offsets need), five or six CTAs an SM (152, 203: fewer registers), L2 prefetch ahead (no change).
+// k_segsum stays for N < 16 S, segments of a few elements, where it is as fast (2^23 segments of 0 to 8:
+// 128 us, 136 as a stream).  Where many tiny segments lie side by side in the data, a range that holds
+// them is slow (10 us a tile of one-element segments): half of 2^21 segments of one element, the others
+// of 60, 197 us, 101 by k_segsum; a run of 500,000 empty ones inside one tile, 355 us, 1,950 by k_segsum.
+template <typename Tin, typename Tout, bool SQ>
+__global__ void __launch_bounds__(kThreads, 4)
+k_segsum_stream(const Tin* __restrict__ data, int64_t N, const int64_t* __restrict__ off, int64_t S, int64_t span, int64_t ranges,
+                int map_op, double scalar, Tout* __restrict__ out, int64_t* __restrict__ lo_arr,
+                int64_t* __restrict__ tail_seg, int64_t* __restrict__ tail_val) {
+    constexpr int IT = items<Tin>();
+    constexpr int TE = tile_elems<Tin>();
+    constexpr int PV = 16 / (int)sizeof(Tin);
+    constexpr int NW = kThreads / 32;
+    constexpr int kSeg = 31 * NW;                      // segments looked at together
+    __shared__ __align__(16) int4 s_vec[2][kVecs];
+    __shared__ uint64_t s_ex[2][kThreads];             // the sum of the lanes before, within the warp
+    __shared__ uint64_t s_tot[2][NW];                  // the warps' sums
+    __shared__ uint64_t s_open[2];                     // prefix at the open segment's start
+    __shared__ uint64_t s_base[2];                     // ... at the end of the tile
+    __shared__ int64_t s_first;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int64_t sc = (int64_t)scalar;
+
+    // the warp's vectors 32 r + lane of the tile at e, zeros beyond the data
+    const int v0 = warp * (kVecs / NW) + lane;
+    int4 raw[kVecPerThread];
+    auto load = [&](int64_t e) {
+        if (e + TE <= N) {
+            const int4* src = reinterpret_cast<const int4*>(data + e) + v0;
+#pragma unroll
+            for (int r = 0; r < kVecPerThread; ++r) raw[r] = __ldg(src + r * 32);
+            return;
+        }
+#pragma unroll
+        for (int r = 0; r < kVecPerThread; ++r) {
+            Tin* x = reinterpret_cast<Tin*>(&raw[r]);
+#pragma unroll
+            for (int i = 0; i < PV; ++i) {
+                const int64_t at = e + (int64_t)(v0 + r * 32) * PV + i;
+                x[i] = at < N ? data[at] : Tin(0);
+            }
+        }
+    };
+    // (every map but x*x + 1 takes 0 to 0; the sum of that one's ones is the position)
+    auto g = [&](Tin x) -> uint64_t { return SQ ? (uint64_t)sq_wide(x) : gmap<Tin>(map_op, (int64_t)x, sc); };
+
+    const int j = warp * 31 + lane;                    // the lane's boundary: the start of segment q + j
+    // (unconditional loads: behind a test one waits for the other)
+    auto off_at = [&](int64_t s) {
+        const int64_t v = off[s < S ? s : S];
+        return s <= S ? v : N + TE;
+    };
+    int b = 0;
+    for (int64_t range = blockIdx.x; range < ranges; range += gridDim.x) {
+        const int64_t E0 = range * span, E1 = E0 + span < N ? E0 + span : N;
+        load(E0);
+        if (warp == 0) {
+            // the first segment whose end lies beyond E0 (in the first range: 0)
+            int64_t a = 0, z = E0 > 0 ? S : 0;             // it is in [a, z]
+            while (a < z) {
+                const int64_t step = (z - a + 31) / 32, at = a + (lane + 1) * step - 1;
+                const bool before = at < z && off[at + 1] <= E0;
+                const int k = __popc(__ballot_sync(0xffffffffu, before));
+                a += k * step;
+                z = a + step - 1 < z ? a + step - 1 : z;
+            }
+            if (lane == 0) {
+                s_first = a < z ? a : z;
+                s_open[b ^ 1] = s_base[b ^ 1] = 0;
+            }
+        }
+        __syncthreads();
+        int64_t q = s_first;                               // the first segment that has not ended
+        if (t == 0) {
+            lo_arr[range] = q;
+            if (range == ranges - 1) lo_arr[ranges] = S;
+        }
+        int64_t bd = off_at(q + j);
+        for (int64_t e0 = E0; e0 < E1; e0 += TE, b ^= 1) {
+            const int64_t e1 = e0 + TE < E1 ? e0 + TE : E1;
+            // ---- the lanes' sums and their scan
+#pragma unroll
+            for (int r = 0; r < kVecPerThread; ++r) s_vec[b][swz(v0 + r * 32)] = raw[r];
+            if (e0 + TE < E1) load(e0 + TE);
+            __syncwarp();
+            uint64_t own = 0;
+#pragma unroll
+            for (int r = 0; r < kVecPerThread; ++r) {
+                const int4 v = s_vec[b][swz(t * kVecPerThread + r)];
+                const Tin* x = reinterpret_cast<const Tin*>(&v);
+#pragma unroll
+                for (int i = 0; i < PV; ++i) own += g(x[i]);
+            }
+            uint64_t inc = own;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint64_t o = __shfl_up_sync(0xffffffffu, inc, d);
+                if (lane >= d) inc += o;
+            }
+            s_ex[b][t] = inc - own;
+            if (lane == 31) s_tot[b][warp] = inc;
+            int n = __syncthreads_count(lane > 0 && bd <= e1);   // segments that end here, of the next kSeg
+            // ---- the boundaries
+            if (warp * 31 <= n) {
+                uint64_t grp = lane < NW ? s_tot[b][lane] : 0ull;   // the sum of the warps up to the lane's
+                const uint64_t G = s_base[b ^ 1];
+#pragma unroll
+                for (int d = 1; d < NW; d <<= 1) {
+                    const uint64_t o = __shfl_up_sync(0xffffffffu, grp, d);
+                    if (lane >= d) grp += o;
+                }
+                if (t == NW - 1) s_base[b] = G + grp + (SQ ? (uint64_t)(e1 - e0) : 0ull);
+                // segments s .. s + 30, whose boundaries the lanes hold; those before `end` end in this tile
+                auto finish = [&](int64_t s, int64_t end, int64_t bd) {
+                    const int64_t rel = bd - e0;
+                    const int p = rel < 0 ? 0 : rel > TE ? TE : (int)rel, k = p > 0 ? p - 1 : 0, tt = k / IT;
+                    uint64_t P = s_ex[b][tt];
+                    const uint64_t before = __shfl_sync(0xffffffffu, grp, (tt >> 5) > 0 ? (tt >> 5) - 1 : 0);
+                    if (tt >> 5) P += before;
+#pragma unroll
+                    for (int r = 0; r < kVecPerThread; ++r) {
+                        const int4 v = s_vec[b][swz(tt * kVecPerThread + r)];
+                        const Tin* x = reinterpret_cast<const Tin*>(&v);
+#pragma unroll
+                        for (int i = 0; i < PV; ++i)
+                            if (r * PV + i <= k % IT) P += g(x[i]);
+                    }
+                    if (SQ) P += (uint64_t)p;
+                    P = bd < e0 ? s_open[b ^ 1] : p > 0 ? G + P : G;
+                    const uint64_t left = __shfl_up_sync(0xffffffffu, P, 1);
+                    if (lane > 0 && s + lane <= end) out[s + lane - 1] = (Tout)(int64_t)(P - left);
+                    if (s + lane == end) s_open[b] = P;    // (the one left open)
+                };
+                finish(q + warp * 31, q + n, bd);
+                if (n == kSeg) {
+                    // Many segments end here: every warp looks for the first that does not and takes every
+                    // eighth group of those before it, four at a time; a long run of empty ones goes by its
+                    // first and last.
+                    q += kSeg;
+                    int64_t a = q, z = q + TE < S && off[q + TE + 1] > e1 ? q + TE : S;   // it is in [a, z]
+                    while (a < z) {
+                        const int64_t step = (z - a + 31) / 32, at = a + (lane + 1) * step - 1;
+                        const int c = __popc(__ballot_sync(0xffffffffu, at < z && off[at + 1] <= e1));
+                        a += c * step;
+                        z = a + step - 1 < z ? a + step - 1 : z;
+                    }
+                    const int64_t end = a < z ? a : z;
+                    constexpr int kRun = 32 * kThreads;
+                    for (; q + kRun <= end && off[q] == off[q + kRun]; q += kRun)
+                        for (int i = t; i < kRun; i += kThreads) out[q + i] = Tout(0);
+                    for (int64_t s = q + warp * 31; s <= end; s += 4 * kSeg) {
+                        int64_t four[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) four[u] = off_at(s + u * kSeg + lane);
+                        if (lane % 16 == 0)                // the offsets of the round after the next
+#pragma unroll
+                            for (int u = 8; u < 12; ++u)
+                                if (s + u * kSeg + lane <= S) asm volatile("prefetch.global.L2 [%0];" ::"l"(off + s + u * kSeg + lane));
+#pragma unroll 1
+                        for (int u = 0; u < 4; ++u) {
+                            if (s + u * kSeg > end) break;
+                            finish(s + u * kSeg, end, four[0]);
+                            four[0] = four[1];
+                            four[1] = four[2];
+                            four[2] = four[3];
+                        }
+                    }
+                    q = end;
+                    n = 0;
+                }
+            }
+            q += n;
+            bd = off_at(q + j);
+        }
+        // ---- the segment left open
+        __syncthreads();
+        if (t == 0) {
+            const bool open = q < S && bd < E1;
+            tail_seg[range] = open ? q : -1;
+            if (open) tail_val[range] = (int64_t)(s_base[b ^ 1] - s_open[b ^ 1]);
+        }
+    }
+}
+
 // Folds the carry-outs of the tiles preceding b into the first segment b owns, when that
 // segment started in an earlier tile.  Tile order is kept, so float results are
 // deterministic.
@@ -496,12 +701,11 @@ static Layout layout(int64_t N, int64_t S, size_t in_size) {
     return L;
 }
 
-// Tiles half a wave ahead: half the CTAs resident at once on the device (measured at 2^20
-// segments: half a wave 3,452 GB/s, one wave 3,409, two waves 3,342, none 3,187).
+// CTAs of a kernel resident at once on the device (looked up once per device and kernel).
 template <typename KernT>
-static int64_t prefetch_distance(KernT kern) {
+static int64_t resident_ctas(KernT kern) {
     static std::mutex mu;
-    static std::map<std::pair<int, const void*>, int64_t> cache;   // per device and kernel
+    static std::map<std::pair<int, const void*>, int64_t> cache;
     int dev = 0;
     cudaGetDevice(&dev);
     const auto key = std::make_pair(dev, (const void*)kern);
@@ -513,10 +717,13 @@ static int64_t prefetch_distance(KernT kern) {
         cudaGetLastError();
         per_sm = 0;
     }
-    const int64_t d = (int64_t)per_sm * num_sms() / 2;
-    cache[key] = d;
-    return d;
+    return cache[key] = (int64_t)per_sm * num_sms();
 }
+
+// Tiles half a wave ahead: half the CTAs resident at once on the device (measured at 2^20
+// segments: half a wave 3,452 GB/s, one wave 3,409, two waves 3,342, none 3,187).
+template <typename KernT>
+static int64_t prefetch_distance(KernT kern) { return resident_ctas(kern) / 2; }
 
 template <typename Tin, typename Tout>
 static accel_status run(int32_t op, int32_t map_op, const void* d_data, int64_t N, const int64_t* d_off,
@@ -546,6 +753,35 @@ static accel_status run(int32_t op, int32_t map_op, const void* d_data, int64_t 
         return after_launch(st, "accel_segreduce", 1);
     }
     int64_t te = tile_elems<Tin>();
+    if constexpr (std::is_integral<C>::value) {
+        // (many segments of a few elements: the partition and the tiles' prefix arrays)
+        if (op == ACCEL_RED_ADD && N >= 16 * S) {
+            auto stream = [&](auto kern) {
+                // Up to six ranges a CTA, one after the other from all over the data, so that a part of many
+                // tiny segments does not fall to a few CTAs; as many as leave the most loaded CTA with the
+                // fewest tiles.
+                const int64_t slots = std::max<int64_t>(resident_ctas(kern), 1);
+                int64_t per = 0, least = 0;
+                for (int64_t k = 1; k <= 6; ++k) {
+                    const int64_t c = (L.ntiles + slots * k - 1) / (slots * k), n = (L.ntiles + c - 1) / c;
+                    const int64_t most = (n + slots - 1) / slots * c;
+                    if (k == 1 || most <= least) {
+                        least = most;
+                        per = c;
+                    }
+                }
+                const int64_t ranges = (L.ntiles + per - 1) / per;
+                kern<<<(unsigned)std::min(ranges, slots), kThreads, 0, st>>>((const Tin*)d_data, N, d_off, S, per * te,
+                                                                             ranges, map_op, scalar, out, lo, tseg,
+                                                                             (int64_t*)tval);
+                k_fixup<Tout, ACCEL_RED_ADD><<<(unsigned)((ranges + 255) / 256), 256, 0, st>>>(d_off, lo, ranges, per * te,
+                                                                                              tseg, tval, out);
+            };
+            if (map_op == ACCEL_MAP_SQ_PLUS_ONE) stream(k_segsum_stream<Tin, Tout, true>);
+            else stream(k_segsum_stream<Tin, Tout, false>);
+            return after_launch(st, "accel_segreduce", 2);
+        }
+    }
     k_partition_scatter<<<(unsigned)((S + 1 + 255) / 256), 256, 0, st>>>(d_off, S, N, te, L.ntiles, lo);
     if constexpr (std::is_integral<C>::value) {
         if (op == ACCEL_RED_ADD) {
