@@ -547,6 +547,14 @@ accel_status pairwise_mapreduce(int32_t op, const float* d_x, const float* d_y, 
                                 const float* d_m, int64_t n, float eps, float* d_ax, float* d_ay,
                                 float* d_az, void* stream);
 
+/* The same with scratch space: with at least pairwise_mapreduce_workspace_size(op, n) bytes (16-byte
+ * aligned; 0: no use for any) each pair of bodies is evaluated once for both.  With less, or without, as
+ * pairwise_mapreduce.  The two forms add in different orders. */
+size_t pairwise_mapreduce_workspace_size(int32_t op, int64_t n);
+accel_status pairwise_mapreduce_ws(int32_t op, const float* d_x, const float* d_y, const float* d_z,
+                                   const float* d_m, int64_t n, float eps, float* d_ax, float* d_ay,
+                                   float* d_az, void* d_ws, size_t ws_bytes, void* stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -551,6 +551,14 @@ class HMMLogLik(torch.autograd.Function):
 
 
 # ------------------------------------------------------------------------- all-pairs
+def _optional_ws(need, device):
+    """Scratch space that a call does without if it has to."""
+    try:
+        return _ws(need, device) if need else None
+    except torch.OutOfMemoryError:
+        return None
+
+
 def pairwise_mapreduce(x, y, z, m, eps: float, op: int = L.PAIR_GRAVITY_SOFTENED, out=None):
     lib = L.load()
     _need_cuda(x, y, z, m)
@@ -558,6 +566,9 @@ def pairwise_mapreduce(x, y, z, m, eps: float, op: int = L.PAIR_GRAVITY_SOFTENED
     if out is None:
         out = tuple(torch.empty(n, dtype=torch.float32, device=x.device) for _ in range(3))
     ax, ay, az = out
-    L.check("pairwise_mapreduce", lib.pairwise_mapreduce(op, _ptr(x), _ptr(y), _ptr(z), _ptr(m), n, float(eps),
-                                                         _ptr(ax), _ptr(ay), _ptr(az), _stream()))
+    need = lib.pairwise_mapreduce_workspace_size(op, n)
+    ws = _optional_ws(need, x.device)
+    L.check("pairwise_mapreduce", lib.pairwise_mapreduce_ws(op, _ptr(x), _ptr(y), _ptr(z), _ptr(m), n, float(eps),
+                                                            _ptr(ax), _ptr(ay), _ptr(az), _ptr(ws),
+                                                            need if ws is not None else 0, _stream()))
     return ax, ay, az

@@ -194,6 +194,180 @@ accel_status launch_gravity(const float* d_x, const float* d_y, const float* d_z
     return after_launch(st, "pairwise_mapreduce", 1);
 }
 
+// ---------------------------------------------------------------- each pair of bodies once
+// With room for partial sums, d, r and r^(-3/2) of a pair serve both of its bodies: 16 FP32 operations
+// and one rsqrt for two interactions, instead of 24 and two.  A unit is 1,024 bodies I (a CTA of 8 warps
+// of 128, four bodies a lane) against 512 bodies J, J not before I; the units within I itself (J < I + 1,024)
+// take both directions one by one and give sums to I only.
+//  * A warp goes through the 64-body groups of J in turn, warp w starting at group w, with a barrier
+//    between turns, so that a group's sums have one writer at a time and a fixed order.
+//  * In a group, a lane holds the sums of two bodies of J (a packed pair), which move on by one lane after
+//    each of 32 steps; the bodies' coordinates are read from shared memory at the moving index.
+//  * Sums over I go to partial[unit], those over J to partial[I block]; k_pairs_sum adds a body's
+//    partial sums in a fixed order: results are deterministic for a given n.
+// What bounds it: the FP32 pipe (packed: 128 cycles for 4 x 2 pairs a lane, beside about 90 issue slots).
+// Against k_gravity, which evaluates both directions: n = 24,576 253 -> 193 us, 65,536 1,660 -> 1,155,
+// 131,072 6,598 -> 4,466; the error against 64 bits is about half as large (more, shorter sums).  From
+// kPairsMin on, where the units (594) give every SM two rounds of two CTAs; at 16,384 there is less than
+// one.  Up to kPairsMax: the partial sums grow as n^2 (385 MB there).
+constexpr int kPT = 256;
+constexpr int kPI = 1024, kPJ = 512;
+constexpr int64_t kPairsMin = 24576, kPairsMax = 131072;
+
+struct PairsPrm {
+    const float *X, *Y, *Z, *M;
+    int64_t n;
+    int ni, nj;              // blocks of I, of J
+    float eps2;
+    float *pi, *pj;          // [3][units][kPI], [3][ni][nj kPJ]
+    float *AX, *AY, *AZ;
+};
+
+// Units of the I blocks before i: sum of nj - 2 i'.
+__host__ __device__ __forceinline__ int units_before(int i, int nj) { return i * nj - i * (i - 1); }
+
+__global__ void __launch_bounds__(kPT, 2) k_pairs(PairsPrm p) {
+    __shared__ __align__(16) float4 s_xy[kPJ / 2], s_zm[kPJ / 2];   // pairs: (x, x', y, y'), (z, z', m, m')
+    __shared__ float2 s_a[3][kPJ / 2];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int u = blockIdx.x, units = units_before(p.ni, p.nj);
+    int lo = 0, hi = p.ni - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (units_before(mid, p.nj) <= u) lo = mid; else hi = mid - 1;
+    }
+    const int I = lo, J = 2 * I + u - units_before(I, p.nj);
+    const bool both = J >= 2 * (I + 1);
+    {
+        // bodies past the end sit at the origin with zero mass
+        const int64_t j = (int64_t)J * kPJ + 2 * t;
+        const bool in0 = j < p.n, in1 = j + 1 < p.n;
+        s_xy[t] = make_float4(in0 ? p.X[j] : 0.f, in1 ? p.X[j + 1] : 0.f, in0 ? p.Y[j] : 0.f, in1 ? p.Y[j + 1] : 0.f);
+        s_zm[t] = make_float4(in0 ? p.Z[j] : 0.f, in1 ? p.Z[j + 1] : 0.f, in0 ? p.M[j] : 0.f, in1 ? p.M[j + 1] : 0.f);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) s_a[c][t] = make_float2(0.f, 0.f);
+    }
+    float2 nx[4], ny[4], nz[4], nm[4], ax[4], ay[4], az[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int64_t i = (int64_t)I * kPI + w * 128 + k * 32 + lane;
+        const bool in = i < p.n;
+        const float x = in ? -p.X[i] : 0.f, y = in ? -p.Y[i] : 0.f, z = in ? -p.Z[i] : 0.f, m = in ? -p.M[i] : 0.f;
+        nx[k] = make_float2(x, x);
+        ny[k] = make_float2(y, y);
+        nz[k] = make_float2(z, z);
+        nm[k] = make_float2(m, m);
+        ax[k] = ay[k] = az[k] = make_float2(0.f, 0.f);
+    }
+    const float2 e2 = make_float2(p.eps2, p.eps2);
+    __syncthreads();
+    for (int turn = 0; turn < 8; ++turn) {
+        const int g = ((turn + w) & 7) * 32;      // the group's first pair
+        if (both) {
+            float2 bx = make_float2(0.f, 0.f), by = bx, bz = bx;
+#pragma unroll 2
+            for (int step = 0; step < 32; ++step) {
+                const int q = g + ((lane + step) & 31);
+                const float4 xy = s_xy[q], zm = s_zm[q];
+                const float2 xj = make_float2(xy.x, xy.y), yj = make_float2(xy.z, xy.w), zj = make_float2(zm.x, zm.y),
+                             mj = make_float2(zm.z, zm.w);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float2 dx = __fadd2_rn(xj, nx[k]), dy = __fadd2_rn(yj, ny[k]), dz = __fadd2_rn(zj, nz[k]);
+                    float2 r = __ffma2_rn(dz, dz, e2);
+                    r = __ffma2_rn(dy, dy, r);
+                    r = __ffma2_rn(dx, dx, r);
+                    const float2 inv = make_float2(rsqrt_ftz(r.x), rsqrt_ftz(r.y));
+                    const float2 c3 = __fmul2_rn(__fmul2_rn(inv, inv), inv);
+                    const float2 si = __fmul2_rn(c3, mj), sj = __fmul2_rn(c3, nm[k]);
+                    ax[k] = __ffma2_rn(si, dx, ax[k]);
+                    ay[k] = __ffma2_rn(si, dy, ay[k]);
+                    az[k] = __ffma2_rn(si, dz, az[k]);
+                    bx = __ffma2_rn(sj, dx, bx);
+                    by = __ffma2_rn(sj, dy, by);
+                    bz = __ffma2_rn(sj, dz, bz);
+                }
+                // the sums move on with their bodies
+                const int from = (lane + 1) & 31;
+                bx = make_float2(__shfl_sync(0xffffffffu, bx.x, from), __shfl_sync(0xffffffffu, bx.y, from));
+                by = make_float2(__shfl_sync(0xffffffffu, by.x, from), __shfl_sync(0xffffffffu, by.y, from));
+                bz = make_float2(__shfl_sync(0xffffffffu, bz.x, from), __shfl_sync(0xffffffffu, bz.y, from));
+            }
+            const float2 sx = s_a[0][g + lane], sy = s_a[1][g + lane], sz = s_a[2][g + lane];
+            s_a[0][g + lane] = make_float2(sx.x + bx.x, sx.y + bx.y);
+            s_a[1][g + lane] = make_float2(sy.x + by.x, sy.y + by.y);
+            s_a[2][g + lane] = make_float2(sz.x + bz.x, sz.y + bz.y);
+        } else {
+#pragma unroll 2
+            for (int step = 0; step < 32; ++step) {
+                const float4 xy = s_xy[g + step], zm = s_zm[g + step];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    interact2(make_float2(xy.x, xy.y), make_float2(xy.z, xy.w), make_float2(zm.x, zm.y),
+                              make_float2(zm.z, zm.w), nx[k], ny[k], nz[k], e2, ax[k], ay[k], az[k]);
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        float* at = p.pi + (int64_t)u * kPI + w * 128 + k * 32 + lane;
+        const int64_t plane = (int64_t)units * kPI;
+        at[0] = ax[k].x + ax[k].y;
+        at[plane] = ay[k].x + ay[k].y;
+        at[2 * plane] = az[k].x + az[k].y;
+    }
+    if (both) {
+        const int64_t row = (int64_t)p.nj * kPJ, plane = p.ni * row;
+        float* at = p.pj + I * row + (int64_t)J * kPJ + 2 * t;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) *reinterpret_cast<float2*>(at + c * plane) = s_a[c][t];
+    }
+}
+
+// A body's sums: over the units of its I block, then over the I blocks before it.
+__global__ void __launch_bounds__(256) k_pairs_sum(PairsPrm p) {
+    const int64_t b = blockIdx.x * (int64_t)256 + threadIdx.x;
+    if (b >= p.n) return;
+    const int I = (int)(b / kPI), u0 = units_before(I, p.nj), nu = p.nj - 2 * I;
+    const int64_t pl_i = (int64_t)units_before(p.ni, p.nj) * kPI, row = (int64_t)p.nj * kPJ, pl_j = p.ni * row;
+    float* const out[3] = {p.AX, p.AY, p.AZ};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const float* fi = p.pi + c * pl_i + (int64_t)u0 * kPI + b % kPI;
+        const float* fj = p.pj + c * pl_j + b;
+        float a[8] = {};                      // (eight sums, added in pairs: fewer roundings)
+        auto add = [&](const float* f, int n, int64_t stride) {
+            int q = 0;
+            for (; q + 8 <= n; q += 8)
+#pragma unroll
+                for (int k = 0; k < 8; ++k) a[k] += f[(q + k) * stride];
+            for (; q < n; ++q) a[0] += f[q * stride];
+        };
+        add(fi, nu, kPI);
+        add(fj, I, row);
+        out[c][b] = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+    }
+}
+
+size_t pairs_ws(int64_t n) {
+    if (n < kPairsMin || n > kPairsMax) return 0;
+    const int64_t ni = (n + kPI - 1) / kPI, nj = (n + kPJ - 1) / kPJ;
+    return (size_t)(3 * (units_before((int)ni, (int)nj) * (int64_t)kPI + ni * nj * kPJ)) * sizeof(float);
+}
+
+accel_status launch_pairs(const float* d_x, const float* d_y, const float* d_z, const float* d_m, int64_t n, float eps,
+                          float* d_ax, float* d_ay, float* d_az, void* ws, cudaStream_t st) {
+    PairsPrm p{d_x, d_y, d_z, d_m, n, (int)((n + kPI - 1) / kPI), (int)((n + kPJ - 1) / kPJ), eps * eps,
+               nullptr, nullptr, d_ax, d_ay, d_az};
+    const int units = units_before(p.ni, p.nj);
+    p.pi = (float*)ws;
+    p.pj = p.pi + 3 * (int64_t)units * kPI;
+    k_pairs<<<units, kPT, 0, st>>>(p);
+    k_pairs_sum<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p);
+    return after_launch(st, "pairwise_mapreduce", 2);
+}
+
 }  // namespace pair
 }  // namespace accel
 
@@ -201,8 +375,18 @@ using namespace accel;
 
 extern "C" {
 
+size_t pairwise_mapreduce_workspace_size(int32_t op, int64_t n) {
+    return op == ACCEL_PAIR_GRAVITY_SOFTENED ? pair::pairs_ws(n) : 0;
+}
+
 accel_status pairwise_mapreduce(int32_t op, const float* d_x, const float* d_y, const float* d_z, const float* d_m,
                                 int64_t n, float eps, float* d_ax, float* d_ay, float* d_az, void* stream) {
+    return pairwise_mapreduce_ws(op, d_x, d_y, d_z, d_m, n, eps, d_ax, d_ay, d_az, nullptr, 0, stream);
+}
+
+accel_status pairwise_mapreduce_ws(int32_t op, const float* d_x, const float* d_y, const float* d_z, const float* d_m,
+                                   int64_t n, float eps, float* d_ax, float* d_ay, float* d_az, void* d_ws,
+                                   size_t ws_bytes, void* stream) {
     ACCEL_REQUIRE(op == ACCEL_PAIR_GRAVITY_SOFTENED, ACCEL_ERR_INVALID_ARG, "pairwise_mapreduce: bad op %d", op);
     ACCEL_REQUIRE(n >= 0, ACCEL_ERR_INVALID_ARG, "pairwise_mapreduce: n < 0");
     // the j = i term (and a padding body's) is 0 * r^(-3/2) with r >= eps^2: it stays 0 only
@@ -214,6 +398,10 @@ accel_status pairwise_mapreduce(int32_t op, const float* d_x, const float* d_y, 
     ACCEL_REQUIRE(d_x && d_y && d_z && d_m && d_ax && d_ay && d_az, ACCEL_ERR_INVALID_ARG, "pairwise_mapreduce: null pointer");
     ACCEL_REQUIRE((n + pair::kBodies - 1) / pair::kBodies * pair::kMaxCluster <= (int64_t)INT32_MAX,
                   ACCEL_ERR_UNSUPPORTED, "pairwise_mapreduce: n too large");
+    ACCEL_REQUIRE(((uintptr_t)d_ws % 16) == 0, ACCEL_ERR_INVALID_ARG, "pairwise_mapreduce: d_ws must be 16-byte aligned");
+    const size_t need = pair::pairs_ws(n);
+    if (d_ws && need > 0 && ws_bytes >= need)
+        return pair::launch_pairs(d_x, d_y, d_z, d_m, n, eps, d_ax, d_ay, d_az, d_ws, as_stream(stream));
     return pair::launch_gravity(d_x, d_y, d_z, d_m, n, eps, d_ax, d_ay, d_az, pair::choose_cluster(n),
                                 as_stream(stream));
 }
