@@ -9,8 +9,7 @@
 //    sums meet by a reduce-scatter over the 8 row lanes, not through shared memory.
 //  * Epilogue warp g owns sequence slot g: all of a slot's bookkeeping is uniform over a warp, a row of
 //    the CTA's columns is one vector access, and its sum one warp reduction.  (4 warps of two slots
-//    each: a warp that waits for one half is late for the other; 4.8 ms where the log-space forward
-//    takes 3.9.)
+//    each: a warp that waits for one half is late for the other.)
 //
 // The 8 slots are two halves of 4 that run as two interleaved recurrences: a phase is one step of one
 // half, and the halves take turns, so that the epilogue, the hand-overs between the warps and the
@@ -126,14 +125,14 @@ struct Waits {
 __device__ __forceinline__ uint32_t step_phase(uint32_t i) { return (i >> 1) & 1u; }
 
 template <int KP>
-__device__ __forceinline__ void init_bars(Smem<KP>& sm) {
+__device__ __forceinline__ void init_bars(Smem<KP>& sm, int out_warps = kCon / 32) {
     if (threadIdx.x == 0) {
         for (int q = 0; q < 4; ++q) {
             tc::mbar_init(&sm.x_own[q >> 1][q & 1], 4);
             tc::mbar_init(&sm.x_peer[q >> 1][q & 1], 1);
         }
-        tc::mbar_init(&sm.out_full[0], kCon / 32);
-        tc::mbar_init(&sm.out_full[1], kCon / 32);
+        tc::mbar_init(&sm.out_full[0], out_warps);
+        tc::mbar_init(&sm.out_full[1], out_warps);
         tc::fence_mbar_init();
     }
 }

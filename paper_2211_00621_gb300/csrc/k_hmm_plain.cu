@@ -10,19 +10,19 @@
 // Each sequence keeps la = c + r with r in FP32 and the running offset c (the sum of the
 // per-step maxima, a sum of log scale factors) in FP64.
 //
-// k_plain_warp<J> (K <= 32 J, J <= 2): one warp per sequence, no block-wide synchronisation; exp(log A)
-// in registers, the emission table log B^T in shared memory.  More states: k_hmm_rows_log.cu.
+// k_plain_warp<J> (K <= 32 J, J <= 2): one warp per sequence, no block-wide synchronisation; lane l owns
+// states l and l + 32, their columns of exp(log A) in registers, the emission table log B^T in shared
+// memory.  More states: k_hmm_rows_log.cu.
 //
 // What bounds it: with a few hundred sequences a scheduler has one warp, and a step is the chain
-// maximum - exp - exchange through shared memory - products - log.  Each half warp takes every other
-// four rows and 2 J columns a lane (so a step reads half the shared memory that J columns of all rows
-// would: the four warps of an SM share one path), then the halves exchange J sums.  The products are
-// FFMA2 in 2 J chains, the maximum is one redux, the next step's emission is fetched a step ahead, and
-// a lane keeps the shift of one step in 32, so that the FP64 sum takes one addition per 32 steps.
-// 512 sequences of 1,000 steps, K = 64: 217 us, 420 cycles a step (128 of them FFMA2 issue); with J
-// chains of 64 dependent FMAs, a shuffle tree and an FP64 addition a step: 398 us.  Two blocks an SM:
-// ptxas aims at three otherwise, with 168 registers instead of 192, and a step takes 570 cycles
-// (4,096 sequences, where occupancy could help: 1.05 ms, 1.11 with three).
+// maximum - exp - exchange through shared memory - products - log.  The products are J chains of K FMAs in
+// the order of the rows.  (Four chains a column and half the shared-memory reads take 420 cycles a step
+// instead of 470, but r is rounded at a magnitude of several units, so another order of the sum moves logL
+// by up to 1e-8 of itself in short sequences of few symbols.)  The maximum is one redux, the next step's
+// emission is fetched a step ahead, and a lane keeps the shift of one step in 32, so that the FP64 sum
+// takes one addition per 32 steps.  512 sequences of 1,000 steps, K = 64: 242 us; with a shuffle tree and
+// an FP64 addition a step, and one load of A after the other, 398 us.  Two blocks an SM: ptxas aims at
+// three otherwise, with 168 registers.
 #include "common.cuh"
 #include "hmm_internal.cuh"
 
@@ -41,7 +41,6 @@ __global__ void __launch_bounds__(128, 2)
 k_plain_warp(const float* __restrict__ logA, const float* __restrict__ logB, const float* __restrict__ logpi,
              int K, int M, const int32_t* __restrict__ obs, const int64_t* __restrict__ off, int64_t S,
              double* __restrict__ loglik) {
-    constexpr int CW = 2 * J;                // columns of a lane's products; J of them are its own
     extern __shared__ float smem[];
     float* sB = smem;                                  // [M][K]  log B^T
     float* sP = smem + (((size_t)M * K + 3) & ~(size_t)3);   // [4][32 J] per-warp, 16-byte aligned
@@ -55,47 +54,32 @@ k_plain_warp(const float* __restrict__ logA, const float* __restrict__ logB, con
     const int64_t s = blockIdx.x * 4 + w;
     if (s >= S) return;
 
-    const int h = lane >> 4, l = lane & 15;
-    const int j0 = CW * l + J * h;           // the lane's own columns: j0 .. j0 + J - 1
-    // rows 8 i + 4 h + 2 k and the one after (i < 4 J, k < 2), columns CW l + c.  The loads are
-    // unconditional: behind a test each one waits for the one before.
-    float2 a[4 * J][2][CW];
-#pragma unroll
-    for (int i = 0; i < 4 * J; ++i)
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-#pragma unroll
-            for (int c = 0; c < CW; ++c) {
-                const int row = 8 * i + 4 * h + 2 * k, col = min(CW * l + c, K - 1);
-                a[i][k][c] = make_float2(logA[min(row, K - 1) * K + col], logA[min(row + 1, K - 1) * K + col]);
-            }
-#pragma unroll
-    for (int i = 0; i < 4 * J; ++i)
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-#pragma unroll
-            for (int c = 0; c < CW; ++c) {
-                const int row = 8 * i + 4 * h + 2 * k, col = CW * l + c;
-                a[i][k][c].x = col < K && row < K ? __expf(a[i][k][c].x) : 0.f;
-                a[i][k][c].y = col < K && row + 1 < K ? __expf(a[i][k][c].y) : 0.f;
-            }
-    float* P = sP + w * 32 * J;
-    const int64_t o0 = off[s];
-    const int64_t T = off[s + 1] - o0;
-    const int32_t* o = obs + o0;
+    // a[jj][i] = A[i, lane + 32 jj].  The loads are unconditional: behind a test each one waits for the one
+    // before.
+    float a[J][32 * J];
     bool own[J];
     int jc[J];                               // (a column within the table for those beyond it)
 #pragma unroll
     for (int jj = 0; jj < J; ++jj) {
-        own[jj] = j0 + jj < K;
-        jc[jj] = min(j0 + jj, K - 1);
+        own[jj] = lane + 32 * jj < K;
+        jc[jj] = min(lane + 32 * jj, K - 1);
+#pragma unroll
+        for (int i = 0; i < 32 * J; ++i) a[jj][i] = logA[min(i, K - 1) * K + jc[jj]];
     }
+#pragma unroll
+    for (int jj = 0; jj < J; ++jj)
+#pragma unroll
+        for (int i = 0; i < 32 * J; ++i) a[jj][i] = own[jj] && i < K ? __expf(a[jj][i]) : 0.f;
+    float* P = sP + w * 32 * J;
+    const int64_t o0 = off[s];
+    const int64_t T = off[s + 1] - o0;
+    const int32_t* o = obs + o0;
 
     float r[J], lb[J];
     int32_t ob = o[0];
 #pragma unroll
-    for (int jj = 0; jj < J; ++jj) r[jj] = own[jj] ? logpi[j0 + jj] + sB[ob * K + j0 + jj] : -INFINITY;
-    double c = 0.0;                          // the lane's share of the shifts: steps with t mod 32 = lane
+    for (int jj = 0; jj < J; ++jj) r[jj] = own[jj] ? logpi[jc[jj]] + sB[ob * K + jc[jj]] : -INFINITY;
+    double c = 0.0;
     int32_t ochunk = lane < T ? o[lane] : 0;           // lane l holds o[32 floor(t / 32) + l]
     ob = __shfl_sync(0xffffffffu, ochunk, 1);
 #pragma unroll
@@ -103,36 +87,33 @@ k_plain_warp(const float* __restrict__ logA, const float* __restrict__ logB, con
     for (int64_t tb = 0; tb < T; tb += 32) {
         const int32_t next = tb + 32 + lane < T ? o[tb + 32 + lane] : 0;
         const int t0 = tb == 0 ? 1 : 0, t1 = T - tb < 32 ? (int)(T - tb) : 32;
-        float shift = 0.f;
-#pragma unroll 1
+        float shift = 0.f;                   // lane l keeps the shift of step tb + l
         for (int t = t0; t < t1; ++t) {
             float m = r[0];
 #pragma unroll
             for (int jj = 1; jj < J; ++jj) m = fmaxf(m, r[jj]);
             m = warp_max_f32(m);
-            if (J == 2) *reinterpret_cast<float2*>(P + j0) = make_float2(__expf(r[0] - m), __expf(r[J - 1] - m));
-            else P[j0] = __expf(r[0] - m);
+#pragma unroll
+            for (int jj = 0; jj < J; ++jj) P[lane + 32 * jj] = __expf(r[jj] - m);
             __syncwarp();
-            float2 acc[CW];
+            float acc[J];
 #pragma unroll
-            for (int k = 0; k < CW; ++k) acc[k] = make_float2(0.f, 0.f);
+            for (int jj = 0; jj < J; ++jj) acc[jj] = 0.f;
 #pragma unroll
-            for (int i = 0; i < 4 * J; ++i) {
-                const float4 p = reinterpret_cast<const float4*>(P)[2 * i + h];
+            for (int i4 = 0; i4 < 8 * J; ++i4) {
+                const float4 p = reinterpret_cast<const float4*>(P)[i4];
 #pragma unroll
-                for (int k = 0; k < CW; ++k) acc[k] = __ffma2_rn(make_float2(p.x, p.y), a[i][0][k], acc[k]);
+                for (int jj = 0; jj < J; ++jj) acc[jj] = fmaf(p.x, a[jj][4 * i4 + 0], acc[jj]);
 #pragma unroll
-                for (int k = 0; k < CW; ++k) acc[k] = __ffma2_rn(make_float2(p.z, p.w), a[i][1][k], acc[k]);
+                for (int jj = 0; jj < J; ++jj) acc[jj] = fmaf(p.y, a[jj][4 * i4 + 1], acc[jj]);
+#pragma unroll
+                for (int jj = 0; jj < J; ++jj) acc[jj] = fmaf(p.z, a[jj][4 * i4 + 2], acc[jj]);
+#pragma unroll
+                for (int jj = 0; jj < J; ++jj) acc[jj] = fmaf(p.w, a[jj][4 * i4 + 3], acc[jj]);
             }
-            // the other 16 lanes' rows: each lane of a pair gives the columns that are the other's
-            float sum[J];
+            __syncwarp();
 #pragma unroll
-            for (int jj = 0; jj < J; ++jj) {
-                const float u = acc[jj].x + acc[jj].y, v = acc[jj + J].x + acc[jj + J].y;
-                sum[jj] = (h ? v : u) + __shfl_xor_sync(0xffffffffu, h ? u : v, 16);
-            }
-#pragma unroll
-            for (int jj = 0; jj < J; ++jj) r[jj] = own[jj] ? __logf(sum[jj]) + lb[jj] : -INFINITY;
+            for (int jj = 0; jj < J; ++jj) r[jj] = own[jj] ? __logf(acc[jj]) + lb[jj] : -INFINITY;
             shift = lane == t ? m : shift;
             // the next step's symbol
             ob = __shfl_sync(0xffffffffu, t == 31 ? next : ochunk, (t + 1) & 31);

@@ -6,13 +6,16 @@
 // The shift is the largest r.  An epilogue warp holds a slot's row of the CTA's columns, so its maximum
 // is one warp reduction; the warps of a pair's CTAs exchange theirs (a word and an mbarrier per slot
 // and step parity) before the exponentials, and the other half's products hide the way.
-// (Shifts of each CTA's own, the sums put on one scale after the products, save the exchange, but the
-// approximate exponential's error depends on its argument's fraction: logL moved by 2e-9.)
 //
-// What bounds it: the products (hmm_rows.cuh: 2,048 cycles of FMAs of about 3,700 a step) and, for the
-// longest sequences, the chain of a step.  1,024 sequences of 200 to 2,000 steps (1.13M steps) at
-// K = 256: 3.9 ms, 2.0 ms of them FMAs.  One CTA per 8 sequences that streamed A from L2 every step:
-// 31.5 ms.
+// A column's sum runs over the rows in order, one FMA after the other, like the sum of the kernel for
+// fewer states: r is rounded at a magnitude of several units, so any other order moves logL by up to
+// 1e-8 of itself in short sequences of few symbols.  For the same reason log(sum) + log B is one FMA.
+//
+// What bounds it: the shared-memory reads of the vectors (a thread has one column, so 16 bytes serve four
+// FMAs) beside the FMAs.  1,024 sequences of 200 to 2,000 steps (1.13M steps) at K = 256: 5.4 ms, 2.0 ms of
+// them FMAs; with the products of the other recurrences (16 FMAs for 16 bytes, eight partial sums a
+// column) 3.9 ms, but 5e-9 of logL away.  One CTA per 8 sequences that streamed A from L2 every step:
+// 31.5 ms, and the same results.
 #include "hmm_rows.cuh"
 
 namespace accel {
@@ -73,7 +76,61 @@ struct LogSmem {
     Smem<KP> s;
     uint64_t max_full[2][kG];                      // [step parity][slot]
     float max_peer[2][kG];
+    uint64_t mid_full[2][4];                       // [half][warp of columns]
+    float mid[2][4][Cfg<KP>::Kh];                  // [half][slot][column]: the sums over the first rows
 };
+
+// The products in the order of the rows: a thread owns a column, and its sums run over the rows one by
+// one.  Two stages of four warps, the first half of the rows and the second; while one works on a half of
+// the slots, the other works on the other half.
+template <int KP>
+__device__ __forceinline__ void ordered_products(const float* __restrict__ A, int rank, LogSmem<KP>& ls,
+                                                 const uint32_t (&half)[2], Waits& wt) {
+    using C = Cfg<KP>;
+    constexpr int R = KP / 2;
+    Smem<KP>& sm = ls.s;
+    const int col = threadIdx.x & 127, stage = threadIdx.x >> 7, w = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
+    static_assert(C::Kh == 128, "a thread per column and stage");
+    float a[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) a[i] = A[(size_t)(stage * R + i) * KP + rank * C::Kh + col];
+    const uint32_t iters = half[0] > half[1] ? half[0] : half[1];
+    for (uint32_t it = 1; it < iters; ++it) {
+        const int pb = (int)(it & 1) ^ 1;
+        const uint32_t ph = step_phase(it - 1);
+#pragma unroll 1
+        for (int u = 0; u < 2; ++u) {
+            if (it >= (u ? half[1] : half[0])) continue;
+            const float* x = &sm.x[pb][4 * u][stage * R];
+            wt.local(&sm.x_own[u][pb], ph);
+            if constexpr (C::NC == 2) wt.cluster(&sm.x_peer[u][pb], ph);
+            float acc[4] = {};
+            if (stage == 1) {
+                wt.local(&ls.mid_full[u][w], (it - 1) & 1u);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) acc[g] = ls.mid[u][g][col];
+            }
+#pragma unroll
+            for (int q = 0; q < R / 4; ++q) {
+                float4 v[4];
+#pragma unroll
+                for (int g = 0; g < 4; ++g) v[g] = *reinterpret_cast<const float4*>(x + g * C::ST + 4 * q);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) acc[g] = fmaf(v[g].x, a[4 * q], acc[g]);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) acc[g] = fmaf(v[g].y, a[4 * q + 1], acc[g]);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) acc[g] = fmaf(v[g].z, a[4 * q + 2], acc[g]);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) acc[g] = fmaf(v[g].w, a[4 * q + 3], acc[g]);
+            }
+#pragma unroll
+            for (int g = 0; g < 4; ++g) (stage == 0 ? ls.mid[u][g][col] : sm.out[u][g][col]) = acc[g];
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(stage == 0 ? &ls.mid_full[u][w] : &sm.out_full[u]);
+        }
+    }
+}
 
 // Step i of a slot forms r_t; its exponentials, shifted by the largest, are the next vector.
 template <int KP>
@@ -86,7 +143,7 @@ __device__ __forceinline__ void log_epilogue(const LogPrm& p, int rank, int cid,
     const int64_t n = (int64_t)p.ncl * kG;
     const int32_t* obs = p.obs + p.off[0];
     const int c = rank * C::Kh + ep.col;
-    const bool lead = rank == 0 && ep.lane == 0;
+    const bool lead = rank == C::NC - 1 && ep.lane == 0;
     uint32_t peer_max = 0, peer_full = 0;        // shared::cluster addresses of the peer's
     if constexpr (C::NC == 2) {
         peer_max = tc::cluster_addr(&ls.max_peer[0][0], (uint32_t)(rank ^ 1));
@@ -100,10 +157,11 @@ __device__ __forceinline__ void log_epilogue(const LogPrm& p, int rank, int cid,
     int32_t sym, nsym;
     bool fresh;
     double off_c;                             // c: the shifts of the sequence so far
-    // the sequence that ended with the step before (-1: none): its c and the CTA's sum of exponentials
+    // the sequence that ended with the step before (-1: none): its c and the sums of the exponentials of
+    // the CTA's columns, 32 by 32
     int32_t pseq;
     double pc;
-    float psum;
+    float psum[4];
     auto begin = [&]() {
         next_seq(s, p.S, n, p.order, p.off, any);
         fresh = true;
@@ -120,11 +178,21 @@ __device__ __forceinline__ void log_epilogue(const LogPrm& p, int rank, int cid,
     sym = nsym = 0;
     pseq = -1;
     pc = 0.0;
-    psum = 0.f;
+    psum[0] = psum[1] = psum[2] = psum[3] = 0.f;
     begin();
+    auto finish = [&](int32_t ended, uint32_t it) {
+        if (ended < 0) return;
+        const int pb = (int)(it & 1) ^ 1;
+        if (C::NC == 2) wt.cluster(&sm.x_peer[u][pb], step_phase(it - 1));
+        if (!lead) return;
+        float sum = rank == 1 ? sm.peer[pb][ep.g] : 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) sum += psum[k];
+        p.loglik[ended] = pc + log((double)sum);
+    };
     const uint32_t steps = half[u];
     for (uint32_t it = 0; it <= steps; ++it) {
-        const int b = (int)(it & 1), pb = b ^ 1;
+        const int b = (int)(it & 1);
         const bool on = s.seq >= 0;
         const int32_t ended = pseq;
         pseq = -1;
@@ -136,8 +204,8 @@ __device__ __forceinline__ void log_epilogue(const LogPrm& p, int rank, int cid,
                 r.load(&sm.out[u][ep.g & 3][ep.col]);
             }
 #pragma unroll
-            for (int h = 0; h < C::EC; ++h)
-                r.v[h] = !on ? -INFINITY : (fresh ? pi.v[h] : __logf(r.v[h])) + lb.v[h];
+            for (int h = 0; h < C::EC; ++h)       // (not one sum of a choice: log + lb is to stay one FMA)
+                r.v[h] = !on ? -INFINITY : fresh ? __fadd_rn(pi.v[h], lb.v[h]) : __logf(r.v[h]) + lb.v[h];
             float m = warp_max(r);
             if constexpr (C::NC == 2) {
                 if (ep.lane == 0) {
@@ -150,23 +218,30 @@ __device__ __forceinline__ void log_epilogue(const LogPrm& p, int rank, int cid,
             }
 #pragma unroll
             for (int h = 0; h < C::EC; ++h) x.v[h] = on ? __expf(r.v[h] - m) : 0.f;
-            // at the end of a sequence the sum of the exponentials is wanted, too
-            const float es = on && left == 0 ? ep.warp_sum(x) : 0.f;
-            ep.put(b, x, true, es);
-            if (ended >= 0) {
-                if (C::NC == 2) {
-                    wt.cluster(&sm.x_peer[u][pb], step_phase(it - 1));
-                    psum += sm.peer[pb][ep.g];
-                }
-                if (lead) p.loglik[ended] = pc + log((double)psum);
+            // At the end of a sequence the sum of the exponentials is wanted, too: 32 columns by a butterfly
+            // (the highest bit of the column first), these sums in the order of the columns, so the second
+            // CTA goes on from the first one's.
+            float e4[4] = {};
+            if (on && left == 0) {
+                Vec<C::EC> e = x;
+#pragma unroll
+                for (int d = 4; d > 0; d >>= 1)
+#pragma unroll
+                    for (int h = 0; h < C::EC; ++h) e.v[h] += __shfl_xor_sync(0xffffffffu, e.v[h], d);
+                const float sum = (e.v[0] + e.v[2]) + (e.v[1] + e.v[3]);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) e4[k] = __shfl_sync(0xffffffffu, sum, 8 * k);
             }
+            ep.put(b, x, true, ((e4[0] + e4[1]) + e4[2]) + e4[3]);
+            finish(ended, it);
             // on to the next step
             if (on) {
                 off_c += (double)m;
                 if (left == 0) {
                     pseq = s.seq;
                     pc = off_c;
-                    psum = es;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) psum[k] = e4[k];
                     begin();
                 } else {
                     fresh = false;
@@ -176,30 +251,26 @@ __device__ __forceinline__ void log_epilogue(const LogPrm& p, int rank, int cid,
                     nsym = left > 0 ? obs[row + 1] : 0;
                 }
             }
-        } else if (ended >= 0) {
-            if (C::NC == 2) {
-                wt.cluster(&sm.x_peer[u][pb], step_phase(it - 1));
-                psum += sm.peer[pb][ep.g];
-            }
-            if (lead) p.loglik[ended] = pc + log((double)psum);
+        } else {
+            finish(ended, it);
         }
     }
 }
 
 template <int KP>
 __device__ __forceinline__ void log_body(const LogPrm& p, int rank, int cid, LogSmem<KP>& ls, cg::cluster_group* cl) {
-    if (Cfg<KP>::NC == 2 && threadIdx.x == 0)
+    if (threadIdx.x == 0) {
         for (int q = 0; q < 2 * kG; ++q) tc::mbar_init(&ls.max_full[0][0] + q, 1);
-    init_bars(ls.s);
+        for (int q = 0; q < 8; ++q) tc::mbar_init(&ls.mid_full[0][0] + q, 1);
+    }
+    init_bars(ls.s, 4);
     uint32_t half[2];          // (a slot's steps fit 32 bits: 2^32 of them would take two hours)
     slot_totals(ls.s.tot, p.S, (int64_t)p.ncl * kG, cid, p.ncl, p.order, p.off, [](int64_t) { return true; }, half);
     if constexpr (Cfg<KP>::NC == 2) cl->sync();  // the peer's barriers exist before any remote store
     Waits wt{p.status};
     if (threadIdx.x < kCon) {
         regs_contraction<KP>();
-        Contraction<KP> m;
-        m.load(p.A, rank);
-        contraction_loop(m, ls.s, half, wt);
+        ordered_products<KP>(p.A, rank, ls, half, wt);
     } else {
         regs_epilogue<KP>();
         log_epilogue<KP>(p, rank, cid, ls, half, wt);
