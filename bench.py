@@ -238,19 +238,17 @@ class Workload:
     # one step, device-resident inputs.  With `ev` (per-row (start, end) events) the rows run one
     # after another on the current stream, so each row's time is its own.  Without it the
     # step overlaps independent rows: the batched BF16 forward -- a latency-bound persistent
-    # launch whose CTAs fill the register files of the SMs they hold and leave the others
-    # idle -- runs on a second stream; the adjoint's forward phase runs on a third within the
+    # launch -- runs on a second stream; the adjoint's forward phase runs on a third within the
     # SMs the BF16 launch leaves (accel_set_sm_budget), and the seg-reduce, plain FP32 and
     # all-pairs rows on the main stream take what is free; the adjoint's backward rounds and
     # the re-estimation, which want every SM, follow.
     def adj_budget(self):
         """SMs for the adjoint's forward phase in the step: those the BF16 forward's persistent
-        clusters leave, less a tenth of the device for the rows that run beside them (measured
-        at 152 SMs: budgets 94 / 86 / 78 / 70 gave steps of 19.70 / 19.60 / 19.45 / 19.67 ms)."""
+        CTAs leave, less a tenth of the device for the rows that run beside them; 0 (no limit: its
+        clusters start as SMs come free) if that is less than half of the device."""
         units = (self.tuned or {}).get("units", 0)
-        nc = 2 if (self.tuned or {}).get("pair", 0) == 1 else 4 if (self.tuned or {}).get("pair", 0) == 2 else 1
-        free = self.n_sms - units * nc - self.n_sms // 10
-        return free if units > 0 and free > 0 else 0
+        free = self.n_sms - units - self.n_sms // 10
+        return free if units > 0 and free >= self.n_sms // 2 else 0
 
     def adj_forward_side(self, cur, adj_inputs):
         """The adjoint's forward phase on the third stream within the free SMs; returns
@@ -333,7 +331,7 @@ class Workload:
             a = self.adj
 
             def adjoint():
-                # one pass: the adjoint's checkpointed forward returns logL, then the backward
+                # one pass: the adjoint's forward returns logL, then the backward
                 return api.hmm_adjoint(a["log_A"], a["log_B"], a["log_pi"], a["obs"], a["offsets"],
                                        max_T=a["maxT"], want_loglik=True)
             if overlap:
@@ -478,12 +476,11 @@ def rooflines(W, row_ms, peaks, fp32_peak):
                           "peak": peaks["hbm_gbs"], "unit": "GB/s"}
     if W.adj is not None and "hmm_adjoint" in row_ms:
         a = W.adj
-        # 8 K^2 flop per time step: the forward, the checkpoint recomputation, the backward
-        # recursion and the xi accumulation, 2 K^2 each (6 K^2 without the recomputation)
+        # 6 K^2 flop per time step: the forward, the backward recursion and the xi accumulation,
+        # 2 K^2 each (every alpha is kept, so nothing is recomputed)
         sec = row_ms["hmm_adjoint"] * 1e-3
-        r["hmm_adjoint"] = {"bound": "alu", "achieved": 8 * a["K"] ** 2 * a["sumT"] / sec / 1e12,
-                            "peak": fp32_peak, "unit": "TFLOP/s", "flop_per_step": "8 K^2",
-                            "achieved_6K2": 6 * a["K"] ** 2 * a["sumT"] / sec / 1e12}
+        r["hmm_adjoint"] = {"bound": "alu", "achieved": 6 * a["K"] ** 2 * a["sumT"] / sec / 1e12,
+                            "peak": fp32_peak, "unit": "TFLOP/s", "flop_per_step": "6 K^2"}
     r["allpairs"] = {"bound": "alu", "achieved": 20.0 * W.N * W.N / (row_ms["allpairs"] * 1e-3) / 1e12,
                      "peak": fp32_peak, "unit": "TFLOP/s"}
     for v in r.values():
