@@ -103,6 +103,8 @@ _lock = threading.Lock()
 def load(path: str = LIB_PATH):
     """Load libaccel.so and declare its signatures (once)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib

@@ -21,12 +21,19 @@ _DT = {torch.int32: L.I32, torch.int64: L.I64, torch.float32: L.F32, torch.float
 _TORCH = {v: k for k, v in _DT.items()}
 
 
+# The current stream's handle.  A small call's time is its host work: the raw handle is had without
+# a Stream object (2 us), and integers go to ctypes as they are, without a c_void_p each.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _ptr(t):
-    return C.c_void_p(t.data_ptr()) if t is not None else C.c_void_p(0)
+    return t.data_ptr() if t is not None else None
 
 
 def _dt(t_or_dtype):
@@ -275,8 +282,8 @@ def _tensor_desc(t: torch.Tensor):
     d.data = t.data_ptr()
     d.dtype = _dt(t)
     d.rank = t.dim()
-    for i in range(min(t.dim(), L.MAX_RANK)):
-        d.dims[i] = t.shape[i]
+    for i, n in enumerate(t.shape[:L.MAX_RANK]):
+        d.dims[i] = n
     return d
 
 
