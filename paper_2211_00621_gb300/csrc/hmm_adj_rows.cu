@@ -89,7 +89,7 @@ template <int KP>
 __device__ __forceinline__ void fwd_epilogue(const RowsPrm& p, int rank, int cid, Smem<KP>& sm, const int32_t (&half)[2],
                                              Waits& wt) {
     using C = Cfg<KP>;
-    Epilogue<KP> ep(sm, rank);
+    Epilogue<KP> ep(sm, rank, false);
     const int u = ep.u;
     const int64_t n = (int64_t)p.ncl * kG;
     const int Cmax = p.Cmax;
@@ -154,7 +154,7 @@ __device__ __forceinline__ void fwd_epilogue(const RowsPrm& p, int rank, int cid
             Vec<C::EC> x;
 #pragma unroll
             for (int h = 0; h < C::EC; ++h) x.v[h] = on ? (fresh ? pi.v[h] : o.v[h] * sc) * em.v[h] : 0.f;
-            psum = ep.warp_sum(x);
+            psum = C::NC == 2 && left == 0 ? ep.warp_sum_by8(x) : ep.warp_sum(x);
             ep.put(b, x, true, psum);
             if (on) x.store(p.X + (size_t)row * KP + c);
         }
@@ -194,7 +194,7 @@ template <int KP>
 __device__ __forceinline__ void bwd_epilogue(const RowsPrm& p, int rank, int cid, Smem<KP>& sm, const int32_t (&half)[2],
                                              Waits& wt) {
     using C = Cfg<KP>;
-    Epilogue<KP> ep(sm, rank);
+    Epilogue<KP> ep(sm, rank, false);
     const int u = ep.u;
     const int64_t n = (int64_t)p.ncl * kG;
     const int Cmax = p.Cmax;

@@ -192,6 +192,18 @@ __device__ __forceinline__ void slot_totals(int64_t* tot, int64_t S, int64_t n, 
 }
 
 // ---------------------------------------------------------------- contraction warps
+// A product's sum over the rows is eight contiguous parts of NQ chunks of four, each part in the order of
+// the positions p (chunk pos_swap(p)), even and odd rows apart, and the parts are added one after the other:
+// the order of the checkpointed form's pairs of CTAs, so that both forms give the same bits for K = 64, 128
+// and 256.  Row lane ip takes part ip; chunk c of a vector lies at chunk vec_pos(c), where the eight lanes'
+// chunks of a step are next to each other.
+__device__ __forceinline__ int pos_swap(int p) { return p ^ ((p >> 3) & 1); }
+template <int KP>
+__device__ __forceinline__ int vec_pos(int c) {
+    const int p = pos_swap(c);
+    return 8 * (p % Cfg<KP>::NQ) + p / Cfg<KP>::NQ;
+}
+
 template <int KP>
 struct Contraction {
     using C = Cfg<KP>;
@@ -208,7 +220,7 @@ struct Contraction {
         for (int q = 0; q < C::NQ; ++q)
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-                const float* p = Mx + (size_t)(32 * q + 4 * ip + 2 * k) * KP + rank * C::Kh + w * C::WC + cg * C::CW;
+                const float* p = Mx + (size_t)(4 * pos_swap(C::NQ * ip + q) + 2 * k) * KP + rank * C::Kh + w * C::WC + cg * C::CW;
 #pragma unroll
                 for (int h = 0; h < C::CW; ++h) a[2 * q + k][h] = make_float2(p[h], p[KP + h]);
             }
@@ -229,35 +241,26 @@ struct Contraction {
             }
         }
     }
-    // the sums over the 8 row lanes into out (row stride SO): two levels halve the slots, the last the
-    // columns
-    __device__ __forceinline__ void reduce(const float2 (&acc)[4][C::CW], float* out) const {
-        float v[4][C::CW];
+    // the sums over the 8 row lanes, in their order, into out (row stride SO), by way of the warp's `part`
+    static constexpr int PS = 16 * C::CW + 4 * C::CW;              // row lane stride: conflict-free
+    __device__ __forceinline__ void reduce(const float2 (&acc)[4][C::CW], float* part, float* out) const {
 #pragma unroll
-        for (int g = 0; g < 4; ++g)
+        for (int g = 0; g < 4; ++g) {
+            Vec<C::CW> v;
 #pragma unroll
-            for (int h = 0; h < C::CW; ++h) v[g][h] = acc[g][h].x + acc[g][h].y;
-#pragma unroll
-        for (int n = 2, d = 16; n >= 1; n >>= 1, d >>= 1) {
-            const bool up = (lane & d) != 0;
-#pragma unroll
-            for (int g = 0; g < 2; ++g) {
-                if (g < n) {
-#pragma unroll
-                    for (int h = 0; h < C::CW; ++h) {
-                        const float keep = up ? v[g + n][h] : v[g][h], send = up ? v[g][h] : v[g + n][h];
-                        v[g][h] = keep + __shfl_xor_sync(0xffffffffu, send, d);
-                    }
-                }
-            }
+            for (int h = 0; h < C::CW; ++h) v.v[h] = acc[g][h].x + acc[g][h].y;
+            v.store(part + ip * PS + g * C::WC + cg * C::CW);
         }
-        const bool up = (lane & 4) != 0;
-        Vec<C::OC> o;
+        __syncwarp();
+        const int at = (ip >> 1) * C::WC + cg * C::CW + (ip & 1) * C::OC;
+        Vec<C::OC> o, v[8];
 #pragma unroll
-        for (int h = 0; h < C::OC; ++h) {
-            const float keep = up ? v[0][h + C::OC] : v[0][h], send = up ? v[0][h] : v[0][h + C::OC];
-            o.v[h] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-        }
+        for (int l = 0; l < 8; ++l) v[l].load(part + l * PS + at);
+        o = v[0];
+#pragma unroll
+        for (int l = 1; l < 8; ++l)
+#pragma unroll
+            for (int h = 0; h < C::OC; ++h) o.v[h] += v[l].v[h];
         o.store(out + (ip >> 1) * C::SO + w * C::WC + cg * C::CW + (ip & 1) * C::OC);
     }
 };
@@ -266,6 +269,7 @@ struct Contraction {
 template <int KP, typename I>
 __device__ __forceinline__ void contraction_loop(const Contraction<KP>& m, Smem<KP>& sm, const I (&half)[2], Waits& wt) {
     using C = Cfg<KP>;
+    __shared__ __align__(16) float part[kCon / 32][8 * Contraction<KP>::PS];
     const I iters = half[0] > half[1] ? half[0] : half[1];
     for (I it = 1; it < iters; ++it) {
         const int pb = (int)(it & 1) ^ 1;
@@ -283,7 +287,7 @@ __device__ __forceinline__ void contraction_loop(const Contraction<KP>& m, Smem<
             // (products of the own columns before this wait: a second bubble a phase, 3% slower)
             if constexpr (C::NC == 2) wt.cluster(&sm.x_peer[u][pb], ph);
             m.add(x, acc);
-            m.reduce(acc, &sm.out[u][0][0]);
+            m.reduce(acc, part[m.w], &sm.out[u][0][0]);
             __syncwarp();
             if (m.lane == 0) tc::mbar_arrive(&sm.out_full[u]);
         }
@@ -297,12 +301,16 @@ struct Epilogue {
     Smem<KP>& sm;
     int rank, g, u, lane;                          // the warp's slot and its half
     int col;                                       // the lane's first column within the CTA's
+    int xcol;                                      // where it lies in a vector
     uint32_t peer_x, peer_s, peer_bar;             // the peer's buffers (shared::cluster addresses)
-    __device__ __forceinline__ Epilogue(Smem<KP>& s, int r) : sm(s), rank(r) {
+    // (in_order: vectors in the order of the states, not by vec_pos)
+    __device__ __forceinline__ Epilogue(Smem<KP>& s, int r, bool in_order) : sm(s), rank(r) {
         g = (threadIdx.x - kCon) >> 5;
         u = g >> 2;
         lane = threadIdx.x & 31;
         col = C::EC * lane;
+        const int c = r * C::Kh + col;
+        xcol = in_order ? c : 4 * vec_pos<KP>(c >> 2) + (c & 3);
         if constexpr (C::NC == 2) {
             const uint32_t pr = (uint32_t)(r ^ 1);
             peer_x = tc::cluster_addr(&s.x[0][0][0], pr);
@@ -314,11 +322,10 @@ struct Epilogue {
     }
     // The slot's new vector (and a scalar of it) into parity b of both CTAs, and the end of the phase.
     __device__ __forceinline__ void put(int b, const Vec<C::EC>& v, bool scalar, float s) {
-        const int c = rank * C::Kh + col;
-        v.store(&sm.x[b][g][c]);
+        v.store(&sm.x[b][g][xcol]);
         if constexpr (C::NC == 2) {
             const uint32_t bar = peer_bar + 8u * (uint32_t)(2 * u + b);
-            v.send(peer_x + 4u * (uint32_t)((b * kG + g) * C::ST + c), bar);
+            v.send(peer_x + 4u * (uint32_t)((b * kG + g) * C::ST + xcol), bar);
             if (scalar && lane == 0) tc::st_async1(peer_s + 4u * (uint32_t)(b * kG + g), s, bar);
         }
         __syncwarp();
@@ -327,6 +334,23 @@ struct Epilogue {
             if (C::NC == 2 && (g & 3) == 0)              // the peer's bytes of this step
                 tc::mbar_arrive_expect_tx(&sm.x_peer[u][b], (uint32_t)(4 * C::Kh * 4 + (scalar ? 4 * 4 : 0)));
         }
+    }
+    // K > 128, as 16 threads of eight columns each add: eight columns in order, then the threads pairwise
+    __device__ __forceinline__ float warp_sum_by8(const Vec<C::EC>& v) const {
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const float before = __shfl_xor_sync(0xffffffffu, s, 1);
+            if ((lane & 1) == k) {
+                s = k ? before + v.v[0] : v.v[0];
+#pragma unroll
+                for (int h = 1; h < C::EC; ++h) s += v.v[h];
+            }
+        }
+        s = __shfl_sync(0xffffffffu, s, lane | 1);
+#pragma unroll
+        for (int d = 2; d < 32; d <<= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+        return s;
     }
     __device__ __forceinline__ float warp_sum(const Vec<C::EC>& v) const {
         float s = v.v[0];

@@ -138,7 +138,7 @@ __device__ __forceinline__ void log_epilogue(const LogPrm& p, int rank, int cid,
                                              Waits& wt) {
     using C = Cfg<KP>;
     Smem<KP>& sm = ls.s;
-    Epilogue<KP> ep(sm, rank);
+    Epilogue<KP> ep(sm, rank, true);
     const int u = ep.u;
     const int64_t n = (int64_t)p.ncl * kG;
     const int32_t* obs = p.obs + p.off[0];
