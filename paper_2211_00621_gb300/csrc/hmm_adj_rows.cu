@@ -85,11 +85,11 @@ __device__ __forceinline__ int seg_len(int64_t T) {       // ceil(sqrt(T)), as t
 
 // Step i of a slot computes one X_t; the sum of X_{t-1}, and with it e_{t-1}, is complete by then.  A
 // last step only finishes the last ones' books.
-template <int KP>
+template <int KP, bool ORD>
 __device__ __forceinline__ void fwd_epilogue(const RowsPrm& p, int rank, int cid, Smem<KP>& sm, const int32_t (&half)[2],
                                              Waits& wt) {
     using C = Cfg<KP>;
-    Epilogue<KP> ep(sm, rank, false);
+    Epilogue<KP> ep(sm, rank, ORD);
     const int u = ep.u;
     const int64_t n = (int64_t)p.ncl * kG;
     const int Cmax = p.Cmax;
@@ -111,7 +111,7 @@ __device__ __forceinline__ void fwd_epilogue(const RowsPrm& p, int rank, int cid
     // the step computed last: whether there was one, whether it ended its sequence, the CTA's sum of it
     int32_t pseq;
     bool pon, plast;
-    float psum;
+    float psum, e4[4] = {};
     int64_t E;
     auto begin = [&]() {
         next_seq(s, p.S, n, p.order, p.off, fits);
@@ -136,11 +136,13 @@ __device__ __forceinline__ void fwd_epilogue(const RowsPrm& p, int rank, int cid
         const bool on = s.seq >= 0;
         Vec<C::EC> em, o;
         if (on) em.load(p.BT + (size_t)sym * KP + c);
-        float sum = psum;
+        float sum = psum, peer_sum = 0.f;
+        const float last4[4] = {e4[0], e4[1], e4[2], e4[3]};
         if (it > 0) {
             if (C::NC == 2) {                // the peer's sum: in the order of the columns
                 wt.cluster(&sm.x_peer[u][pb], step_phase(it - 1));
                 const float q = sm.peer[pb][ep.g];
+                peer_sum = q;
                 sum = rank == 0 ? sum + q : q + sum;
             }
             if (it < steps) {
@@ -154,16 +156,28 @@ __device__ __forceinline__ void fwd_epilogue(const RowsPrm& p, int rank, int cid
             Vec<C::EC> x;
 #pragma unroll
             for (int h = 0; h < C::EC; ++h) x.v[h] = on ? (fresh ? pi.v[h] : o.v[h] * sc) * em.v[h] : 0.f;
-            psum = C::NC == 2 && left == 0 ? ep.warp_sum_by8(x) : ep.warp_sum(x);
+            // (the last step's sum is the sequence's c: in the checkpointed form's order)
+            if (ORD && left == 0) {
+                ep.sums_by32(x, e4);
+                psum = ((e4[0] + e4[1]) + e4[2]) + e4[3];
+            } else {
+                psum = C::NC == 2 && left == 0 ? ep.warp_sum_by8(x) : ep.warp_sum(x);
+            }
             ep.put(b, x, true, psum);
             if (on) x.store(p.X + (size_t)row * KP + c);
         }
         // the books of the step before
         if (pon) {
             if (plast) {
-                if (lead) {
-                    p.clast[pseq] = sum;
-                    if (p.loglik) p.loglik[pseq] = 0.6931471805599453 * (double)E + log((double)sum);
+                float c_last = sum;
+                if (ORD && C::NC == 2) {         // CTA 1 goes on from CTA 0's
+                    c_last = peer_sum;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) c_last += last4[k];
+                }
+                if (ep.lane == 0 && rank == (ORD ? C::NC - 1 : 0)) {
+                    p.clast[pseq] = c_last;
+                    if (p.loglik) p.loglik[pseq] = 0.6931471805599453 * (double)E + log((double)c_last);
                 }
                 E = 0;
             } else {
@@ -284,9 +298,13 @@ __device__ __forceinline__ void bwd_epilogue(const RowsPrm& p, int rank, int cid
     if (C::NC == 2 && steps > 0) wt.cluster(&sm.x_peer[u][(steps - 1) & 1], step_phase(steps - 1));
 }
 
-template <int KP, bool BWD>
-__device__ __forceinline__ void rows_body(const RowsPrm& p, int rank, int cid, Smem<KP>& sm, cg::cluster_group* cl) {
-    init_bars(sm);
+// ORD: products in the order of the rows (forward, K other than 64, 128 and 256: the order of the
+// checkpointed form there).
+template <int KP, bool BWD, bool ORD>
+__device__ __forceinline__ void rows_body(const RowsPrm& p, int rank, int cid, Smem<KP>& sm, Mid<KP>* mid,
+                                          cg::cluster_group* cl) {
+    if constexpr (ORD) mid->init();
+    init_bars(sm, ORD ? Mid<KP>::W : kCon / 32);
     const int Cmax = p.Cmax;
     int32_t half[2];
     slot_totals(sm.tot, p.S, (int64_t)p.ncl * kG, cid, p.ncl, p.order, p.off,
@@ -295,27 +313,41 @@ __device__ __forceinline__ void rows_body(const RowsPrm& p, int rank, int cid, S
     Waits wt{p.status};
     if (threadIdx.x < kCon) {
         regs_contraction<KP>();
-        Contraction<KP> m;
-        m.load(BWD ? p.At : p.A, rank);
-        contraction_loop(m, sm, half, wt);
+        if constexpr (ORD) {
+            products_in_order<KP>(p.A, rank, sm, *mid, half, wt);
+        } else {
+            Contraction<KP> m;
+            m.load(BWD ? p.At : p.A, rank);
+            contraction_loop(m, sm, half, wt);
+        }
     } else {
         regs_epilogue<KP>();
         if constexpr (BWD) bwd_epilogue<KP>(p, rank, cid, sm, half, wt);
-        else fwd_epilogue<KP>(p, rank, cid, sm, half, wt);
+        else fwd_epilogue<KP, ORD>(p, rank, cid, sm, half, wt);
     }
     if constexpr (Cfg<KP>::NC == 2) cl->sync();  // the peer no longer addresses this CTA's shared memory
 }
 
-template <int KP, bool BWD>
+template <int KP, bool BWD, bool ORD>
 __global__ void __launch_bounds__(kT, Cfg<KP>::MINB) k_rows(RowsPrm p) {
     __shared__ __align__(16) Smem<KP> sm;
-    rows_body<KP, BWD>(p, 0, (int)blockIdx.x, sm, nullptr);
+    if constexpr (ORD) {
+        __shared__ __align__(16) Mid<KP> mid;
+        rows_body<KP, BWD, ORD>(p, 0, (int)blockIdx.x, sm, &mid, nullptr);
+    } else {
+        rows_body<KP, BWD, ORD>(p, 0, (int)blockIdx.x, sm, nullptr, nullptr);
+    }
 }
-template <bool BWD>
+template <bool BWD, bool ORD>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kT, 1) k_rows_pair(RowsPrm p) {
     __shared__ __align__(16) Smem<256> sm;
     cg::cluster_group cl = cg::this_cluster();
-    rows_body<256, BWD>(p, (int)cl.block_rank(), (int)(blockIdx.x >> 1), sm, &cl);
+    if constexpr (ORD) {
+        __shared__ __align__(16) Mid<256> mid;
+        rows_body<256, BWD, ORD>(p, (int)cl.block_rank(), (int)(blockIdx.x >> 1), sm, &mid, &cl);
+    } else {
+        rows_body<256, BWD, ORD>(p, (int)cl.block_rank(), (int)(blockIdx.x >> 1), sm, nullptr, &cl);
+    }
 }
 
 // Block q of kPiParts: pig[q][j] = sum of gamma_0(j) over its share of the sequences, in order.  The
@@ -446,8 +478,11 @@ Layout layout(int K, int M, int64_t S, int64_t total_T) {
 }
 
 using Kern = void (*)(RowsPrm);
-Kern fwd_kernel(int KP) { return KP == 64 ? k_rows<64, false> : KP == 128 ? k_rows<128, false> : k_rows_pair<false>; }
-Kern bwd_kernel(int KP) { return KP == 64 ? k_rows<64, true> : KP == 128 ? k_rows<128, true> : k_rows_pair<true>; }
+Kern fwd_kernel(int K, int KP) {
+    if (K == KP) return KP == 64 ? k_rows<64, false, false> : KP == 128 ? k_rows<128, false, false> : k_rows_pair<false, false>;
+    return KP == 64 ? k_rows<64, false, true> : KP == 128 ? k_rows<128, false, true> : k_rows_pair<false, true>;
+}
+Kern bwd_kernel(int KP) { return KP == 64 ? k_rows<64, true, false> : KP == 128 ? k_rows<128, true, false> : k_rows_pair<true, false>; }
 
 void fill(RowsPrm& p, const Layout& L, const RowsArgs& a) {
     char* ws = (char*)a.ws;
@@ -495,7 +530,7 @@ accel_status rows_forward(const RowsArgs& a, double* d_loglik, cudaStream_t st, 
     accel_status r = order_by_length(a.off, a.S, (int32_t*)(ws + L.order), ws + L.order + align_up((size_t)a.S * 4, 256), st);
     if (r != ACCEL_OK) return r;
     p.order = (int32_t*)(ws + L.order);
-    const Kern kern = fwd_kernel(L.KP);
+    const Kern kern = fwd_kernel(K, L.KP);
     p.ncl = clusters_for(kern, L.KP, a.S, sm_budget());
     kern<<<(unsigned)(p.ncl * (L.KP == 256 ? 2 : 1)), kT, 0, st>>>(p);
     nlaunch += 5;

@@ -294,6 +294,68 @@ __device__ __forceinline__ void contraction_loop(const Contraction<KP>& m, Smem<
     }
 }
 
+// ---------------------------------------------------------------- products in the order of the rows
+// A thread owns a column, and its sum runs over the rows one by one.  Two stages of four warps take half of
+// the rows each (four of two warps a quarter, for 64 columns); while one works on a half of the slots,
+// another works on the other half.
+template <int KP>
+struct Mid {
+    static constexpr int Kh = Cfg<KP>::Kh, NS = kCon / Kh, W = Kh / 32;
+    uint64_t full[2][NS - 1][W];                   // [half][stage][warp of columns]
+    float sum[2][4][Kh];                           // [half][slot][column]: over the rows so far
+    __device__ __forceinline__ void init() {
+        if (threadIdx.x == 0)
+            for (int q = 0; q < 2 * (NS - 1) * W; ++q) tc::mbar_init(&full[0][0][0] + q, 1);
+    }
+};
+template <int KP, typename I>
+__device__ __forceinline__ void products_in_order(const float* __restrict__ A, int rank, Smem<KP>& sm, Mid<KP>& mid,
+                                                  const I (&half)[2], Waits& wt) {
+    using C = Cfg<KP>;
+    constexpr int NS = Mid<KP>::NS, R = KP / NS;
+    const int col = threadIdx.x % C::Kh, stage = threadIdx.x / C::Kh, w = col >> 5, lane = threadIdx.x & 31;
+    float a[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) a[i] = A[(size_t)(stage * R + i) * KP + rank * C::Kh + col];
+    const I iters = half[0] > half[1] ? half[0] : half[1];
+    for (I it = 1; it < iters; ++it) {
+        const int pb = (int)(it & 1) ^ 1;
+        const uint32_t ph = step_phase((uint32_t)(it - 1));
+#pragma unroll 1
+        for (int u = 0; u < 2; ++u) {
+            if (it >= (u ? half[1] : half[0])) continue;
+            const float* x = &sm.x[pb][4 * u][stage * R];
+            wt.local(&sm.x_own[u][pb], ph);
+            if constexpr (C::NC == 2) wt.cluster(&sm.x_peer[u][pb], ph);
+            float acc[4] = {};
+            if (stage > 0) {
+                wt.local(&mid.full[u][stage - 1][w], (uint32_t)(it - 1) & 1u);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) acc[g] = mid.sum[u][g][col];
+            }
+#pragma unroll
+            for (int q = 0; q < R / 4; ++q) {
+                float4 v[4];
+#pragma unroll
+                for (int g = 0; g < 4; ++g) v[g] = *reinterpret_cast<const float4*>(x + g * C::ST + 4 * q);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) acc[g] = fmaf(v[g].x, a[4 * q], acc[g]);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) acc[g] = fmaf(v[g].y, a[4 * q + 1], acc[g]);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) acc[g] = fmaf(v[g].z, a[4 * q + 2], acc[g]);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) acc[g] = fmaf(v[g].w, a[4 * q + 3], acc[g]);
+            }
+            const bool last = stage == NS - 1;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) (last ? sm.out[u][g][col] : mid.sum[u][g][col]) = acc[g];
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(last ? &sm.out_full[u] : &mid.full[u][last ? 0 : stage][w]);
+        }
+    }
+}
+
 // ---------------------------------------------------------------- epilogue warps
 template <int KP>
 struct Epilogue {
@@ -334,6 +396,19 @@ struct Epilogue {
             if (C::NC == 2 && (g & 3) == 0)              // the peer's bytes of this step
                 tc::mbar_arrive_expect_tx(&sm.x_peer[u][b], (uint32_t)(4 * C::Kh * 4 + (scalar ? 4 * 4 : 0)));
         }
+    }
+    // The sums of 32 columns each (e[k]: columns 32 k ..), by a butterfly, the highest bit of the column first
+    __device__ __forceinline__ void sums_by32(const Vec<C::EC>& v, float (&e)[4]) const {
+        Vec<C::EC> t = v;
+#pragma unroll
+        for (int d = 16 / C::EC; d > 0; d >>= 1)
+#pragma unroll
+            for (int h = 0; h < C::EC; ++h) t.v[h] += __shfl_xor_sync(0xffffffffu, t.v[h], d);
+        float s;
+        if constexpr (C::EC == 4) s = (t.v[0] + t.v[2]) + (t.v[1] + t.v[3]);
+        else s = t.v[0] + t.v[1];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) e[k] = k < C::Kh / 32 ? __shfl_sync(0xffffffffu, s, (32 / C::EC * k) & 31) : 0.f;
     }
     // K > 128, as 16 threads of eight columns each add: eight columns in order, then the threads pairwise
     __device__ __forceinline__ float warp_sum_by8(const Vec<C::EC>& v) const {

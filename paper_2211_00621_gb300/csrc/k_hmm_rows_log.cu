@@ -76,61 +76,8 @@ struct LogSmem {
     Smem<KP> s;
     uint64_t max_full[2][kG];                      // [step parity][slot]
     float max_peer[2][kG];
-    uint64_t mid_full[2][4];                       // [half][warp of columns]
-    float mid[2][4][Cfg<KP>::Kh];                  // [half][slot][column]: the sums over the first rows
+    Mid<KP> mid;
 };
-
-// The products in the order of the rows: a thread owns a column, and its sums run over the rows one by
-// one.  Two stages of four warps, the first half of the rows and the second; while one works on a half of
-// the slots, the other works on the other half.
-template <int KP>
-__device__ __forceinline__ void ordered_products(const float* __restrict__ A, int rank, LogSmem<KP>& ls,
-                                                 const uint32_t (&half)[2], Waits& wt) {
-    using C = Cfg<KP>;
-    constexpr int R = KP / 2;
-    Smem<KP>& sm = ls.s;
-    const int col = threadIdx.x & 127, stage = threadIdx.x >> 7, w = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
-    static_assert(C::Kh == 128, "a thread per column and stage");
-    float a[R];
-#pragma unroll
-    for (int i = 0; i < R; ++i) a[i] = A[(size_t)(stage * R + i) * KP + rank * C::Kh + col];
-    const uint32_t iters = half[0] > half[1] ? half[0] : half[1];
-    for (uint32_t it = 1; it < iters; ++it) {
-        const int pb = (int)(it & 1) ^ 1;
-        const uint32_t ph = step_phase(it - 1);
-#pragma unroll 1
-        for (int u = 0; u < 2; ++u) {
-            if (it >= (u ? half[1] : half[0])) continue;
-            const float* x = &sm.x[pb][4 * u][stage * R];
-            wt.local(&sm.x_own[u][pb], ph);
-            if constexpr (C::NC == 2) wt.cluster(&sm.x_peer[u][pb], ph);
-            float acc[4] = {};
-            if (stage == 1) {
-                wt.local(&ls.mid_full[u][w], (it - 1) & 1u);
-#pragma unroll
-                for (int g = 0; g < 4; ++g) acc[g] = ls.mid[u][g][col];
-            }
-#pragma unroll
-            for (int q = 0; q < R / 4; ++q) {
-                float4 v[4];
-#pragma unroll
-                for (int g = 0; g < 4; ++g) v[g] = *reinterpret_cast<const float4*>(x + g * C::ST + 4 * q);
-#pragma unroll
-                for (int g = 0; g < 4; ++g) acc[g] = fmaf(v[g].x, a[4 * q], acc[g]);
-#pragma unroll
-                for (int g = 0; g < 4; ++g) acc[g] = fmaf(v[g].y, a[4 * q + 1], acc[g]);
-#pragma unroll
-                for (int g = 0; g < 4; ++g) acc[g] = fmaf(v[g].z, a[4 * q + 2], acc[g]);
-#pragma unroll
-                for (int g = 0; g < 4; ++g) acc[g] = fmaf(v[g].w, a[4 * q + 3], acc[g]);
-            }
-#pragma unroll
-            for (int g = 0; g < 4; ++g) (stage == 0 ? ls.mid[u][g][col] : sm.out[u][g][col]) = acc[g];
-            __syncwarp();
-            if (lane == 0) tc::mbar_arrive(stage == 0 ? &ls.mid_full[u][w] : &sm.out_full[u]);
-        }
-    }
-}
 
 // Step i of a slot forms r_t; its exponentials, shifted by the largest, are the next vector.
 template <int KP>
@@ -259,18 +206,17 @@ __device__ __forceinline__ void log_epilogue(const LogPrm& p, int rank, int cid,
 
 template <int KP>
 __device__ __forceinline__ void log_body(const LogPrm& p, int rank, int cid, LogSmem<KP>& ls, cg::cluster_group* cl) {
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0)
         for (int q = 0; q < 2 * kG; ++q) tc::mbar_init(&ls.max_full[0][0] + q, 1);
-        for (int q = 0; q < 8; ++q) tc::mbar_init(&ls.mid_full[0][0] + q, 1);
-    }
-    init_bars(ls.s, 4);
+    ls.mid.init();
+    init_bars(ls.s, Mid<KP>::W);
     uint32_t half[2];          // (a slot's steps fit 32 bits: 2^32 of them would take two hours)
     slot_totals(ls.s.tot, p.S, (int64_t)p.ncl * kG, cid, p.ncl, p.order, p.off, [](int64_t) { return true; }, half);
     if constexpr (Cfg<KP>::NC == 2) cl->sync();  // the peer's barriers exist before any remote store
     Waits wt{p.status};
     if (threadIdx.x < kCon) {
         regs_contraction<KP>();
-        ordered_products<KP>(p.A, rank, ls, half, wt);
+        products_in_order<KP>(p.A, rank, ls.s, ls.mid, half, wt);
     } else {
         regs_epilogue<KP>();
         log_epilogue<KP>(p, rank, cid, ls, half, wt);
