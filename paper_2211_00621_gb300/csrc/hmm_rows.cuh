@@ -3,10 +3,10 @@
 //
 // States are padded to KP = 64, 128 or 256 (zero probabilities add exact zeros); a CTA owns Kh = KP /
 // NC of them.  It has 8 contraction warps and 8 epilogue warps.
-//  * Contraction warp w takes WC = Kh / 8 columns, lane 4 ip + cg the rows 32 q + 4 ip .. + 3
-//    (q < KP / 32) and CW = WC / 4 columns: the thread's KP / 8 x CW block of Mx is loaded once per
+//  * Contraction warp w takes WC = Kh / 8 columns, lane 4 ip + cg part ip of the rows (eight
+//    contiguous parts, see Contraction) and CW = WC / 4 columns: the thread's KP / 8 x CW block of Mx is loaded once per
 //    kernel.  The vectors come from shared memory (8 x 16 consecutive bytes a load); the rows' partial
-//    sums meet by a reduce-scatter over the 8 row lanes, not through shared memory.
+//    sums meet in a part of shared memory of the warp's own.
 //  * Epilogue warp g owns sequence slot g: all of a slot's bookkeeping is uniform over a warp, a row of
 //    the CTA's columns is one vector access, and its sum one warp reduction.  (4 warps of two slots
 //    each: a warp that waits for one half is late for the other.)
@@ -17,7 +17,7 @@
 // hide behind the other half's products.  A half whose slots have all finished is left out.  In one
 // group of warps that did both (and a CTA barrier per step) a step took 5,300 cycles at K = 256, of
 // which the FMA pipe was busy 2,350: two warps per scheduler cannot cover the epilogue's latencies.
-// Now a step of both halves takes about 3,600 cycles, of which the FMA pipe needs 2,048.
+// Now a step of both halves takes about 3,700 cycles, of which the FMA pipe needs 2,048.
 //
 // Slots and sequences: slot sl = cluster + clusters * g of n = 8 * clusters runs the sequences
 // k n + sl (k even) and k n + n - 1 - sl (k odd) of the order (by decreasing length), one after the
