@@ -4,9 +4,9 @@
 // States are padded to KP = 64, 128 or 256 (zero probabilities add exact zeros); a CTA owns Kh = KP /
 // NC of them.  It has 8 contraction warps and 8 epilogue warps.
 //  * Contraction warp w takes WC = Kh / 8 columns, lane 4 ip + cg part ip of the rows (eight
-//    contiguous parts, see Contraction) and CW = WC / 4 columns: the thread's KP / 8 x CW block of Mx is loaded once per
-//    kernel.  The vectors come from shared memory (8 x 16 consecutive bytes a load); the rows' partial
-//    sums meet in a part of shared memory of the warp's own.
+//    contiguous parts, see Contraction) and CW = WC / 4 columns: the thread's KP / 8 x CW block of Mx
+//    is loaded once per kernel.  The vectors come from shared memory (8 x 16 consecutive bytes a
+//    load); the rows' partial sums meet in a part of shared memory of the warp's own.
 //  * Epilogue warp g owns sequence slot g: all of a slot's bookkeeping is uniform over a warp, a row of
 //    the CTA's columns is one vector access, and its sum one warp reduction.  (4 warps of two slots
 //    each: a warp that waits for one half is late for the other.)
