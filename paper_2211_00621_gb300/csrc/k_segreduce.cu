@@ -549,8 +549,9 @@ k_segsum_stream(const Tin* __restrict__ data, int64_t N, const int64_t* __restri
                     if (lane >= d) grp += o;
                 }
                 if (t == NW - 1) s_base[b] = G + grp + (SQ ? (uint64_t)(e1 - e0) : 0ull);
-                // segments s .. s + 30, whose boundaries the lanes hold; those before `end` end in this tile
-                auto finish = [&](int64_t s, int64_t end, int64_t bd) {
+                // segments s .. s + 30, whose boundaries the lanes hold; those before `end` end in this tile,
+                // and `open` is the first that does not, if it is known
+                auto finish = [&](int64_t s, int64_t end, int64_t open, int64_t bd) {
                     const int64_t rel = bd - e0;
                     const int p = rel < 0 ? 0 : rel > TE ? TE : (int)rel, k = p > 0 ? p - 1 : 0, tt = k / IT;
                     uint64_t P = s_ex[b][tt];
@@ -568,9 +569,11 @@ k_segsum_stream(const Tin* __restrict__ data, int64_t N, const int64_t* __restri
                     P = bd < e0 ? s_open[b ^ 1] : p > 0 ? G + P : G;
                     const uint64_t left = __shfl_up_sync(0xffffffffu, P, 1);
                     if (lane > 0 && s + lane <= end) out[s + lane - 1] = (Tout)(int64_t)(P - left);
-                    if (s + lane == end) s_open[b] = P;    // (the one left open)
+                    if (s + lane == open) s_open[b] = P;
                 };
-                finish(q + warp * 31, q + n, bd);
+                // (n = kSeg: more segments may end here, and the last one's boundary is found below; only that
+                // one is written, since no barrier would order two writes of different warps)
+                finish(q + warp * 31, q + n, n == kSeg ? -1 : q + n, bd);
                 if (n == kSeg) {
                     // Many segments end here: every warp looks for the first that does not and takes every
                     // eighth group of those before it, four at a time; a long run of empty ones goes by its
@@ -598,7 +601,7 @@ k_segsum_stream(const Tin* __restrict__ data, int64_t N, const int64_t* __restri
 #pragma unroll 1
                         for (int u = 0; u < 4; ++u) {
                             if (s + u * kSeg > end) break;
-                            finish(s + u * kSeg, end, four[0]);
+                            finish(s + u * kSeg, end, end, four[0]);
                             four[0] = four[1];
                             four[1] = four[2];
                             four[2] = four[3];
