@@ -210,10 +210,13 @@ k_hmm_tc(int M, const float* __restrict__ log_A, const float* __restrict__ log_B
     uint16_t* s_mx = reinterpret_cast<uint16_t*>(smem + L.mx);
     float* s_ps = reinterpret_cast<float*>(smem + L.psum);
     uint64_t* bar_mma = reinterpret_cast<uint64_t*>(smem + L.bar);      // [2] per block of states: D ready
+    // The rest are [2], per step parity: a warp may see a step's phase as late as the step after, so the
+    // same barrier's next completion waits for it - of bar_x for the issuing and the max warps, through
+    // D and through bar_mx and the bookkeeping.
     uint64_t* bar_x = bar_mma + 2;                                      // X written, D read
-    uint64_t* bar_info = bar_mma + 4;                                   // [2] per step parity: scale, sym, ... written
-    uint64_t* bar_ps = bar_mma + 6;                                     // [2] per step parity: row sums written
-    uint64_t* bar_mx = bar_mma + 8;                                     // [2] per step parity: column maxima written
+    uint64_t* bar_info = bar_mma + 4;                                   // scale, sym, ... written
+    uint64_t* bar_ps = bar_mma + 6;                                     // row sums written
+    uint64_t* bar_mx = bar_mma + 8;                                     // column maxima written
     uint32_t* slot = reinterpret_cast<uint32_t*>(smem + L.slot);
     volatile uint32_t* s_fail = slot + 1;         // set by a warp whose wait gave up
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
@@ -227,11 +230,11 @@ k_hmm_tc(int M, const float* __restrict__ log_A, const float* __restrict__ log_B
         if (lane == 0) {
             for (int h = 0; h < 2; ++h) {
                 tc::mbar_init(&bar_mma[h], 1);
+                tc::mbar_init(&bar_x[h], NEPI);
                 tc::mbar_init(&bar_info[h], 1);
                 tc::mbar_init(&bar_ps[h], NEPI);
                 tc::mbar_init(&bar_mx[h], NMX > 0 ? NMX : NEPI);
             }
-            tc::mbar_init(bar_x, NEPI);
             tc::fence_mbar_init();
             *s_fail = 0;
         }
@@ -279,7 +282,7 @@ k_hmm_tc(int M, const float* __restrict__ log_A, const float* __restrict__ log_B
         for (uint32_t iter = 0;; ++iter) {
             const uint32_t par = iter & 1u, pprev = par ^ 1u;
             if (!wait_step(&bar_info[par], (iter >> 1) & 1u, s_fail) || s_ctl[iter & 3u].done != 0) break;
-            if (iter > 0) wait_step(bar_x, pprev, s_fail);
+            if (iter > 0) wait_step(&bar_x[pprev], ((iter - 1) >> 1) & 1u, s_fail);
             tc::tc_fence_after();
             const uint64_t xd = xdesc0 + (uint64_t)(pprev * (L.x_bytes >> 4));
             if (tc::elect_one()) {
@@ -463,7 +466,7 @@ k_hmm_tc(int M, const float* __restrict__ log_A, const float* __restrict__ log_B
         for (uint32_t iter = 0;; ++iter) {
             const uint32_t par = iter & 1u;
             if (!wait_step(&bar_info[par], (iter >> 1) & 1u, s_fail) || s_ctl[iter & 3u].done != 0) break;
-            wait_step(bar_x, par, s_fail);
+            wait_step(&bar_x[par], (iter >> 1) & 1u, s_fail);
             const uint4* v = reinterpret_cast<const uint4*>(xr + par * L.x_bytes);
             uint4 x[8];
 #pragma unroll
@@ -555,7 +558,7 @@ k_hmm_tc(int M, const float* __restrict__ log_A, const float* __restrict__ log_B
                         tc::fence_proxy_async_smem();
                         tc::tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) tc::mbar_arrive(bar_x);
+                        if (lane == 0) tc::mbar_arrive(&bar_x[par]);
                     }
                     if constexpr (NMX == 0) {
                         int word;
@@ -569,7 +572,7 @@ k_hmm_tc(int M, const float* __restrict__ log_A, const float* __restrict__ log_B
                         if (CH == 32 || (lane & ~(CH - 1)) == 0) s_ps[(par * (K / 32) + (j >> 5)) * N + s0 + col] = sum;
                     }
                 } else if (ch == CPT / CH - 1) {
-                    if (lane == 0) tc::mbar_arrive(bar_x);
+                    if (lane == 0) tc::mbar_arrive(&bar_x[par]);
                 }
             }
             if (NMX == 0 || ends) {
