@@ -26,6 +26,7 @@
 // deterministic for a given N and P.
 #include "common.cuh"
 
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 #include <cooperative_groups.h>
@@ -206,13 +207,19 @@ accel_status launch_gravity(const float* d_x, const float* d_y, const float* d_z
 //  * Sums over I go to partial[unit], those over J to partial[I block]; k_pairs_sum adds a body's
 //    partial sums in a fixed order: results are deterministic for a given n.
 // What bounds it: the FP32 pipe (packed: 128 cycles for 4 x 2 pairs a lane, beside about 90 issue slots).
-// Against k_gravity, which evaluates both directions: n = 24,576 253 -> 193 us, 65,536 1,660 -> 1,155,
+// Against k_gravity, which evaluates both directions: n = 24,576 253 -> 193 us, 65,536 1,660 -> 1,162,
 // 131,072 6,598 -> 4,466; the error against 64 bits is about half as large (more, shorter sums).  From
 // kPairsMin on, where the units (594) give every SM two rounds of two CTAs; at 16,384 there is less than
 // one.  Up to kPairsMax: the partial sums grow as n^2 (385 MB there).
 constexpr int kPT = 256;
 constexpr int kPI = 1024, kPJ = 512;
 constexpr int64_t kPairsMin = 24576, kPairsMax = 131072;
+// The inverse cube of a distance is formed once for both bodies where it stays a normal float, for
+// (softened) distances up to 2^42: all that bodies within 2^40 of the origin can have.  Past that it is denormal
+// (and 0 from 1e15 on) however large the masses are, so a unit with such bodies is left to k_pairs_far, which
+// multiplies each mass on its own: one operation more (all units so: 1,245 us at 65,536).  In one kernel
+// the two loops take 1,204 us and more; so, 1,162 (1,155 with no far form at all).
+constexpr float kPNear = 1099511627776.f;
 
 struct PairsPrm {
     const float *X, *Y, *Z, *M;
@@ -220,17 +227,20 @@ struct PairsPrm {
     int ni, nj;              // blocks of I, of J
     float eps2;
     float *pi, *pj;          // [3][units][kPI], [3][ni][nj kPJ]
+    int32_t* far;            // [units]
     float *AX, *AY, *AZ;
 };
 
 // Units of the I blocks before i: sum of nj - 2 i'.
 __host__ __device__ __forceinline__ int units_before(int i, int nj) { return i * nj - i * (i - 1); }
 
-__global__ void __launch_bounds__(kPT, 2) k_pairs(PairsPrm p) {
+// FAR: a unit that the other form has marked.
+template <bool FAR>
+__device__ __forceinline__ void pairs_unit(const PairsPrm& p, int u) {
     __shared__ __align__(16) float4 s_xy[kPJ / 2], s_zm[kPJ / 2];   // pairs: (x, x', y, y'), (z, z', m, m')
     __shared__ float2 s_a[3][kPJ / 2];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int u = blockIdx.x, units = units_before(p.ni, p.nj);
+    const int units = units_before(p.ni, p.nj);
     int lo = 0, hi = p.ni - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -247,12 +257,15 @@ __global__ void __launch_bounds__(kPT, 2) k_pairs(PairsPrm p) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) s_a[c][t] = make_float2(0.f, 0.f);
     }
+    auto is_far = [](float x, float y, float z) { return !(fabsf(x) <= kPNear && fabsf(y) <= kPNear && fabsf(z) <= kPNear); };
+    bool far = p.eps2 > kPNear * kPNear || is_far(s_xy[t].x, s_xy[t].z, s_zm[t].x) || is_far(s_xy[t].y, s_xy[t].w, s_zm[t].y);
     float2 nx[4], ny[4], nz[4], nm[4], ax[4], ay[4], az[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int64_t i = (int64_t)I * kPI + w * 128 + k * 32 + lane;
         const bool in = i < p.n;
         const float x = in ? -p.X[i] : 0.f, y = in ? -p.Y[i] : 0.f, z = in ? -p.Z[i] : 0.f, m = in ? -p.M[i] : 0.f;
+        far = far || is_far(x, y, z);
         nx[k] = make_float2(x, x);
         ny[k] = make_float2(y, y);
         nz[k] = make_float2(z, z);
@@ -260,7 +273,13 @@ __global__ void __launch_bounds__(kPT, 2) k_pairs(PairsPrm p) {
         ax[k] = ay[k] = az[k] = make_float2(0.f, 0.f);
     }
     const float2 e2 = make_float2(p.eps2, p.eps2);
-    __syncthreads();
+    if constexpr (FAR) {
+        __syncthreads();
+    } else {
+        far = __syncthreads_or(far) != 0;
+        if (t == 0) p.far[u] = far;
+        if (far) return;
+    }
     for (int turn = 0; turn < 8; ++turn) {
         const int g = ((turn + w) & 7) * 32;      // the group's first pair
         if (both) {
@@ -278,8 +297,16 @@ __global__ void __launch_bounds__(kPT, 2) k_pairs(PairsPrm p) {
                     r = __ffma2_rn(dy, dy, r);
                     r = __ffma2_rn(dx, dx, r);
                     const float2 inv = make_float2(rsqrt_ftz(r.x), rsqrt_ftz(r.y));
-                    const float2 c3 = __fmul2_rn(__fmul2_rn(inv, inv), inv);
-                    const float2 si = __fmul2_rn(c3, mj), sj = __fmul2_rn(c3, nm[k]);
+                    float2 si, sj;
+                    if constexpr (FAR) {
+                        const float2 inv2 = __fmul2_rn(inv, inv);
+                        si = __fmul2_rn(__fmul2_rn(mj, inv), inv2);
+                        sj = __fmul2_rn(__fmul2_rn(nm[k], inv), inv2);
+                    } else {
+                        const float2 c3 = __fmul2_rn(__fmul2_rn(inv, inv), inv);
+                        si = __fmul2_rn(c3, mj);
+                        sj = __fmul2_rn(c3, nm[k]);
+                    }
                     ax[k] = __ffma2_rn(si, dx, ax[k]);
                     ay[k] = __ffma2_rn(si, dy, ay[k]);
                     az[k] = __ffma2_rn(si, dz, az[k]);
@@ -325,6 +352,21 @@ __global__ void __launch_bounds__(kPT, 2) k_pairs(PairsPrm p) {
     }
 }
 
+__global__ void __launch_bounds__(kPT, 2) k_pairs(PairsPrm p) { pairs_unit<false>(p, blockIdx.x); }
+
+// The marked units, on CTAs that are resident at once: there are none but in units far from 1.
+__global__ void __launch_bounds__(kPT, 2) k_pairs_far(PairsPrm p) {
+    const int units = units_before(p.ni, p.nj);
+    for (int base = blockIdx.x; base < units; base += gridDim.x * kPT) {
+        const int64_t mine = base + (int64_t)threadIdx.x * gridDim.x;
+        if (!__syncthreads_or(mine < units && p.far[mine])) continue;
+        for (int k = 0; k < kPT; ++k) {
+            const int64_t u = base + (int64_t)k * gridDim.x;
+            if (u < units && p.far[u]) pairs_unit<true>(p, (int)u);
+        }
+    }
+}
+
 // A body's sums: over the units of its I block, then over the I blocks before it.
 __global__ void __launch_bounds__(256) k_pairs_sum(PairsPrm p) {
     const int64_t b = blockIdx.x * (int64_t)256 + threadIdx.x;
@@ -353,19 +395,22 @@ __global__ void __launch_bounds__(256) k_pairs_sum(PairsPrm p) {
 size_t pairs_ws(int64_t n) {
     if (n < kPairsMin || n > kPairsMax) return 0;
     const int64_t ni = (n + kPI - 1) / kPI, nj = (n + kPJ - 1) / kPJ;
-    return (size_t)(3 * (units_before((int)ni, (int)nj) * (int64_t)kPI + ni * nj * kPJ)) * sizeof(float);
+    const int64_t units = units_before((int)ni, (int)nj);
+    return (size_t)(3 * (units * kPI + ni * nj * kPJ) + units) * sizeof(float);
 }
 
 accel_status launch_pairs(const float* d_x, const float* d_y, const float* d_z, const float* d_m, int64_t n, float eps,
                           float* d_ax, float* d_ay, float* d_az, void* ws, cudaStream_t st) {
     PairsPrm p{d_x, d_y, d_z, d_m, n, (int)((n + kPI - 1) / kPI), (int)((n + kPJ - 1) / kPJ), eps * eps,
-               nullptr, nullptr, d_ax, d_ay, d_az};
+               nullptr, nullptr, nullptr, d_ax, d_ay, d_az};
     const int units = units_before(p.ni, p.nj);
     p.pi = (float*)ws;
     p.pj = p.pi + 3 * (int64_t)units * kPI;
+    p.far = (int32_t*)(p.pj + 3 * (int64_t)p.ni * p.nj * kPJ);
     k_pairs<<<units, kPT, 0, st>>>(p);
+    k_pairs_far<<<std::min(units, 2 * num_sms()), kPT, 0, st>>>(p);
     k_pairs_sum<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p);
-    return after_launch(st, "pairwise_mapreduce", 2);
+    return after_launch(st, "pairwise_mapreduce", 3);
 }
 
 }  // namespace pair
