@@ -351,7 +351,9 @@ typedef struct accel_hmm_model {
  *  precision  ACCEL_HMM_FP32_LOG: log-space recursion in FP32 (max-shifted sum of exp).
  *             ACCEL_HMM_BF16_SCALED: scaled recursion, alpha and A in BF16 on the tensor
  *             cores (tcgen05, FP32 accumulation in TMEM), per-step power-of-two rescaling,
- *             log-scale sum in FP64; one persistent launch for all sequences.
+ *             log-scale sum in FP64; one persistent launch for all sequences.  Its range: log B
+ *             up to 43 (densities), and two symbols running that every state gives a probability
+ *             down to e^-60; a vector that leaves it gives an infinite or NaN logL.
  *  d_obs      device int32 [total_T], symbols in [0, M); d_offsets device int64 [S+1].
  *  d_loglik   device float64 [S].
  *  d_ws       hmm_forward_workspace_size(...) bytes.

@@ -7,10 +7,12 @@
 //   alpha~_t = (A^T X_{t-1}) o b(o_t),   s_t = sum_j alpha~_t(j),   X_t = alpha~_t 2^-k_t
 //   logL     = ln2 * sum_{t<T-1} k_t + ln s_{T-1}
 // Any integers k_t give the same logL exactly; they only keep X in range:
-//   k_t = x_{t-2} - k_{t-1} - kTarget,   x_t = log2 of the largest entry of X_t,
-// which makes x_t = kTarget + the growth of the last two steps.  The step before last is the
+//   k_t = x_{t-2} - k_{t-1} - target,   x_t = log2 of the largest entry of X_t,
+// which makes x_t = target + the growth of the last two steps.  The step before last is the
 // newest whose maxima are not on the path from one step to the next.  Growth is at most 1 for
-// probabilities, so the target sits high: two steps may shrink the vector by 2^-90 each.
+// probabilities, so the target sits high, at 2^60: two steps may shrink the vector by 2^-90 each.
+// Emissions above 1 (densities) grow it: past 2^25 the target is low enough for two steps of the
+// model's largest, up to 2^63 (target_of).
 //
 // A step's time is its latency (the sequences are long and a step depends on the last), so
 // the tile is laid out for a short step, not for a full tensor core:
@@ -58,7 +60,7 @@ namespace hmm {
 
 namespace {
 
-constexpr int kTarget = 60, kMaxScale = 96;     // log2 of X's target size; largest |k|
+constexpr int kMaxScale = 126;                // largest |k|
 constexpr uint64_t kWaitNs = 2000000000ull;   // bounded mbarrier wait: 2 s of wall clock
 // epilogue: column parts per lane quarter for tiles of N sequences
 __host__ __device__ constexpr int col_parts(int N) { return N <= 16 ? 1 : 2; }
@@ -92,6 +94,13 @@ __host__ __device__ inline TileLayout tile_layout(int K, int M, int N, int esize
     L.slot = o;   o += 16;
     L.bytes = o;
     return L;
+}
+
+// log2 of X's target size for emissions of at most b (as bits) < 2^g: 60, or what leaves room for two of
+// them, for sums over the states (2^8) and for the states' probability to meet in one (2^8) below 2^126.
+__device__ __forceinline__ int32_t target_of(uint32_t b) {
+    const int32_t g = (int32_t)(b >> 23) - 126;
+    return g <= 25 ? 60 : 110 - 2 * g;
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
@@ -237,13 +246,16 @@ k_hmm_tc(int M, const float* __restrict__ log_A, const float* __restrict__ log_B
             }
             tc::fence_mbar_init();
             *s_fail = 0;
+            slot[2] = 0;
         }
     }
+    float top = 0.f;                              // the largest emission
     // b(j, o) = exp(log B[j, o]) rounded to BF16, symbol-major; X starts at zero (its columns
     // without a sequence are never read back)
     for (int idx = tid; idx < M * K; idx += kThreads) {
         const int o = idx / K, s = idx - o * K;
         const __nv_bfloat16 b = __float2bfloat16_rn(__expf(log_B[s * M + o]));
+        top = fmaxf(top, __bfloat162float(b));
         if constexpr (sizeof(TE) == 4) sE[idx] = __bfloat162float(b); else sE[idx] = b;
     }
     for (int idx = tid; idx < (int)(2 * L.x_bytes / 16); idx += kThreads)
@@ -252,6 +264,8 @@ k_hmm_tc(int M, const float* __restrict__ log_A, const float* __restrict__ log_B
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
+    top = warp_max_f32(top);
+    if (lane == 0) atomicMax(slot + 2, __float_as_uint(top));
     const uint32_t tmem = *slot;
     const uint32_t tmem_a = tmem + (uint32_t)(NH * N);
     // A^T into tensor memory: lane j of block `half`, column c = (A[2c][j], A[2c+1][j])
@@ -300,6 +314,7 @@ k_hmm_tc(int M, const float* __restrict__ log_A, const float* __restrict__ log_B
         // ---- the bookkeeping warp (lane l: columns l, l + 32, ...)
         const uint64_t t_launch = watchdog_ns != 0 ? tc::globaltimer_ns() : 0;
         const int64_t ncta = gridDim.x;
+        const int32_t target = target_of(slot[2]);
         // the sequence on the column at the step last published, with the steps left after it
         int32_t seq[NU];
         int64_t left[NU];
@@ -398,7 +413,7 @@ k_hmm_tc(int M, const float* __restrict__ log_A, const float* __restrict__ log_B
                 for (int q = 0; q < MXP; ++q) m = max(m, (uint32_t)s_mx[(pprev * MXP + q) * N + c]);
                 // (at a sequence's second step X_{i-1} is not its own: 0 stands for log2 of 1)
                 const int32_t x = st0[u] & 2u ? 0 : (int32_t)(m >> 7) - 127;
-                int32_t k = x - k0[u] - kTarget;
+                int32_t k = x - k0[u] - target;
                 k = k < -kMaxScale ? -kMaxScale : k > kMaxScale ? kMaxScale : k;
                 kn[u] = (st[u] & 3u) == 1u ? k : 0;
                 if (u * 32 + lane < N) s_scale[pprev * N + u * 32 + lane] = __uint_as_float((uint32_t)(127 - kn[u]) << 23);
