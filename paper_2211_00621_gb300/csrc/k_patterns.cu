@@ -176,8 +176,10 @@ k_reduce_partial(const T* __restrict__ in, int64_t n, typename compute_of<T>::ty
     // the elements before the first whole vector, and after the last
     const int64_t head = min(n, (int64_t)((16 - (uintptr_t)in % 16) % 16 / sizeof(T))), nv = (n - head) / V;
     const vec<T, V>* vin = reinterpret_cast<const vec<T, V>*>(in + head);
+    // (red_combine's min and max leave a NaN out as their second operand only, so the first one is never an
+    // element: a NaN would hide its neighbours)
     auto fold = [&](const vec<T, V>& a) {
-        C r = (C)a.v[0];
+        C r = OP == ACCEL_RED_MIN || OP == ACCEL_RED_MAX ? red_combine<OP, C>(red_neutral<C>(OP), (C)a.v[0]) : (C)a.v[0];
 #pragma unroll
         for (int e = 1; e < V; ++e) r = red_combine<OP, C>(r, (C)a.v[e]);
         return r;
