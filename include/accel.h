@@ -382,7 +382,8 @@ accel_status hmm_forward(const accel_hmm_model* m, int32_t precision, const int3
  *  d_weights  device float64 [S] or NULL (all ones).
  *  d_loglik   device float64 [S] or NULL: the forward's logL_s.
  *  max_T      the largest sequence length (sizes the checkpoint storage; hmm_max_length
- *             computes it on the device).  A sequence longer than the checkpoints allow is
+*             computes it on the device).  A sequence longer than the checkpoints allow, or whose
+ *             offsets lie past total_T (every alpha kept: the rows there is room for), is
  *             skipped and reported as ACCEL_ERR_SHAPE: returned by the call in debug mode,
  *             else recorded in the device status word (accel_set_device_status).
  *  Outputs are overwritten (not accumulated); d_grad_log_pi may be NULL.

@@ -152,7 +152,7 @@ accel_status accel_sync_status(int32_t* d_status, int32_t clear, void* stream) {
         case ACCEL_ERR_TIMEOUT:
             return set_error(h, "device-side status: TIMEOUT (a bounded wait gave up or the watchdog budget ran out)");
         case ACCEL_ERR_SHAPE:
-            return set_error(h, "device-side status: SHAPE (a sequence longer than the max_T the call was sized for)");
+            return set_error(h, "device-side status: SHAPE (a sequence longer than the max_T, or past the total_T, that the call was sized for)");
         default: return set_error(h, "device-side status %d", h);
     }
 }

@@ -23,7 +23,7 @@ namespace rows {
 namespace cg = cooperative_groups;
 
 struct RowsPrm {
-    int64_t S;
+    int64_t S, rows;                        // sequences; rows there is room for
     int32_t ncl, K, M, Cmax;
     const float *A, *At, *BT, *pi;          // padded: [KP][KP], its transpose, [M][KP], [KP]
     const int32_t* obs;
@@ -41,7 +41,7 @@ struct RowsPrm {
 __global__ void k_rows_prep(const float* __restrict__ logA, const float* __restrict__ logB,
                             const float* __restrict__ logpi, int K, int KP, int M, float* __restrict__ A,
                             float* __restrict__ At, float* __restrict__ BT, float* __restrict__ pi,
-                            const int64_t* __restrict__ off, int64_t S, int32_t* __restrict__ d_rows) {
+                            const int64_t* __restrict__ off, int64_t S, int64_t room, int32_t* __restrict__ d_rows) {
     const int64_t nA = (int64_t)KP * KP, nB = (int64_t)M * KP;
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < 2 * nA + nB + KP;
          idx += (int64_t)gridDim.x * blockDim.x) {
@@ -59,7 +59,7 @@ __global__ void k_rows_prep(const float* __restrict__ logA, const float* __restr
             pi[j] = j < K ? __expf(logpi[j]) : 0.f;
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) *d_rows = (int32_t)(off[S] - off[0]);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *d_rows = (int32_t)min(off[S] - off[0], room);
 }
 
 // The scale exponent of a sum c = m 2^e, m in [0.5, 1), and 2^-e.
@@ -83,6 +83,11 @@ __device__ __forceinline__ int seg_len(int64_t T) {       // ceil(sqrt(T)), as t
     return c < 1 ? 1 : c;
 }
 
+// A sequence that the call's sizes have room for: of max_T, and within the rows (offsets past total_T).
+__device__ __forceinline__ bool fits(const RowsPrm& p, int64_t o0, int64_t T) {
+    return seg_len(T) <= p.Cmax && o0 >= 0 && o0 + T <= p.rows;
+}
+
 // Step i of a slot computes one X_t; the sum of X_{t-1}, and with it e_{t-1}, is complete by then.  A
 // last step only finishes the last ones' books.
 template <int KP, bool ORD>
@@ -92,12 +97,11 @@ __device__ __forceinline__ void fwd_epilogue(const RowsPrm& p, int rank, int cid
     Epilogue<KP> ep(sm, rank, ORD);
     const int u = ep.u;
     const int64_t n = (int64_t)p.ncl * kG;
-    const int Cmax = p.Cmax;
     const int32_t* obs = p.obs + p.off[0];       // rows and symbols count from the first sequence
     const int c = rank * C::Kh + ep.col;
     const bool lead = rank == 0 && ep.lane == 0;
-    auto fits = [&](int64_t T) {
-        if (seg_len(T) <= Cmax) return true;
+    auto ok = [&](int64_t o0, int64_t T) {
+        if (fits(p, o0, T)) return true;
         report_status(p.status, ACCEL_ERR_SHAPE);
         return false;
     };
@@ -114,7 +118,7 @@ __device__ __forceinline__ void fwd_epilogue(const RowsPrm& p, int rank, int cid
     float psum, e4[4] = {};
     int64_t E;
     auto begin = [&]() {
-        next_seq(s, p.S, n, p.order, p.off, fits);
+        next_seq(s, p.S, n, p.order, p.off, ok);
         fresh = true;
         if (s.seq < 0) return;
         row = (int32_t)s.o0;
@@ -211,10 +215,9 @@ __device__ __forceinline__ void bwd_epilogue(const RowsPrm& p, int rank, int cid
     Epilogue<KP> ep(sm, rank, false);
     const int u = ep.u;
     const int64_t n = (int64_t)p.ncl * kG;
-    const int Cmax = p.Cmax;
     const int32_t* obs = p.obs + p.off[0];
     const int c = rank * C::Kh + ep.col;
-    auto fits = [&](int64_t T) { return seg_len(T) <= Cmax; };
+    auto ok = [&](int64_t o0, int64_t T) { return fits(p, o0, T); };
     // the warp's slot: the step to compute (row, steps left below it), its symbol and the one
     // below, the exponents of the two steps below, the sequence's weight and 1 / c_{T-1}
     Slot s;
@@ -222,7 +225,7 @@ __device__ __forceinline__ void bwd_epilogue(const RowsPrm& p, int rank, int cid
     float wgt, cinv;
     bool fresh;
     auto begin = [&]() {
-        next_seq(s, p.S, n, p.order, p.off, fits);
+        next_seq(s, p.S, n, p.order, p.off, ok);
         fresh = true;
         if (s.seq < 0) return;
         left = (int32_t)s.T - 1;
@@ -305,10 +308,9 @@ __device__ __forceinline__ void rows_body(const RowsPrm& p, int rank, int cid, S
                                           cg::cluster_group* cl) {
     if constexpr (ORD) mid->init();
     init_bars(sm, ORD ? Mid<KP>::W : kCon / 32);
-    const int Cmax = p.Cmax;
     int32_t half[2];
     slot_totals(sm.tot, p.S, (int64_t)p.ncl * kG, cid, p.ncl, p.order, p.off,
-                [&](int64_t T) { return seg_len(T) <= Cmax; }, half);
+                [&](int64_t o0, int64_t T) { return fits(p, o0, T); }, half);
     if constexpr (Cfg<KP>::NC == 2) cl->sync();  // the peer's barriers exist before any remote store
     Waits wt{p.status};
     if (threadIdx.x < kCon) {
@@ -351,7 +353,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kT, 1) k_rows_pair(R
 }
 
 // Block q of kPiParts: pig[q][j] = sum of gamma_0(j) over its share of the sequences, in order.  The
-// rows of a sequence longer than the call allows (reported, not computed) are cleared.
+// rows of a sequence that the call has no room for (reported, not computed) are cleared.
 constexpr int kPiParts = 64;
 __global__ void __launch_bounds__(256) k_rows_pi(RowsPrm p, int KP, float* __restrict__ pig) {
     const int j = threadIdx.x;
@@ -361,11 +363,12 @@ __global__ void __launch_bounds__(256) k_rows_pi(RowsPrm p, int KP, float* __res
     for (int64_t s = s0; s < s1; ++s) {
         const int64_t o0 = p.off[s] - base, T = p.off[s + 1] - base - o0;
         if (T <= 0) continue;
-        if (seg_len(T) > p.Cmax) {
-            for (int64_t i = j; i < T * KP; i += blockDim.x) {
-                p.X[o0 * KP + i] = 0.f;
-                p.Q[o0 * KP + i] = 0.f;
-                p.Gm[o0 * KP + i] = 0.f;
+        if (!fits(p, o0, T)) {
+            const int64_t a = max(o0, (int64_t)0) * KP, z = min(o0 + T, p.rows) * KP;
+            for (int64_t i = a + j; i < z; i += blockDim.x) {
+                p.X[i] = 0.f;
+                p.Q[i] = 0.f;
+                p.Gm[i] = 0.f;
             }
         } else if (j < KP) {
             sum += p.Gm[o0 * KP + j];
@@ -380,10 +383,10 @@ __global__ void __launch_bounds__(256) k_rows_pi(RowsPrm p, int KP, float* __res
 // CTAs as the tables of its window allow (64 KB at M = 64: three an SM).
 constexpr int kCntSplit = 456, kWin = 64;
 __global__ void __launch_bounds__(256) k_rows_counts(const float* __restrict__ Gm, const int32_t* __restrict__ obs,
-                                                     const int64_t* __restrict__ off, int64_t S, int KP, int M,
-                                                     int nsplit, float* __restrict__ cntp) {
+                                                     const int64_t* __restrict__ off, int64_t S, int64_t room, int KP,
+                                                     int M, int nsplit, float* __restrict__ cntp) {
     extern __shared__ float sc[];                 // [window][KP]
-    const int64_t rows = off[S] - off[0];
+    const int64_t rows = min(off[S] - off[0], room);
     obs += off[0];
     const int sp = blockIdx.x % nsplit, m0 = blockIdx.x / nsplit * kWin, nm = min(kWin, M - m0);
     const int64_t r0 = rows * sp / nsplit, r1 = rows * (sp + 1) / nsplit;
@@ -488,6 +491,7 @@ void fill(RowsPrm& p, const Layout& L, const RowsArgs& a) {
     char* ws = (char*)a.ws;
     p = RowsPrm{};
     p.S = a.S;
+    p.rows = a.total_T;
     p.K = a.m->K;
     p.M = a.m->M;
     p.Cmax = a.Cmax;
@@ -524,7 +528,7 @@ accel_status rows_forward(const RowsArgs& a, double* d_loglik, cudaStream_t st, 
     p.loglik = d_loglik;
     k_rows_prep<<<num_sms() * 2, 256, 0, st>>>(a.m->log_A, a.m->log_B, a.m->log_pi, K, L.KP, M, (float*)p.A,
                                                (float*)p.At, (float*)p.BT, (float*)p.pi, a.off, a.S,
-                                               (int32_t*)(ws + L.rows));
+                                               a.total_T, (int32_t*)(ws + L.rows));
     // the order by length (kept for the backward): the slots' loads balance, and the halves of a
     // cluster's slots finish together
     accel_status r = order_by_length(a.off, a.S, (int32_t*)(ws + L.order), ws + L.order + align_up((size_t)a.S * 4, 256), st);
@@ -557,8 +561,8 @@ accel_status rows_backward(const RowsArgs& a, const double* d_weights, float* gA
     if (r != ACCEL_OK) return r;
     const size_t sm = (size_t)std::min(M, kWin) * L.KP * 4;
     ACCEL_CUDA_TRY(cudaFuncSetAttribute(k_rows_counts, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    k_rows_counts<<<(unsigned)(L.nC * ((M + kWin - 1) / kWin)), L.KP, sm, st>>>(p.Gm, p.obs, p.off, a.S, L.KP, M, L.nC,
-                                                                              cnt);
+    k_rows_counts<<<(unsigned)(L.nC * ((M + kWin - 1) / kWin)), L.KP, sm, st>>>(p.Gm, p.obs, p.off, a.S, a.total_T, L.KP, M,
+                                                                              L.nC, cnt);
     k_rows_finish<<<num_sms() * 4, 256, 0, st>>>(p.A, U, cnt, pig, K, L.KP, M, L.nU, L.nC, gA, gB, gpi);
     nlaunch += 5;
     return ACCEL_OK;

@@ -11,7 +11,8 @@ struct RowsArgs {
     const int32_t* obs;
     const int64_t* off;
     int64_t S, total_T;
-    int Cmax;               // ceil(sqrt(max_T)): a sequence whose own is larger is reported, not computed
+    int Cmax;               // ceil(sqrt(max_T)): a sequence whose own is larger, or that lies past total_T, is
+                            // reported, not computed
     void* ws;
     int32_t* status;
 };

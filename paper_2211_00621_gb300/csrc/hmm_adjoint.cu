@@ -2232,7 +2232,7 @@ static accel_status finish_call(const char* who, const Plan& P, int64_t max_T, c
         int32_t h = 0;
         ACCEL_CUDA_TRY(cudaMemcpyAsync(&h, P.p.status, 4, cudaMemcpyDeviceToHost, st));
         ACCEL_CUDA_TRY(cudaStreamSynchronize(st));
-        if (h == ACCEL_ERR_SHAPE) return set_error(h, "%s: a sequence is longer than max_T=%lld", who, (long long)max_T);
+        if (h == ACCEL_ERR_SHAPE) return set_error(h, "%s: a sequence is longer than max_T=%lld, or lies past total_T", who, (long long)max_T);
         if (h != ACCEL_OK) return set_error(h, "%s: device status %d (a bounded wait gave up)", who, h);
     }
     return ok();

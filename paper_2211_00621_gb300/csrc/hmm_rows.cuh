@@ -147,7 +147,7 @@ struct Slot {
     int64_t o0, T;         // its first row (from the first sequence's offset), its length
 };
 
-// Advance the slot to its next sequence that is neither empty nor refused by `ok`.
+// Advance the slot to its next sequence that is neither empty nor refused by `ok` (first row, length).
 template <typename Ok>
 __device__ __forceinline__ void next_seq(Slot& s, int64_t S, int64_t n, const int32_t* order, const int64_t* off, Ok&& ok) {
     for (;;) {
@@ -162,7 +162,7 @@ __device__ __forceinline__ void next_seq(Slot& s, int64_t S, int64_t n, const in
         const int64_t o0 = off[s.seq];
         s.o0 = o0 - off[0];
         s.T = off[s.seq + 1] - o0;
-        if (s.T > 0 && ok(s.T)) return;
+        if (s.T > 0 && ok(s.o0, s.T)) return;
     }
 }
 
@@ -178,7 +178,7 @@ __device__ __forceinline__ void slot_totals(int64_t* tot, int64_t S, int64_t n, 
             if (q >= S) continue;
             const int64_t sq = order ? (int64_t)order[q] : q;
             const int64_t T = off[sq + 1] - off[sq];
-            if (T > 0 && ok(T)) sum += T;
+            if (T > 0 && ok(off[sq] - off[0], T)) sum += T;
         }
         for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
         if (lane == 0) tot[w] = sum;

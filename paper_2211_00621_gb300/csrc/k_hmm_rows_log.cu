@@ -96,7 +96,7 @@ __device__ __forceinline__ void log_epilogue(const LogPrm& p, int rank, int cid,
         peer_max = tc::cluster_addr(&ls.max_peer[0][0], (uint32_t)(rank ^ 1));
         peer_full = tc::cluster_addr(&ls.max_full[0][0], (uint32_t)(rank ^ 1));
     }
-    auto any = [](int64_t) { return true; };
+    auto any = [](int64_t, int64_t) { return true; };
     Vec<C::EC> pi;
     pi.load(p.logpi + c);
     Slot s;
@@ -211,7 +211,7 @@ __device__ __forceinline__ void log_body(const LogPrm& p, int rank, int cid, Log
     ls.mid.init();
     init_bars(ls.s, Mid<KP>::W);
     uint32_t half[2];          // (a slot's steps fit 32 bits: 2^32 of them would take two hours)
-    slot_totals(ls.s.tot, p.S, (int64_t)p.ncl * kG, cid, p.ncl, p.order, p.off, [](int64_t) { return true; }, half);
+    slot_totals(ls.s.tot, p.S, (int64_t)p.ncl * kG, cid, p.ncl, p.order, p.off, [](int64_t, int64_t) { return true; }, half);
     if constexpr (Cfg<KP>::NC == 2) cl->sync();  // the peer's barriers exist before any remote store
     Waits wt{p.status};
     if (threadIdx.x < kCon) {
