@@ -330,19 +330,39 @@ def hmm_forward(log_A, log_B, log_pi, obs, offsets, precision=L.HMM_FP32_LOG, to
     return out
 
 
+# Workspaces up to this size are taken without a look at the memory there is (a query of the driver each).
+_ADJ_ANY = 256 << 20
+
+
+def _has_room(need, device):
+    """Whether `need` bytes are at most an eighth of the memory that the driver has free and that PyTorch
+    holds unused."""
+    if need <= _ADJ_ANY:
+        return True
+    room = torch.cuda.mem_get_info(device)[0]
+    if need > room // 8:
+        room += torch.cuda.memory_reserved(device) - torch.cuda.memory_allocated(device)
+    return need <= room // 8
+
+
 def _adjoint_ws(lib, m, S, total_T, max_T, device):
-    """The adjoint's workspace: with every alpha kept, or the smaller one of the checkpointed form
-    where that much memory is not to be had."""
-    try:
-        return _ws(lib.hmm_adjoint_workspace_size(C.byref(m), S, total_T, max_T), device)
-    except torch.OutOfMemoryError:
-        return _ws(lib.hmm_adjoint_min_workspace_size(C.byref(m), S, total_T, max_T), device)
+    """The adjoint's workspace: with every alpha kept where that leaves the memory to others (an autograd
+    graph holds it until it is gone, and a program may have several), else the 5 to 6 times smaller one of
+    the checkpointed form."""
+    need = lib.hmm_adjoint_workspace_size(C.byref(m), S, total_T, max_T)
+    if _has_room(need, device):
+        try:
+            return _ws(need, device)
+        except torch.OutOfMemoryError:
+            pass
+    return _ws(lib.hmm_adjoint_min_workspace_size(C.byref(m), S, total_T, max_T), device)
 
 
 def hmm_adjoint(log_A, log_B, log_pi, obs, offsets, weights=None, max_T: int | None = None, want_loglik=True,
                 ws=None):
     """Gradients of sum_s w_s logL_s w.r.t. (log_A, log_B, log_pi) (float32) and logL
-    (float64 [S])."""
+    (float64 [S]).  `ws`: a workspace of hmm_adjoint_workspace_size bytes (every alpha kept) or of
+    hmm_adjoint_min_workspace_size (checkpoints); its size chooses the form."""
     lib = L.load()
     _need_cuda(log_A, log_B, log_pi, obs, offsets, weights)
     m = _model(log_A, log_B, log_pi)
@@ -372,9 +392,9 @@ class AdjointSaved:
         self.ws, self.S, self.total_T, self.max_T = ws, S, total_T, max_T
 
 
-def hmm_adjoint_forward(log_A, log_B, log_pi, obs, offsets, max_T: int | None = None, out=None):
-    """logL (float64 [S]) by the adjoint's checkpointed FP32 forward, and the saved state for
-    hmm_adjoint_backward."""
+def hmm_adjoint_forward(log_A, log_B, log_pi, obs, offsets, max_T: int | None = None, out=None, ws=None):
+    """logL (float64 [S]) by the adjoint's FP32 forward, and the saved state for
+    hmm_adjoint_backward.  `ws` as for hmm_adjoint; the saved state holds it."""
     lib = L.load()
     _need_cuda(log_A, log_B, log_pi, obs, offsets)
     m = _model(log_A, log_B, log_pi)
@@ -382,7 +402,8 @@ def hmm_adjoint_forward(log_A, log_B, log_pi, obs, offsets, max_T: int | None = 
     if max_T is None:
         max_T = int(hmm_max_length(offsets).item()) if S else 0
     ll = torch.empty(S, dtype=torch.float64, device=obs.device) if out is None else out
-    ws = _adjoint_ws(lib, m, S, obs.numel(), max_T, obs.device)
+    if ws is None or ws.numel() < lib.hmm_adjoint_min_workspace_size(C.byref(m), S, obs.numel(), max_T):
+        ws = _adjoint_ws(lib, m, S, obs.numel(), max_T, obs.device)
     L.check("hmm_adjoint_forward", lib.hmm_adjoint_forward(C.byref(m), _ptr(obs), _ptr(offsets), S, obs.numel(), max_T,
                                                            _ptr(ll), _ptr(ws), ws.numel(), _stream()))
     return ll, AdjointSaved(ws, S, obs.numel(), max_T)
@@ -523,7 +544,7 @@ class Graph:
 class HMMLogLik(torch.autograd.Function):
     """logL[S] = HMMLogLik.apply(log_A, log_B, log_pi, obs, offsets, precision, max_T=None).
 
-    With FP32 precision and a gradient to take, the forward is the adjoint's checkpointed
+    With FP32 precision and a gradient to take, the forward is the adjoint's own
     forward (hmm_adjoint_forward), whose saved state the backward uses (hmm_adjoint_backward):
     the forward recursion runs once.  With BF16 precision the forward runs on the tensor cores
     and the backward calls hmm_adjoint.  The incoming gradient enters as per-sequence weights
