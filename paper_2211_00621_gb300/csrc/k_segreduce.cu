@@ -437,10 +437,18 @@ k_segsum(const Tin* __restrict__ data, int64_t N, const int64_t* __restrict__ of
 // CTA per tile (k_segsum) and the fix-up: 154 us.  Tried: cp.async into a third buffer instead of
 // registers (132 us), a prefix per vector (132: the shared memory it takes is L1 that the loads and the
 // offsets need), five or six CTAs an SM (152, 203: fewer registers), L2 prefetch ahead (no change).
-// k_segsum stays for N < 16 S, segments of a few elements, where it is as fast (2^23 segments of 0 to 8:
-// 128 us, 136 as a stream).  Where many tiny segments lie side by side in the data, a range that holds
-// them is slow (10 us a tile of one-element segments): half of 2^21 segments of one element, the others
-// of 60, 197 us, 101 by k_segsum; a run of 500,000 empty ones inside one tile, 355 us, 1,950 by k_segsum.
+//  * A tile in which more segments end than the lanes hold boundaries (248): the warps take every eighth group
+//    of the further ones up to the end of the tile, with no search for the last.  If the first 248 took
+//    less than a third of the tile, the prefix of every element is written over both buffers first, and a
+//    boundary is one read instead of up to 16 elements' sum.
+//
+// k_segsum stays for N < 17 S, segments of a few elements, where it is as fast or faster (2^23 segments of 0 to
+// 8: 128 us, 136 as a stream; 2^22 of 16: 109 against 115; of 18: 122 against 102).  Tiny segments side
+// by side in the data fall to the CTA whose range holds them: half of 2^21 segments of one element, the others
+// of 60, 121 us (197 with a search and no prefixes), 101 by k_segsum; of two elements 93 against 101, of
+// eight 103 against 105; half of 2^19 of one element, the others of 240, 119 against 86.  A run of
+// 500,000 empty ones inside one tile: 352 us, 1,950 by k_segsum.  (Ranges half as long, where the most
+// loaded CTA may have an eighth more tiles: 97 us for the first of these, but 5 to 15% more where lengths are even.)
 template <typename Tin, typename Tout, bool SQ>
 __global__ void __launch_bounds__(kThreads, 4)
 k_segsum_stream(const Tin* __restrict__ data, int64_t N, const int64_t* __restrict__ off, int64_t S, int64_t span, int64_t ranges,
@@ -456,6 +464,7 @@ k_segsum_stream(const Tin* __restrict__ data, int64_t N, const int64_t* __restri
     __shared__ uint64_t s_tot[2][NW];                  // the warps' sums
     __shared__ uint64_t s_open[2];                     // prefix at the open segment's start
     __shared__ uint64_t s_base[2];                     // ... at the end of the tile
+    __shared__ int64_t s_last[2];                      // the last boundary that a lane holds
     __shared__ int64_t s_first;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t sc = (int64_t)scalar;
@@ -538,6 +547,7 @@ k_segsum_stream(const Tin* __restrict__ data, int64_t N, const int64_t* __restri
             }
             s_ex[b][t] = inc - own;
             if (lane == 31) s_tot[b][warp] = inc;
+            if (t == kThreads - 1) s_last[b] = bd;
             int n = __syncthreads_count(lane > 0 && bd <= e1);   // segments that end here, of the next kSeg
             // ---- the boundaries
             if (warp * 31 <= n) {
@@ -549,10 +559,9 @@ k_segsum_stream(const Tin* __restrict__ data, int64_t N, const int64_t* __restri
                     if (lane >= d) grp += o;
                 }
                 if (t == NW - 1) s_base[b] = G + grp + (SQ ? (uint64_t)(e1 - e0) : 0ull);
-                // segments s .. s + 30, whose boundaries the lanes hold; those before `end` end in this tile,
-                // and `open` is the first that does not, if it is known
-                auto finish = [&](int64_t s, int64_t end, int64_t open, int64_t bd) {
-                    const int64_t rel = bd - e0;
+                // the prefix at a boundary
+                auto prefix = [&](int64_t at) -> uint64_t {
+                    const int64_t rel = at - e0;
                     const int p = rel < 0 ? 0 : rel > TE ? TE : (int)rel, k = p > 0 ? p - 1 : 0, tt = k / IT;
                     uint64_t P = s_ex[b][tt];
                     const uint64_t before = __shfl_sync(0xffffffffu, grp, (tt >> 5) > 0 ? (tt >> 5) - 1 : 0);
@@ -566,49 +575,98 @@ k_segsum_stream(const Tin* __restrict__ data, int64_t N, const int64_t* __restri
                             if (r * PV + i <= k % IT) P += g(x[i]);
                     }
                     if (SQ) P += (uint64_t)p;
-                    P = bd < e0 ? s_open[b ^ 1] : p > 0 ? G + P : G;
-                    const uint64_t left = __shfl_up_sync(0xffffffffu, P, 1);
-                    if (lane > 0 && s + lane <= end) out[s + lane - 1] = (Tout)(int64_t)(P - left);
-                    if (s + lane == open) s_open[b] = P;
+                    return at < e0 ? s_open[b ^ 1] : p > 0 ? G + P : G;
                 };
-                // (n = kSeg: more segments may end here, and the last one's boundary is found below; only that
-                // one is written, since no barrier would order two writes of different warps)
-                finish(q + warp * 31, q + n, n == kSeg ? -1 : q + n, bd);
+                {
+                    const uint64_t P = prefix(bd), left = __shfl_up_sync(0xffffffffu, P, 1);
+                    const int64_t s = q + warp * 31 + lane;
+                    if (lane > 0 && s <= q + n) out[s - 1] = (Tout)(int64_t)(P - left);
+                    // (n = kSeg: more segments may end here, and the open one's start is found below; only there is
+                    // it written, since no barrier would order two writes of different warps)
+                    if (n < kSeg && s == q + n) s_open[b] = P;
+                }
                 if (n == kSeg) {
-                    // Many segments end here: every warp looks for the first that does not and takes every
-                    // eighth group of those before it, four at a time; a long run of empty ones goes by its
-                    // first and last.
+                    // More segments may end here: the warps take every eighth group up to the end of the tile.
+                    // The next boundary is at `here`; a long run of empty segments goes by its first and last.
                     q += kSeg;
-                    int64_t a = q, z = q + TE < S && off[q + TE + 1] > e1 ? q + TE : S;   // it is in [a, z]
-                    while (a < z) {
-                        const int64_t step = (z - a + 31) / 32, at = a + (lane + 1) * step - 1;
-                        const int c = __popc(__ballot_sync(0xffffffffu, at < z && off[at + 1] <= e1));
-                        a += c * step;
-                        z = a + step - 1 < z ? a + step - 1 : z;
-                    }
-                    const int64_t end = a < z ? a : z;
-                    constexpr int kRun = 32 * kThreads;
-                    for (; q + kRun <= end && off[q] == off[q + kRun]; q += kRun)
-                        for (int i = t; i < kRun; i += kThreads) out[q + i] = Tout(0);
-                    for (int64_t s = q + warp * 31; s <= end; s += 4 * kSeg) {
-                        int64_t four[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) four[u] = off_at(s + u * kSeg + lane);
-                        if (lane % 16 == 0)                // the offsets of the round after the next
-#pragma unroll
-                            for (int u = 8; u < 12; ++u)
-                                if (s + u * kSeg + lane <= S) asm volatile("prefetch.global.L2 [%0];" ::"l"(off + s + u * kSeg + lane));
-#pragma unroll 1
-                        for (int u = 0; u < 4; ++u) {
-                            if (s + u * kSeg > end) break;
-                            finish(s + u * kSeg, end, end, four[0]);
-                            four[0] = four[1];
-                            four[1] = four[2];
-                            four[2] = four[3];
-                        }
-                    }
-                    q = end;
                     n = 0;
+                    const int64_t here = s_last[b];
+                    constexpr int kRun = 32 * kThreads;
+                    auto groups = [&](auto dense, auto per) {
+                        constexpr int U = decltype(per)::value;      // groups a warp has under way
+                        int64_t s = q + warp * 31;
+                        int64_t v[U];
+                        auto fetch = [&]() {
+#pragma unroll
+                            for (int u = 0; u < U; ++u) v[u] = off_at(s + u * kSeg + lane);
+                        };
+                        int64_t end = off_at(q + kRun);
+                        fetch();
+                        if (end == here) {
+                            for (; end == here; q += kRun, end = off_at(q + kRun))
+                                for (int i = t; i < kRun; i += kThreads) out[q + i] = Tout(0);
+                            s = q + warp * 31;
+                            fetch();
+                        }
+                        uint64_t* pre = reinterpret_cast<uint64_t*>(&s_vec[0][0]);
+                        auto place = [](int k) { return k ^ ((k >> 4) & (IT - 1)); };   // (conflict-free by columns, too)
+                        if constexpr (decltype(dense)::value) {
+                            // the prefix of every element, in both buffers: a boundary is one read
+                            const uint64_t before = __shfl_sync(0xffffffffu, grp, warp > 0 ? warp - 1 : 0);
+                            uint64_t run = G + s_ex[b][t] + (warp > 0 ? before : 0ull) + (SQ ? (uint64_t)(t * IT) : 0ull);
+                            __syncthreads();           // the first segments have been looked up
+#pragma unroll
+                            for (int r = 0; r < kVecPerThread; ++r) raw[r] = s_vec[b][swz(t * kVecPerThread + r)];
+                            __syncthreads();
+#pragma unroll
+                            for (int r = 0; r < kVecPerThread; ++r) {
+                                const Tin* x = reinterpret_cast<const Tin*>(&raw[r]);
+#pragma unroll
+                                for (int i = 0; i < PV; ++i) {
+                                    run += g(x[i]) + (SQ ? 1ull : 0ull);
+                                    pre[place(t * IT + r * PV + i)] = run;
+                                }
+                            }
+                            if (e0 + TE < E1) load(e0 + TE);         // (its registers were taken)
+                            __syncthreads();
+                        }
+                        for (;; s += U * kSeg, fetch()) {
+                            if (lane % 16 == 0)        // the offsets of the round after the next
+#pragma unroll
+                                for (int u = 2 * U; u < 3 * U; ++u)
+                                    if (s + u * kSeg + lane <= S) asm volatile("prefetch.global.L2 [%0];" ::"l"(off + s + u * kSeg + lane));
+                            bool more = true;
+#pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                const bool in = v[u] <= e1;
+                                if (!decltype(dense)::value && !__any_sync(0xffffffffu, in)) {
+                                    more = false;
+                                    break;
+                                }
+                                uint64_t P;
+                                if constexpr (decltype(dense)::value) {
+                                    const int p = in ? (int)(v[u] - e0) : 0;
+                                    P = p > 0 ? pre[place(p - 1)] : G;
+                                } else {
+                                    P = prefix(v[u]);
+                                }
+                                const uint64_t left = __shfl_up_sync(0xffffffffu, P, 1);
+                                const bool next = __shfl_down_sync(0xffffffffu, (int)in, 1) != 0;
+                                const int64_t at = s + u * kSeg + lane;
+                                if (lane > 0 && in) out[at - 1] = (Tout)(int64_t)(P - left);
+                                if (lane < 31 && in && !next) {      // the first that does not end here
+                                    s_open[b] = P;
+                                    s_first = at;
+                                }
+                                more = __shfl_sync(0xffffffffu, (int)in, 31) != 0;
+                            }
+                            if (!more) break;
+                        }
+                        __syncthreads();
+                        q = s_first;
+                    };
+                    if (here - e0 < TE / 3) groups(std::true_type{}, std::integral_constant<int, 4>{});
+                    else groups(std::false_type{}, std::integral_constant<int, 2>{});
                 }
             }
             q += n;
@@ -757,8 +815,8 @@ static accel_status run(int32_t op, int32_t map_op, const void* d_data, int64_t 
     }
     int64_t te = tile_elems<Tin>();
     if constexpr (std::is_integral<C>::value) {
-        // (many segments of a few elements: the partition and the tiles' prefix arrays)
-        if (op == ACCEL_RED_ADD && N >= 16 * S) {
+        // (segments of a few elements: the partition and the tiles' prefix arrays)
+        if (op == ACCEL_RED_ADD && N >= 17 * S) {
             auto stream = [&](auto kern) {
                 // Up to six ranges a CTA, one after the other from all over the data, so that a part of many
                 // tiny segments does not fall to a few CTAs; as many as leave the most loaded CTA with the

@@ -28,7 +28,7 @@ def test_open_segment_after_many_that_end(ends, dtype):
     ln = np.asarray(ln, np.int64)
     off = np.concatenate([[0], np.cumsum(ln)])
     n, S = int(off[-1]), len(ln)
-    assert n > 1 << 20 and n >= 16 * S
+    assert n > 1 << 20 and n >= 17 * S
     x = synth.rng(ends).integers(-1000, 1001, size=n)
     ref = np.concatenate([[0], np.cumsum(x * x + 1)])
     t, o = torch.from_numpy(x).to(DEV).to(dtype), torch.from_numpy(off).to(DEV)
