@@ -488,9 +488,9 @@ accel_status hmm_autotune(const accel_hmm_model* m, int32_t precision, const int
                           void* stream);
 /* The configuration hmm_forward(ACCEL_HMM_BF16_SCALED) uses for these sizes: a CTA takes tiles of
  * 2 rows / split sequences (without a tuned configuration, past tiles of 16, the next smaller tile
- * if the lengths favour it); (h_pair, may be NULL) is kept from files of earlier versions, which
- * split a tile over clusters, and changes nothing; (h_units, may be NULL) the persistent CTAs
- * launched (0: all that fit). */
+ * if the lengths favour it); (h_units, may be NULL) the persistent CTAs launched (0: all that fit);
+ * (h_pair, may be NULL) is kept from files of earlier versions, which split a tile over clusters: 1 or
+ * 2 makes the units pairs or fours of CTAs, 0 CTAs. */
 accel_status hmm_tuned_config(int32_t K, int32_t M, int64_t S, int32_t* h_split, int32_t* h_rows,
                               int32_t* h_pair, int32_t* h_units);
 

@@ -482,8 +482,8 @@ def hmm_autotune(log_A, log_B, log_pi, obs, offsets, precision=L.HMM_BF16_SCALED
     """Times the BF16 forward's launch configurations on these inputs and keeps the fastest
     for later hmm_forward calls (and in `cache_path`, JSON lines, if given).  Returns
     (best ms or 0.0 if cached, (split, rows, pair, units)): a CTA takes tiles of 2 rows / split
-    sequences; pair is 0 (other values come from files of earlier versions and change nothing);
-    units = the persistent CTAs launched (0: all that fit)."""
+    sequences; units = the persistent CTAs launched (0: all that fit); pair is 0 (1 and 2 come from
+    files of earlier versions and make the units pairs and fours of CTAs)."""
     lib = L.load()
     m = _model(log_A, log_B, log_pi)
     S = offsets.numel() - 1

@@ -9,7 +9,7 @@
 //   {"kernel": "hmm_forward_bf16", "device": "<name>", "K": 256, "M": 64, "S_log2": 12,
 //    "split": 4, "rows": 32, "pair": 0, "units": 76, "ms": 2.46}
 // (lines without "units" mean all units; a tile is 2 rows / split sequences; "pair" is kept as it
-// was saved and changes nothing).  hmm_forward consults the table; without an entry it chooses
+// was saved: 1 or 2 makes the units pairs or fours of CTAs, the clusters of earlier versions).  hmm_forward consults the table; without an entry it chooses
 // the tile from the sizes and lengths of the call.
 #include "hmm_internal.cuh"
 

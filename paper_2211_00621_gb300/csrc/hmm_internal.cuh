@@ -32,12 +32,12 @@ accel_status plain_forward(const accel_hmm_model* m, const int32_t* obs, const i
 // Launch configuration of the BF16 tensor-core forward, chosen by the autotuner
 // (hmm_autotune.cu): one CTA takes tiles of 2 rows / split sequences (split 2 or 4, rows 32, 64 or
 // 128: tiles of 16 to 128).  `pair` is kept for configurations saved by earlier versions, which
-// split a tile over a cluster of two or four CTAs; it no longer changes the launch.
+// split a tile over a cluster of two (1) or four (2) CTAs: it says what their units were.
 struct TcConfig {
     int split;
     int rows;
     int pair;
-    int units;      // persistent CTAs launched; 0: all that fit
+    int units;      // persistent CTAs launched, or pairs or fours of them (pair); 0: all that fit
 };
 TcConfig tile_config(int n);             // the configuration of a tile of n sequences
 TcConfig default_config(int64_t S);      // ... used without a tuned one

@@ -709,7 +709,8 @@ accel_status tc_forward_cfg(const accel_hmm_model* mdl, const int32_t* obs, cons
     if (!cfg && n > 16) lo = n / 2;                                  // weighed on the device
     const int64_t tiles = (S + lo - 1) / lo;
     int grid = (int)(tiles < num_sms() ? tiles : num_sms());
-    if (c.units > 0 && c.units < grid) grid = c.units;
+    const int64_t ctas = (int64_t)c.units * (c.pair == 1 ? 2 : c.pair == 2 ? 4 : 1);
+    if (ctas > 0 && ctas < grid) grid = (int)ctas;
     // every sequence on a column of its own from the start needs neither an order nor a queue
     int32_t* order = nullptr;
     unsigned long long* next = nullptr;
