@@ -4,7 +4,10 @@
 #include "common.cuh"
 
 #include <atomic>
+#include <map>
+#include <mutex>
 #include <string>
+#include <utility>
 
 namespace accel {
 
@@ -45,6 +48,19 @@ accel_status after_launch(cudaStream_t stream, const char* what, int nkernels) {
         if (e != cudaSuccess) return set_error(ACCEL_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
     }
     return ok();
+}
+
+cudaError_t allow_smem(const void* kern, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, size_t> largest;   // per device and kernel
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lock(mu);
+    size_t& most = largest[std::make_pair(dev, kern)];
+    const size_t want = bytes > most ? bytes : most;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want);
+    if (e == cudaSuccess) most = want;
+    return e;
 }
 
 int num_sms() {

@@ -43,6 +43,11 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 int num_sms();             // SM count of the current device
 int max_smem_optin();      // max dynamic shared memory per block (opt-in)
 
+// Allow a kernel's launches `bytes` of dynamic shared memory.  The limit is one of the function, not of the
+// launch: host threads that launch it with different sizes at once would lower it under each other, so it is
+// only ever raised.
+cudaError_t allow_smem(const void* kern, size_t bytes);
+
 // ----------------------------------------------------------------- dtypes
 inline bool dtype_valid(int32_t d) { return d >= ACCEL_I32 && d <= ACCEL_F64; }
 inline bool dtype_is_int(int32_t d) { return d == ACCEL_I32 || d == ACCEL_I64; }

@@ -560,7 +560,7 @@ accel_status rows_backward(const RowsArgs& a, const double* d_weights, float* gA
     accel_status r = xi_rows(p.X, p.Q, (const int32_t*)(ws + L.rows), L.KP, L.nU, U, p.status, st);
     if (r != ACCEL_OK) return r;
     const size_t sm = (size_t)std::min(M, kWin) * L.KP * 4;
-    ACCEL_CUDA_TRY(cudaFuncSetAttribute(k_rows_counts, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    ACCEL_CUDA_TRY(allow_smem((const void*)k_rows_counts, sm));
     k_rows_counts<<<(unsigned)(L.nC * ((M + kWin - 1) / kWin)), L.KP, sm, st>>>(p.Gm, p.obs, p.off, a.S, a.total_T, L.KP, M,
                                                                               L.nC, cnt);
     k_rows_finish<<<num_sms() * 4, 256, 0, st>>>(p.A, U, cnt, pig, K, L.KP, M, L.nU, L.nC, gA, gB, gpi);

@@ -2024,19 +2024,19 @@ static accel_status run_forward(Plan& P, const accel_hmm_model* m, double* d_log
         ++nlaunch;
         if (P.planned) {
             const size_t sm_plan = clu::plan_smem_bytes();
-            ACCEL_CUDA_TRY(cudaFuncSetAttribute(clu::k_plan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_plan));
+            ACCEL_CUDA_TRY(allow_smem((const void*)clu::k_plan, sm_plan));
             clu::k_plan<<<(unsigned)(L.Cmax + 2), clu::kPlanThreads, sm_plan, st>>>(p, (int64_t*)p.plan,
                                                                                    (int32_t*)p.split, K == 256 ? 8 : 16);
             ++nlaunch;
         }
         const unsigned grid = (unsigned)(2 * p.ncl_fwd);
         const clu::Kernels kc = clu::kernels_for(K);
-        ACCEL_CUDA_TRY(cudaFuncSetAttribute(kc.fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.sm_c));
+        ACCEL_CUDA_TRY(allow_smem((const void*)kc.fwd, P.sm_c));
         kc.fwd<<<grid, clu::kT, P.sm_c, st>>>(p);
         ++nlaunch;
     } else {
         size_t sm_f = smem_fwd(K, M);
-        ACCEL_CUDA_TRY(cudaFuncSetAttribute(k_forward_cp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_f));
+        ACCEL_CUDA_TRY(allow_smem((const void*)k_forward_cp, sm_f));
         k_forward_cp<<<(unsigned)L.ngroups, kT, sm_f, st>>>(p);
         ++nlaunch;
     }
@@ -2107,12 +2107,12 @@ static accel_status run_backward(Plan& P, const double* d_weights, float* d_grad
     if (S > 0) {
         if (P.use_cluster) {
             const clu::Kernels kc = clu::kernels_for(K);
-            ACCEL_CUDA_TRY(cudaFuncSetAttribute(kc.rec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.sm_c));
-            ACCEL_CUDA_TRY(cudaFuncSetAttribute(kc.bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.sm_c));
+            ACCEL_CUDA_TRY(allow_smem((const void*)kc.rec, P.sm_c));
+            ACCEL_CUDA_TRY(allow_smem((const void*)kc.bwd, P.sm_c));
             const size_t sm_cnt = (size_t)M * 256 * 4;
             if (!P.counts_tc) {
                 ACCEL_REQUIRE(sm_cnt <= (size_t)max_smem_optin(), ACCEL_ERR_UNSUPPORTED, "hmm_adjoint: M=%d too large", M);
-                ACCEL_CUDA_TRY(cudaFuncSetAttribute(k_counts, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_cnt));
+                ACCEL_CUDA_TRY(allow_smem((const void*)k_counts, sm_cnt));
             }
             const int nbc = (K + 255) / 256;
             // Three streams of this thread's phase: the backward passes (hi) and the
@@ -2201,7 +2201,7 @@ static accel_status run_backward(Plan& P, const double* d_weights, float* d_grad
             }
             if (rp != ACCEL_OK) return rp;
         } else {
-            ACCEL_CUDA_TRY(cudaFuncSetAttribute(k_backward_round, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.sm_b));
+            ACCEL_CUDA_TRY(allow_smem((const void*)k_backward_round, P.sm_b));
             for (int round = 0; round < L.Cmax; ++round) {
                 k_backward_round<<<(unsigned)L.ngroups, kT, P.sm_b, st>>>(p, round);
                 k_gemm_ptq<<<P.nb * P.nb * kSplit, 256, 0, st>>>(p.P, p.Q, p.rows + round, K, P.Upart);

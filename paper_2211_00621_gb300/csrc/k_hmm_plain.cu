@@ -147,10 +147,10 @@ accel_status plain_forward(const accel_hmm_model* m, const int32_t* obs, const i
         ACCEL_REQUIRE(smem <= (size_t)max_smem_optin(), ACCEL_ERR_UNSUPPORTED, "hmm_forward: M*K too large for the FP32 kernel");
         unsigned grid = (unsigned)((S + 3) / 4);
         if (K <= 32) {
-            ACCEL_CUDA_TRY(cudaFuncSetAttribute(k_plain_warp<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            ACCEL_CUDA_TRY(allow_smem((const void*)k_plain_warp<1>, smem));
             k_plain_warp<1><<<grid, 128, smem, st>>>(m->log_A, m->log_B, m->log_pi, K, M, obs, off, S, loglik);
         } else {
-            ACCEL_CUDA_TRY(cudaFuncSetAttribute(k_plain_warp<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            ACCEL_CUDA_TRY(allow_smem((const void*)k_plain_warp<2>, smem));
             k_plain_warp<2><<<grid, 128, smem, st>>>(m->log_A, m->log_B, m->log_pi, K, M, obs, off, S, loglik);
         }
         return after_launch(st, "hmm_forward(fp32 warp)", 1);

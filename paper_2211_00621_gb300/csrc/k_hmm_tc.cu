@@ -662,7 +662,7 @@ accel_status launch_tiles(const accel_hmm_model* m, const int32_t* obs, const in
     while ((int)cols < need) cols <<= 1;
     const Kernel kern = K == 64 ? kernel_k<64>(n, es) : K == 128 ? kernel_k<128>(n, es)
                       : K == 192 ? kernel_k<192>(n, es) : kernel_k<256>(n, es);
-    ACCEL_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.bytes));
+    ACCEL_CUDA_TRY(allow_smem((const void*)kern, L.bytes));
     kern<<<grid, tile_threads(K, n), L.bytes, st>>>(M, m->log_A, m->log_B, m->log_pi, obs, off, S, order, next, pick,
                                                     loglik, d_status, watchdog_ns(), cols);
     return ACCEL_OK;

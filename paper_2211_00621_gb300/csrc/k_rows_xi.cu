@@ -262,7 +262,7 @@ accel_status xi_rows(const float* X, const float* Q, const int32_t* d_rows, int 
     auto kern = KP == 64 ? k_rows_xi<64> : KP == 128 ? k_rows_xi<128> : k_rows_xi<256>;
     const uint32_t smem = KP == 64 ? smem_bytes(64) : smem_bytes(128);
     const int nt = (KP / tile(KP)) * (KP / tile(KP));
-    ACCEL_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ACCEL_CUDA_TRY(allow_smem((const void*)kern, smem));
     kern<<<(unsigned)(parts * nt), kThreads, smem, st>>>(X, Q, d_rows, parts, U, status);
     return ACCEL_OK;
 }

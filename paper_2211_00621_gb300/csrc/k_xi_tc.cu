@@ -508,7 +508,7 @@ int xi_tc_splits(int K, int M, bool counts) {
     void (*kern)(XiPrm) = xi_kernel(K, counts);
     const size_t smem = xi_smem_bytes(K, Mp, counts, nullptr, nullptr);
     int maxcl = 0;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) {
+    if (allow_smem((const void*)kern, smem) == cudaSuccess) {
         cudaLaunchConfig_t lc = {};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -554,7 +554,7 @@ accel_status xi_tc_round(const float* P, const float* Q, const float* G, const i
                   "hmm_adjoint: count/transition stages do not fit in shared memory (K=%d, M=%d)", K, M);
     p.stages = stages;
     void (*kern)(XiPrm) = xi_kernel(K, counts);
-    ACCEL_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ACCEL_CUDA_TRY(allow_smem((const void*)kern, smem));
     cudaLaunchConfig_t lc = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
