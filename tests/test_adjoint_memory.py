@@ -57,6 +57,15 @@ def test_graphs_held_at_once_leave_the_memory_to_others(memory):
     assert memory["free"] >= 100 * GB
 
 
+def test_an_allocator_without_figures(memory, monkeypatch):
+    def none(d=None):
+        raise RuntimeError("not supported")
+
+    monkeypatch.setattr(torch.cuda, "memory_reserved", none)
+    memory.update(free=20 * GB)
+    assert _ask(3 * GB, 1 * GB) == 1 * GB and _ask(2 * GB, 1 * GB) == 2 * GB
+
+
 def test_a_refused_allocation_falls_back(memory):
     memory.update(free=270 * GB, refuse=2 * GB)
     assert _ask(3 * GB, 1 * GB) == 1 * GB
