@@ -158,7 +158,7 @@ constexpr size_t kStatusBytes = 256;
 // Device status word of a call made on this thread: the word the caller registered with
 // accel_set_device_status, or `fallback` (the call's own word in its workspace) if none.
 int32_t* status_word(int32_t* fallback);
-// Watchdog budget of the persistent single-CTA BF16 forward (accel_set_watchdog_ns; 0 = off).
+// Watchdog budget of the persistent BF16 forward (accel_set_watchdog_ns; 0 = off).
 uint64_t watchdog_ns();
 // SM budget of the adjoint's forward recursion on this host thread (accel_set_sm_budget; 0 = all).
 int32_t sm_budget();

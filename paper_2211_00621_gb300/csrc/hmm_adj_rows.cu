@@ -8,7 +8,7 @@
 // The rows X_t, w v_{t+1} and gamma_t of every step go to memory (12 KP bytes a step, at the row
 // off[s] + t of the flat observations), so nothing is recomputed and one launch runs all steps of
 // all sequences forward, one backward, and one contracts the rows on the tensor cores
-// (k_xi_tc.cu).  The checkpointed form (hmm_adjoint.cu) recomputes X segment by segment in
+// (k_rows_xi.cu).  The checkpointed form (hmm_adjoint.cu) recomputes X segment by segment in
 // sqrt(T) rounds: it needs 5 to 6 times less memory and is kept for calls whose rows would not
 // fit kRowBytesMax or the caller's workspace.  Rows count from the first sequence's offset.
 #include "hmm_adj_rows.cuh"

@@ -155,7 +155,8 @@ accel_status plain_forward(const accel_hmm_model* m, const int32_t* obs, const i
         }
         return after_launch(st, "hmm_forward(fp32 warp)", 1);
     }
-    // the models taken: a K x K stream ring, the emission table and eight vectors within shared memory
+    // The models taken: those whose rows ring, emission table and eight vectors once fitted shared memory.  The
+    // kernel needs none of it (the table is read from global memory); the limit stays as the call's contract.
     const size_t Kp = (size_t)((K + 3) & ~3);
     const size_t bytes = align_up(3 * 32 * Kp * 4 + 24, 16) + ((((size_t)M * K + 3) & ~(size_t)3) + 8 * Kp) * sizeof(float);
     ACCEL_REQUIRE(bytes <= (size_t)max_smem_optin(), ACCEL_ERR_UNSUPPORTED, "hmm_forward: M*K too large for the FP32 kernel");

@@ -38,7 +38,7 @@
 // Row sums: 32 states per warp, added in a fixed binary tree by a reduce-scatter over the
 // lanes, then over the warps in order of states.
 //
-// Measured (GB300; K = 256, M = 64, 4,096 sequences of log-uniform 50 to 5,000 steps): 2.42 ms,
+// Measured (GB300; K = 256, M = 64, 4,096 sequences of log-uniform 50 to 5,000 steps): 2.44 ms,
 // 0.49 us a step of the longest sequence with tiles of 16.  One CTA per 128 sequences with the
 // sequences on the lanes took 12.7 ms, and clusters of two CTAs splitting the states of 32
 // sequences 8.8 ms: 2.5 and 1.75 us a step.  What is left of a step is a chain of latencies (the

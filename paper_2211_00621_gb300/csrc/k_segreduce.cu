@@ -429,6 +429,10 @@ k_segsum(const Tin* __restrict__ data, int64_t N, const int64_t* __restrict__ of
 //    differences are exact.  A lane looks up one boundary, a warp 32 (and so 31 segments); warps without
 //    any go on to the next tile.  Ranges meet by the fix-up kernel, as tiles do.
 //  * One barrier a tile (buffers alternate): it counts the segments that end in the tile.
+//  * A tile in which more segments end than the lanes hold boundaries (248): the warps take every eighth group
+//    of the further ones up to the end of the tile, with no search for the last.  If the first 248 took
+//    less than a third of the tile, the prefix of every element is written over both buffers first, and a
+//    boundary is one read instead of up to 16 elements' sum.
 // The CTA finds its first segment by a 32-way search of the offsets while its first tile is under way;
 // no partition pass over the offsets.
 //
@@ -437,11 +441,6 @@ k_segsum(const Tin* __restrict__ data, int64_t N, const int64_t* __restrict__ of
 // CTA per tile (k_segsum) and the fix-up: 154 us.  Tried: cp.async into a third buffer instead of
 // registers (132 us), a prefix per vector (132: the shared memory it takes is L1 that the loads and the
 // offsets need), five or six CTAs an SM (152, 203: fewer registers), L2 prefetch ahead (no change).
-//  * A tile in which more segments end than the lanes hold boundaries (248): the warps take every eighth group
-//    of the further ones up to the end of the tile, with no search for the last.  If the first 248 took
-//    less than a third of the tile, the prefix of every element is written over both buffers first, and a
-//    boundary is one read instead of up to 16 elements' sum.
-//
 // k_segsum stays for N < 17 S, segments of a few elements, where it is as fast or faster (2^23 segments of 0 to
 // 8: 128 us, 136 as a stream; 2^22 of 16: 109 against 115; of 18: 122 against 102).  Tiny segments side
 // by side in the data fall to the CTA whose range holds them: half of 2^21 segments of one element, the others
